@@ -48,6 +48,13 @@ extern "C" {
  * multiple of 256; 256-byte aligned base).  Contents need not persist. */
 MESHRAST_API size_t knn_workspace_bytes(int64_t N);
 
+/* Bytes with which knn_points (chamfer_fwd: K = 1) may search these batches through
+ * a spatial index (never less than knn_workspace_bytes(N), and that where the
+ * index does not pay for these sizes; 0 for invalid sizes).  A call given
+ * less scans every candidate instead: same results, more time. */
+MESHRAST_API size_t knn_index_workspace_bytes(int64_t N, int64_t P1, int64_t P2, int32_t D,
+                                              int32_t K);
+
 /* K nearest neighbours (Section 3.1, "K Nearest Neighbors").
  * idx (P1, K) int64: the global row in p2 of the k-th nearest candidate of
  * each query row, -1 where the candidate cloud has fewer than k + 1 points;

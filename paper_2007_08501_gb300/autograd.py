@@ -307,7 +307,7 @@ class _KnnPoints(torch.autograd.Function):
     def forward(ctx, p1, p2, first1, len1, first2, len2, K):
         idx = torch.empty((p1.shape[0], K), dtype=torch.int64, device=p1.device)
         dists = torch.empty((p1.shape[0], K), dtype=torch.float32, device=p1.device)
-        ws = ops.alloc_knn_workspace(first1.shape[0], p1.device)
+        ws = ops.alloc_knn_workspace(first1.shape[0], p1.device, p1.shape[0], p2.shape[0], p1.shape[1], K)
         ops.knn_points(p1, first1, len1, p2, first2, len2, K, idx, dists, ws)
         ctx.save_for_backward(p1, p2, idx)
         ctx.mark_non_differentiable(idx)
@@ -340,7 +340,7 @@ class _Chamfer(torch.autograd.Function):
         d_qp = torch.empty(q.shape[0], dtype=torch.float32, device=dev)
         per = torch.empty(N, dtype=torch.float32, device=dev)
         loss = torch.empty((), dtype=torch.float32, device=dev)
-        ws = ops.alloc_knn_workspace(N, dev)
+        ws = ops.alloc_knn_workspace(N, dev, p.shape[0], q.shape[0], p.shape[1])
         ops.chamfer_fwd(p, first1, len1, q, first2, len2, idx_pq, d_pq, idx_qp, d_qp, per, loss, ws)
         ctx.save_for_backward(p, q, first1, len1, first2, len2, idx_pq, idx_qp)
         return loss, per

@@ -20,6 +20,8 @@
 //                the same candidates for its own queries; the lists live in
 //                shared memory and each admitted candidate is inserted by the
 //                whole warp (a ballot ranks it, later entries shift a lane)
+//                Both scans serve small problems and workspaces without room
+//                for the spatial index (knn_index.cu), which serves the rest.
 //   k_pair_sums / k_mean   per-pair Chamfer terms and the batch mean, fixed
 //                reduction order
 //   k_chamfer_bwd / k_knn_bwd   gradients, scatter to the neighbours with
@@ -30,6 +32,7 @@
 #include <cstdint>
 
 #include "knn.h"
+#include "knn_index.h"
 #include "meshrast.h"
 #include "rast_common.cuh"
 
@@ -525,37 +528,52 @@ __device__ __forceinline__ double block_sum(double v, double *s_red) {
     return r;
 }
 
+constexpr int kPairParts = 8;   // blocks per (pair, direction) where the workspace has room for their sums
+
 struct PairArgs {
     const int64_t *first1, *len1, *first2, *len2;
-    const int64_t *idx_pq, *idx_qp;
     const float *d_pq, *d_qp;
+    double *part;   // (2, N, parts): distance sums
     float *per_pair, *loss;
-    int N;
+    int N, parts;
 };
 
-// FP64 accumulation: a few adds per thread, far from any throughput limit
-__global__ void __launch_bounds__(256) k_pair_sums(PairArgs a) {
+// Block (pair, direction, part) sums every parts-th run of 8,192 distances,
+// eight loads in flight per thread.  FP64 accumulation in a fixed order: bound
+// by the FP64 adds of one SM, hence the parts.  A row without a neighbour has
+// distance +infinity, every other one a finite distance.
+__global__ void __launch_bounds__(1024) k_pair_sums(PairArgs a) {
     __shared__ double s_red[32];
-    const int i = blockIdx.x;
-    double out = 0.0;
-    for (int dir = 0; dir < 2; ++dir) {
-        const int64_t f = dir ? a.first2[i] : a.first1[i];
-        const int64_t n = dir ? a.len2[i] : a.len1[i];
-        const int64_t *ix = dir ? a.idx_qp : a.idx_pq;
-        const float *d = dir ? a.d_qp : a.d_pq;
-        double s = 0.0;
-        for (int64_t r = f + threadIdx.x; r < f + n; r += blockDim.x)
-            if (ix[r] >= 0) s += d[r];
-        s = block_sum(s, s_red);
-        if (threadIdx.x == 0 && n > 0) out += s / (double)n;
+    const int i = blockIdx.x, dir = blockIdx.y;
+    const int64_t n = dir ? a.len2[i] : a.len1[i];
+    const float *d = (dir ? a.d_qp : a.d_pq) + (dir ? a.first2[i] : a.first1[i]);
+    double s = 0.0;
+    for (int64_t r = (int64_t)blockIdx.z * 8192 + threadIdx.x; r < n; r += (int64_t)a.parts * 8192) {
+        float v[8];
+#pragma unroll
+        for (int u = 0; u < 8; ++u) v[u] = r + u * 1024 < n ? d[r + u * 1024] : INFINITY;
+#pragma unroll
+        for (int u = 0; u < 8; ++u)
+            if (v[u] < INFINITY) s += v[u];
     }
-    if (threadIdx.x == 0) a.per_pair[i] = (float)out;
+    s = block_sum(s, s_red);
+    if (threadIdx.x == 0) a.part[((size_t)dir * a.N + i) * a.parts + blockIdx.z] = s;
 }
 
 __global__ void __launch_bounds__(1024) k_mean(PairArgs a) {
     __shared__ double s_red[32];
     double s = 0.0;
-    for (int i = threadIdx.x; i < a.N; i += blockDim.x) s += a.per_pair[i];
+    for (int i = threadIdx.x; i < a.N; i += blockDim.x) {
+        double t = 0.0;
+        for (int dir = 0; dir < 2; ++dir) {
+            const int64_t n = dir ? a.len2[i] : a.len1[i];
+            double u = 0.0;
+            for (int k = 0; k < a.parts; ++k) u += a.part[((size_t)dir * a.N + i) * a.parts + k];
+            if (n > 0) t += u / (double)n;
+        }
+        a.per_pair[i] = (float)t;
+        s += (float)t;
+    }
     s = block_sum(s, s_red);
     if (threadIdx.x == 0) a.loss[0] = a.N > 0 ? (float)(s / a.N) : 0.f;
 }
@@ -748,6 +766,11 @@ bool ws_ok(void *ws, size_t bytes, int64_t N) {
     return ws && (reinterpret_cast<uintptr_t>(ws) & 255u) == 0 && bytes >= ws_bytes(N);
 }
 
+// The index is used when the sizes favour it and the workspace has room for it.
+bool use_index(int64_t N, int64_t P1, int64_t P2, int D, int K, size_t bytes) {
+    return nn_index_wins(N, P1, P2, K) && bytes >= ws_bytes(N) + nn_index_bytes(N, P1, P2, D);
+}
+
 // fill one problem; returns its number of blocks (an upper bound of its tiles)
 long long set_problem(KnnProblem &pr, const float *p1, int64_t P1, const int64_t *first1, const int64_t *len1,
                       const float *p2, int64_t P2, const int64_t *first2, const int64_t *len2, int64_t N, int K,
@@ -779,6 +802,11 @@ extern "C" {
 
 MESHRAST_API size_t knn_workspace_bytes(int64_t N) { return N < 0 ? 0 : ws_bytes(N); }
 
+MESHRAST_API size_t knn_index_workspace_bytes(int64_t N, int64_t P1, int64_t P2, int32_t D, int32_t K) {
+    if (N < 0 || P1 < 0 || P2 < 0 || D < 1 || D > 4 || K < 1 || K > 32) return 0;
+    return ws_bytes(N) + (nn_index_wins(N, P1, P2, K) ? nn_index_bytes(N, P1, P2, D) : 0);
+}
+
 MESHRAST_API int knn_points(const float *p1, int64_t P1, const int64_t *first1, const int64_t *len1,
                             const float *p2, int64_t P2, const int64_t *first2, const int64_t *len2, int64_t N,
                             int32_t D, int32_t K, int64_t *idx, float *dists, void *workspace,
@@ -790,6 +818,13 @@ MESHRAST_API int knn_points(const float *p1, int64_t P1, const int64_t *first1, 
     if (!ws_ok(workspace, workspace_bytes, N)) return MESHRAST_ERR_WORKSPACE;
     if (N == 0 || P1 == 0) return MESHRAST_OK;
     cudaStream_t st = reinterpret_cast<cudaStream_t>(stream);
+    if (use_index(N, P1, P2, D, K, workspace_bytes)) {
+        NnSide side[2];
+        if (nn_index_build(side, p1, P1, first1, len1, p2, P2, first2, len2, N, D, false,
+                           reinterpret_cast<char *>(workspace) + ws_bytes(N), st) != cudaSuccess)
+            return MESHRAST_ERR_CUDA;
+        return nn_index_search(side[0], side[1], D, K, idx, dists, st) == cudaSuccess ? MESHRAST_OK : MESHRAST_ERR_CUDA;
+    }
     const int km = km_for_knn(K);
     KnnArgs a{};
     a.nprob = 1;
@@ -834,25 +869,39 @@ MESHRAST_API int chamfer_fwd(const float *p, int64_t P1, const int64_t *first1, 
     if ((P1 > 0 && (!p || !idx_pq || !d_pq)) || (P2 > 0 && (!q || !idx_qp || !d_qp))) return MESHRAST_ERR_INVALID_ARG;
     if (!ws_ok(workspace, workspace_bytes, N)) return MESHRAST_ERR_WORKSPACE;
     cudaStream_t st = reinterpret_cast<cudaStream_t>(stream);
-    PairArgs pa{first1, len1, first2, len2, idx_pq, idx_qp, d_pq, d_qp, loss_per_pair, loss, (int)N};
+    PairArgs pa{first1, len1, first2, len2, d_pq, d_qp, reinterpret_cast<double *>(workspace), loss_per_pair, loss,
+                (int)N, 1};
     if (N == 0) {
         k_mean<<<1, 1024, 0, st>>>(pa);
         return cudaGetLastError() == cudaSuccess ? MESHRAST_OK : MESHRAST_ERR_CUDA;
     }
-    long long *tiles = reinterpret_cast<long long *>(workspace);
-    KnnArgs a{};
-    a.nprob = 2;
-    // both directions in one launch: blocks [0, b0) find neighbours of p in q, [b0, b0 + b1) of q in p
-    const long long b0 = set_problem(a.pr[0], p, P1, first1, len1, q, P2, first2, len2, N, 1, 1, idx_pq, d_pq,
-                                     tiles, 0);
-    if (b0 > INT_MAX) return MESHRAST_ERR_INVALID_ARG;
-    const long long b1 = set_problem(a.pr[1], q, P2, first2, len2, p, P1, first1, len1, N, 1, 1, idx_qp, d_qp,
-                                     tiles + (N + 1), (int)b0);
-    if (b0 + b1 > INT_MAX) return MESHRAST_ERR_INVALID_ARG;
-    k_knn_plan<<<2, 1024, 0, st>>>(a);
-    if (cudaGetLastError() != cudaSuccess) return MESHRAST_ERR_CUDA;
-    if (launch_knn(a, D, 1, (int)(b0 + b1), st) != cudaSuccess) return MESHRAST_ERR_CUDA;
-    k_pair_sums<<<(int)N, 256, 0, st>>>(pa);
+    if (use_index(N, P1, P2, D, 1, workspace_bytes)) {
+        NnSide side[2];
+        if (nn_index_build(side, p, P1, first1, len1, q, P2, first2, len2, N, D, true,
+                           reinterpret_cast<char *>(workspace) + ws_bytes(N), st) != cudaSuccess ||
+            nn_index_search(side[0], side[1], D, 1, idx_pq, d_pq, st) != cudaSuccess ||
+            nn_index_search(side[1], side[0], D, 1, idx_qp, d_qp, st) != cudaSuccess)
+            return MESHRAST_ERR_CUDA;
+        // the index is done with: its first bytes (at least 256 N) hold the sums
+        pa.part = reinterpret_cast<double *>(reinterpret_cast<char *>(workspace) + ws_bytes(N));
+        pa.parts = kPairParts;
+    } else {
+        long long *tiles = reinterpret_cast<long long *>(workspace);
+        KnnArgs a{};
+        a.nprob = 2;
+        // both directions in one launch: blocks [0, b0) find neighbours of p in q, [b0, b0 + b1) of q in p
+        const long long b0 = set_problem(a.pr[0], p, P1, first1, len1, q, P2, first2, len2, N, 1, 1, idx_pq, d_pq,
+                                         tiles, 0);
+        if (b0 > INT_MAX) return MESHRAST_ERR_INVALID_ARG;
+        const long long b1 = set_problem(a.pr[1], q, P2, first2, len2, p, P1, first1, len1, N, 1, 1, idx_qp, d_qp,
+                                         tiles + (N + 1), (int)b0);
+        if (b0 + b1 > INT_MAX) return MESHRAST_ERR_INVALID_ARG;
+        k_knn_plan<<<2, 1024, 0, st>>>(a);
+        if (cudaGetLastError() != cudaSuccess) return MESHRAST_ERR_CUDA;
+        if (launch_knn(a, D, 1, (int)(b0 + b1), st) != cudaSuccess) return MESHRAST_ERR_CUDA;
+    }
+    // (without the index the tile prefixes, no longer needed, make room for 2 N sums)
+    k_pair_sums<<<dim3((unsigned)N, 2, pa.parts), 1024, 0, st>>>(pa);
     k_mean<<<1, 1024, 0, st>>>(pa);
     return cudaGetLastError() == cudaSuccess ? MESHRAST_OK : MESHRAST_ERR_CUDA;
 }

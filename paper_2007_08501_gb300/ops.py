@@ -37,7 +37,7 @@ EXPORTED = ("rast_workspace_bytes", "rast_mesh_fwd", "rast_mesh_bwd", "blend_fwd
             "blend_rast_bwd", "rast_blend_fwd",
             "pts_workspace_bytes", "pts_rasterize_fwd", "pts_rasterize_bwd", "pts_composite_fwd",
             "pts_composite_bwd", "pts_bin_occupancy", "shade_fwd", "shade_bwd",
-            "knn_workspace_bytes", "knn_points", "knn_points_bwd", "chamfer_fwd", "chamfer_bwd")
+            "knn_workspace_bytes", "knn_index_workspace_bytes", "knn_points", "knn_points_bwd", "chamfer_fwd", "chamfer_bwd")
 
 SHADE_FLAT, SHADE_GOURAUD, SHADE_PHONG = 0, 1, 2
 SHADE_SOFTMAX, SHADE_HARD = 0, 1
@@ -156,6 +156,8 @@ def load(build_if_missing: bool = False):
     i32 = ctypes.c_int32
     L.knn_workspace_bytes.argtypes = [i64]
     L.knn_workspace_bytes.restype = sz
+    L.knn_index_workspace_bytes.argtypes = [i64, i64, i64, i32, i32]
+    L.knn_index_workspace_bytes.restype = sz
     L.knn_points.argtypes = [vp, i64, vp, vp, vp, i64, vp, vp, i64, i32, i32, vp, vp, vp, sz, vp]
     L.knn_points.restype = ctypes.c_int
     L.knn_points_bwd.argtypes = [vp, i64, vp, i64, i32, i32, vp, vp, vp, vp, vp]
@@ -598,9 +600,11 @@ def knn_workspace_bytes(N):
     return int(load().knn_workspace_bytes(int(N)))
 
 
-def alloc_knn_workspace(N, device="cuda"):
-    """256-byte aligned device workspace for knn_points / chamfer_fwd over N clouds."""
-    n = max(knn_workspace_bytes(N), 256)
+def alloc_knn_workspace(N, device="cuda", P1=0, P2=0, D=3, K=1):
+    """256-byte aligned device workspace for knn_points / chamfer_fwd over N clouds; with
+    the batches' rows P1 and P2, their dimension and K (Chamfer: 1), one that lets the call
+    search through its spatial index."""
+    n = max(int(load().knn_index_workspace_bytes(int(N), int(P1), int(P2), int(D), int(K))), knn_workspace_bytes(N), 256)
     return torch.empty(n // 8, dtype=torch.int64, device=device)
 
 
