@@ -24,8 +24,8 @@
 //                for the spatial index (knn_index.cu), which serves the rest.
 //   k_pair_sums / k_mean   per-pair Chamfer terms and the batch mean, fixed
 //                reduction order
-//   k_chamfer_bwd / k_knn_bwd   gradients, scatter to the neighbours with
-//                warp aggregation by target row
+//   k_chamfer_bwd / k_knn_bwd   gradients, scattered to the neighbours by
+//                vector reductions
 #include <cuda_runtime.h>
 
 #include <climits>
@@ -592,19 +592,6 @@ __device__ __forceinline__ int cloud_of(long long r, const int64_t *first, const
     return r < first[lo] + len[lo] ? lo : -1;
 }
 
-// atomically add -v to grad[target], lanes with equal targets summed first
-template <int D>
-__device__ __forceinline__ void scatter_neg(long long target, float (&v)[D], float *grad) {
-    const unsigned lane = threadIdx.x & 31u;
-    const long long key = target >= 0 ? target : -1 - (long long)lane;   // invalid lanes stay alone
-    const unsigned peers = __match_any_sync(0xffffffffu, key);
-    group_sum<D>(peers, v);
-    if (target >= 0 && (__ffs(peers) - 1) == (int)lane) {
-#pragma unroll
-        for (int c = 0; c < D; ++c) atomicAdd(grad + target * D + c, -v[c]);
-    }
-}
-
 struct ChamferBwdArgs {
     const float *p, *q;
     const int64_t *first1, *len1, *first2, *len2;
@@ -615,44 +602,30 @@ struct ChamferBwdArgs {
     int N;
 };
 
+// A thread per point of either batch: its own term and its neighbour's, sent
+// straight to the reduction units (see k_knn_bwd).
 template <int D>
 __global__ void __launch_bounds__(256) k_chamfer_bwd(ChamferBwdArgs a) {
     const long long r = (long long)blockIdx.x * blockDim.x + threadIdx.x;
     const bool dir = r >= a.P1;   // false: rows of p (p -> q), true: rows of q (q -> p)
     const long long rr = dir ? r - a.P1 : r;
-    const bool in_range = r < a.P1 + a.P2;
+    if (r >= a.P1 + a.P2) return;
     const float *x = dir ? a.q : a.p, *y = dir ? a.p : a.q;
     float *gx = dir ? a.grad_q : a.grad_p, *gy = dir ? a.grad_p : a.grad_q;
-    long long target = -1;
-    float v[D];
+    const int i = dir ? cloud_of(rr, a.first2, a.len2, a.N) : cloud_of(rr, a.first1, a.len1, a.N);
+    const long long nb = (dir ? a.idx_qp : a.idx_pq)[rr];
+    if (i < 0 || nb < 0) return;
+    float w = a.grad_per_pair ? a.grad_per_pair[i] : 0.f;
+    if (a.grad_loss) w += a.grad_loss[0] / (float)a.N;
+    const float coef = 2.f * w / (float)(dir ? a.len2[i] : a.len1[i]);
+    float v[D], m[D];
 #pragma unroll
-    for (int c = 0; c < D; ++c) v[c] = 0.f;
-    if (in_range) {
-        const int i = dir ? cloud_of(rr, a.first2, a.len2, a.N) : cloud_of(rr, a.first1, a.len1, a.N);
-        const long long nb = (dir ? a.idx_qp : a.idx_pq)[rr];
-        if (i >= 0 && nb >= 0) {
-            float w = a.grad_per_pair ? a.grad_per_pair[i] : 0.f;
-            if (a.grad_loss) w += a.grad_loss[0] / (float)a.N;
-            const float coef = 2.f * w / (float)(dir ? a.len2[i] : a.len1[i]);
-#pragma unroll
-            for (int c = 0; c < D; ++c) {
-                v[c] = coef * (x[rr * D + c] - y[nb * D + c]);
-                atomicAdd(gx + rr * D + c, v[c]);
-            }
-            target = nb;
-        }
+    for (int c = 0; c < D; ++c) {
+        v[c] = coef * (x[rr * D + c] - y[nb * D + c]);
+        m[c] = -v[c];
     }
-    // lanes of one warp may straddle the two directions: scatter each separately
-    const unsigned both = __ballot_sync(0xffffffffu, dir);
-    if (both == 0u || both == 0xffffffffu) {
-        scatter_neg<D>(target, v, gy);
-    } else {
-        float w0[D], w1[D];
-#pragma unroll
-        for (int c = 0; c < D; ++c) { w0[c] = dir ? 0.f : v[c]; w1[c] = dir ? v[c] : 0.f; }
-        scatter_neg<D>(dir ? -1 : target, w0, a.grad_q);
-        scatter_neg<D>(dir ? target : -1, w1, a.grad_p);
-    }
+    red_add_row<D>(gx, rr, v, (reinterpret_cast<uintptr_t>(gx) & 7u) == 0);
+    red_add_row<D>(gy, nb, m, (reinterpret_cast<uintptr_t>(gy) & 7u) == 0);
 }
 
 struct KnnBwdArgs {
@@ -664,37 +637,36 @@ struct KnnBwdArgs {
     int K;
 };
 
+// A thread per query, its K neighbours' terms sent straight to the reduction
+// units.  Bound by the reductions; grouping a warp's equal targets first only
+// pays when neighbouring rows share neighbours, which sampled clouds do not.
 template <int D>
 __global__ void __launch_bounds__(256) k_knn_bwd(KnnBwdArgs a) {
     const long long r = (long long)blockIdx.x * blockDim.x + threadIdx.x;
-    const bool in_range = r < a.P1;
+    if (r >= a.P1) return;
+    const bool pairs = (reinterpret_cast<uintptr_t>(a.grad_p2) & 7u) == 0;
     float x[D], own[D];
 #pragma unroll
     for (int c = 0; c < D; ++c) {
-        x[c] = in_range ? a.p1[r * D + c] : 0.f;
+        x[c] = a.p1[r * D + c];
         own[c] = 0.f;
     }
+#pragma unroll 4
     for (int k = 0; k < a.K; ++k) {
-        long long nb = in_range ? a.idx[r * a.K + k] : -1;
-        if (nb >= a.P2) nb = -1;
+        const long long nb = a.idx[r * a.K + k];
+        if (nb < 0 || nb >= a.P2) continue;
+        const float g2 = 2.f * a.grad_dists[r * a.K + k];
         float v[D];
-        if (nb >= 0) {
-            const float g2 = 2.f * a.grad_dists[r * a.K + k];
 #pragma unroll
-            for (int c = 0; c < D; ++c) {
-                v[c] = g2 * (x[c] - a.p2[nb * D + c]);
-                own[c] += v[c];
-            }
-        } else {
-#pragma unroll
-            for (int c = 0; c < D; ++c) v[c] = 0.f;
+        for (int c = 0; c < D; ++c) {
+            const float t = g2 * (x[c] - a.p2[nb * D + c]);
+            own[c] += t;
+            v[c] = -t;
         }
-        scatter_neg<D>(nb, v, a.grad_p2);
+        red_add_row<D>(a.grad_p2, nb, v, pairs);
     }
-    if (in_range) {
 #pragma unroll
-        for (int c = 0; c < D; ++c) a.grad_p1[r * D + c] = own[c];
-    }
+    for (int c = 0; c < D; ++c) a.grad_p1[r * D + c] = own[c];
 }
 
 // ---------------------------------------------------------------------------

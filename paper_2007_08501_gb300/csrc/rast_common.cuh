@@ -472,6 +472,35 @@ __device__ __forceinline__ void group_sum(unsigned peers, float (&x)[NV]) {
     }
 }
 
+// Adds v to row `row` of a packed (rows, D) float array with as few reductions
+// as its 4 D-byte rows allow: pairs of floats on 8-byte boundaries go as one
+// vector reduction (a row of three: one pair and one float).  `pairs`: the
+// array starts on an 8-byte boundary; without it every float goes alone.
+__device__ __forceinline__ void red_add2(float *p, float x, float y) {
+    asm volatile("red.relaxed.gpu.global.add.v2.f32 [%0], {%1, %2};" ::"l"(p), "f"(x), "f"(y) : "memory");
+}
+template <int D>
+__device__ __forceinline__ void red_add_row(float *g, int64_t row, const float (&v)[D], bool pairs) {
+    float *p = g + row * D;
+    if constexpr (D == 2 || D == 4) {
+        if (pairs) {
+#pragma unroll
+            for (int c = 0; c < D; c += 2) red_add2(p + c, v[c], v[c + 1]);
+            return;
+        }
+    }
+    if constexpr (D == 3) {
+        if (pairs) {
+            const bool odd = row & 1;   // an odd row starts 4 bytes past a boundary
+            atomicAdd(odd ? p : p + 2, odd ? v[0] : v[2]);
+            red_add2(odd ? p + 1 : p, odd ? v[1] : v[0], odd ? v[2] : v[1]);
+            return;
+        }
+    }
+#pragma unroll
+    for (int c = 0; c < D; ++c) atomicAdd(p + c, v[c]);
+}
+
 __device__ __forceinline__ void set_status(unsigned *status, unsigned bits) {
     if (bits) atomicOr(status, bits);
 }
