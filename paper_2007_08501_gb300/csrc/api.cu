@@ -276,7 +276,7 @@ static int forward(const rast_params *p, const float *verts, int64_t V, const in
         if (fa2.image && blended) *blended = true;
         return mr::launch_frag_attr(fa2, st) == cudaSuccess ? MESHRAST_OK : MESHRAST_ERR_CUDA;
     }
-    ka.sort_cap = mr::fine_sort_cap(p->max_faces_per_bin, (int)K, p->bin_size * p->bin_size);
+    ka.sort_cap = 0;
     if (fine_blend) {
         ka.blend = *blend;
         ka.blend.frag = no_frag ? 0 : 1;

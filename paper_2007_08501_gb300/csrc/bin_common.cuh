@@ -228,6 +228,256 @@ __device__ __forceinline__ void sort_entries(unsigned long long *s_sort, const u
     }
 }
 
+// ---------------------------------------------------------------------------
+// A bin's list in front-to-back windows, for the fine passes.
+//
+// What a fine pass keeps (the K nearest by depth and id) does not depend on the
+// order it meets the candidates in; order only buys the early stop once every
+// pixel's K-th depth lies in front of what is left.  So the list is not sorted
+// but dealt into 256 depth buckets (linear in the key between the bin's
+// smallest and largest) and handed out in windows of consecutive buckets that
+// fit WIN entries of shared memory: one pass for the range, one for the
+// counts, one per window to fetch its entries, about six barriers for a bin of
+// up to WIN entries where a bitonic sort of 1,024 takes 55 exchange stages.
+// A bucket that does not fit is dealt into 256 buckets of its own; what does
+// not fit then (entries at nearly one depth) is handed out in pieces of the
+// list, in whatever order it has.
+//
+// The bucket of a key is monotone in the key (a rounded subtraction, a rounded
+// product, a truncation), so if bucket(x) < bucket(key), then x < key: comparing
+// the bucket of a pixel's K-th depth with a window's buckets decides, without
+// knowing any window's smallest key, that everything from there on is behind.
+// ---------------------------------------------------------------------------
+constexpr int kBuckets = 256;
+
+struct KeyMap {
+    float lo, scale;
+    // NaN (0 x inf) converts to 0, values past the int range saturate
+    __device__ __forceinline__ int operator()(float key) const {
+        return min(kBuckets - 1, __float2int_rz(__fmul_rn(__fsub_rn(key, lo), scale)));
+    }
+};
+
+__device__ __forceinline__ float entry_key(unsigned long long e) { return __uint_as_float((unsigned)(e >> 32)); }
+
+// Where a block is in its bin's list; the same in every thread.
+struct WindowState {
+    const unsigned long long *list;
+    int cnt;
+    KeyMap map[2];
+    int b0, b1;      // next bucket of level 0; of level 1 while `deep`
+    int seg;         // >= 0: next piece of the list (unordered, or a level-1 bucket that does not fit)
+    int deep, plain;
+    int sorted;      // level whose buckets order the current window, -1: none
+};
+
+template <int WIN>
+struct WindowShared {
+    unsigned long long ent[WIN];      // the current window
+    int pre[2][kBuckets + 1];         // entries before each bucket, per level
+    int cur[kBuckets];
+    int wsum[8];
+    unsigned lo, hi;
+    int n;
+    WindowState st;
+
+    // bucket that orders the current window (constant when nothing does)
+    __device__ __forceinline__ int rank(float key) const { return st.sorted < 0 ? 0 : st.map[st.sorted](key); }
+
+    // whether every entry not yet handed out lies behind depth z
+    __device__ __forceinline__ bool rest_behind(float z) const {
+        if (st.plain) return false;
+        const int k = st.map[0](z);
+        return k < st.b0 || (st.deep && k == st.b0 && st.map[1](z) < st.b1);
+    }
+};
+
+template <int BD, int WIN>
+struct WindowLoader : WindowState {
+    WindowShared<WIN> &s;
+    __device__ __forceinline__ WindowLoader(WindowShared<WIN> &sh) : WindowState(sh.st), s(sh) {}
+
+    __device__ __forceinline__ bool mine(float key, int level) const { return level == 0 || map[0](key) == b0; }
+
+    // ranges and counts of the buckets of a level
+    template <int level>
+    __device__ __forceinline__ void deal() {
+        const int tid = threadIdx.x;
+        __syncthreads();
+        if (tid == 0) { s.lo = 0xffffffffu; s.hi = 0u; }
+        for (int b = tid; b < kBuckets; b += BD) s.cur[b] = 0;
+        __syncthreads();
+        unsigned lo = 0xffffffffu, hi = 0u;  // keys are positive: bits order like values
+        for (int i = tid; i < cnt; i += BD) {
+            const unsigned long long e = __ldg(list + i);
+            if (!mine(entry_key(e), level)) continue;
+            lo = min(lo, (unsigned)(e >> 32));
+            hi = max(hi, (unsigned)(e >> 32));
+        }
+        lo = __reduce_min_sync(0xffffffffu, lo);
+        hi = __reduce_max_sync(0xffffffffu, hi);
+        if ((tid & 31) == 0) { atomicMin(&s.lo, lo); atomicMax(&s.hi, hi); }
+        __syncthreads();
+        KeyMap m;
+        m.lo = __uint_as_float(s.lo);
+        const float d = __uint_as_float(s.hi) - m.lo;
+        m.scale = d > 0.f ? __fdiv_rn((float)kBuckets, d) : 0.f;
+        map[level] = m;
+        for (int i = tid; i < cnt; i += BD) {
+            const float key = entry_key(__ldg(list + i));
+            if (mine(key, level)) atomicAdd(&s.cur[m(key)], 1);
+        }
+        __syncthreads();
+        // exclusive prefix of the counts: kBuckets / BD consecutive buckets per thread
+        constexpr int E = kBuckets / BD;
+        int v[E], sum = 0;
+#pragma unroll
+        for (int e = 0; e < E; ++e) { v[e] = s.cur[tid * E + e]; sum += v[e]; }
+        int x = sum;
+#pragma unroll
+        for (int o = 1; o < 32; o <<= 1) {
+            const int y = __shfl_up_sync(0xffffffffu, x, o);
+            if ((tid & 31) >= o) x += y;
+        }
+        if ((tid & 31) == 31) s.wsum[tid >> 5] = x;
+        __syncthreads();
+        int base = x - sum;
+        for (int w = 0; w < (tid >> 5); ++w) base += s.wsum[w];
+#pragma unroll
+        for (int e = 0; e < E; ++e) {
+            s.pre[level][tid * E + e] = base;
+            base += v[e];
+        }
+        if (tid == BD - 1) s.pre[level][kBuckets] = base;
+        for (int b = tid; b < kBuckets; b += BD) s.cur[b] = 0;
+        __syncthreads();
+    }
+
+    // one past the last bucket of the longest run from b that fits WIN entries
+    __device__ __forceinline__ int run_end(int level, int b) const {
+        const int *p = s.pre[level];
+        const int lim = p[b] + WIN;
+        int lo = b, hi = kBuckets;  // p[lo] <= lim
+        while (lo < hi) {
+            const int mid = (lo + hi + 1) >> 1;
+            if (p[mid] <= lim) lo = mid;
+            else hi = mid - 1;
+        }
+        return lo;
+    }
+
+    // entries of buckets [b, e) of a level, in bucket order
+    template <int level>
+    __device__ __forceinline__ int fetch(int b, int e) {
+        const int n = s.pre[level][e] - s.pre[level][b];
+        if (n > 0) {
+            const KeyMap m = map[level];
+            for (int i = threadIdx.x; i < cnt; i += BD) {
+                const unsigned long long v = __ldg(list + i);
+                const float key = entry_key(v);
+                if (!mine(key, level)) continue;
+                const int k = m(key);
+                if (k < b || k >= e) continue;
+                s.ent[s.pre[level][k] - s.pre[level][b] + atomicAdd(&s.cur[k], 1)] = v;
+            }
+            __syncthreads();
+        }
+        sorted = level;
+        return n;
+    }
+
+    // the next window's size; 0 at the end
+    __device__ __forceinline__ int next() {
+        while (cnt > 0) {
+            if (plain) {
+                const int m = min(WIN, cnt - seg);
+                if (m <= 0) return 0;
+                for (int i = threadIdx.x; i < m; i += BD) s.ent[i] = __ldg(list + seg + i);
+                seg += m;
+                __syncthreads();
+                return m;
+            }
+            if (seg >= 0) {
+                if (seg >= cnt) { seg = -1; ++b1; continue; }
+                if (threadIdx.x == 0) s.n = 0;
+                __syncthreads();
+                const int m = min(WIN, cnt - seg);
+                for (int i = threadIdx.x; i < m; i += BD) {
+                    const unsigned long long v = __ldg(list + seg + i);
+                    const float key = entry_key(v);
+                    if (map[0](key) == b0 && map[1](key) == b1) s.ent[atomicAdd(&s.n, 1)] = v;
+                }
+                seg += m;
+                sorted = -1;
+                __syncthreads();
+                const int n = s.n;
+                __syncthreads();  // s.n is reset by the next piece
+                if (n == 0) continue;
+                return n;
+            }
+            if (deep) {
+                if (b1 >= kBuckets) {
+                    deep = false;
+                    ++b0;
+                    for (int b = threadIdx.x; b < kBuckets; b += BD) s.cur[b] = 0;
+                    __syncthreads();
+                    continue;
+                }
+                const int e = run_end(1, b1);
+                if (e == b1) { seg = 0; continue; }
+                const int n = fetch<1>(b1, e);
+                b1 = e;
+                if (n > 0) return n;
+                continue;
+            }
+            if (b0 >= kBuckets) return 0;
+            const int e = run_end(0, b0);
+            if (e == b0) { deal<1>(); deep = true; b1 = 0; continue; }
+            const int n = fetch<0>(b0, e);
+            b0 = e;
+            if (n > 0) return n;
+        }
+        return 0;
+    }
+};
+
+// Starts on a list; `ordered` false hands it out as it is.  Every thread of the
+// block calls this and window_next.
+template <int BD, int WIN>
+__device__ __forceinline__ void window_begin(WindowShared<WIN> &s, const unsigned long long *list, int cnt,
+                                             bool ordered) {
+    __syncthreads();
+    if (threadIdx.x == 0) {
+        s.st.list = list;
+        s.st.cnt = cnt;
+        s.st.b0 = ordered ? -1 : 0;
+        s.st.b1 = 0;
+        s.st.seg = ordered ? -1 : 0;
+        s.st.deep = 0;
+        s.st.plain = !ordered;
+        s.st.sorted = -1;
+    }
+    __syncthreads();
+}
+
+// Loads the next window into s.ent and returns its size; 0 at the end.  Every
+// thread must be done with the last window.  Not inlined: the walk between two
+// windows keeps its registers.
+template <int BD, int WIN>
+static __device__ __noinline__ int window_next(WindowShared<WIN> &s) {
+    WindowLoader<BD, WIN> w(s);
+    if (w.cnt <= 0) return 0;
+    if (w.b0 < 0) {
+        w.template deal<0>();
+        w.b0 = 0;
+    }
+    const int n = w.next();
+    __syncthreads();
+    if (threadIdx.x == 0) s.st = w;
+    __syncthreads();
+    return n;
+}
+
 // large-K variant: per-thread sorted lists in shared memory; element k of a
 // thread's list sits at z[k * stride], f[k * stride]
 struct SmemTopK {

@@ -436,15 +436,20 @@ __device__ __forceinline__ void write_pixel_smem(const FineOut &o, int64_t pix, 
 // ---------------------------------------------------------------------------
 // fine pass: persistent blocks, one bin (bin x bin pixels = block) per item
 // ---------------------------------------------------------------------------
+// entries per window of the bin's list: a window of the usual bin is the whole
+// of it, and at 8 KB the blocks an SM holds stay limited by registers
+constexpr int fine_window(int BS) { return BS >= 16 ? 1024 : 512; }
+
 template <int KM, int BS, bool BL>
 __global__ void __launch_bounds__(BS *BS) k_fine(FineArgs a) {
     constexpr int BD = BS * BS;
-    __shared__ FaceRec s_rec[BD];
-    __shared__ int s_id[BD];
-    __shared__ float s_key[BD];
+    constexpr int WIN = fine_window(BS);
+    __shared__ float4 s_rec[BD][5];  // a, b, d, e, h of the staged records; boxes apart, lanes read them side by side
+    __shared__ float4 s_box[BD];
+    __shared__ WindowShared<WIN> s_win;
     __shared__ int s_item;
-    // dynamic: sort_cap bin entries; K > 16: afterwards the per-thread lists
-    extern __shared__ unsigned long long s_sort[];
+    // K > 16: the per-thread lists
+    extern __shared__ unsigned long long s_lists[];
     const int tid = threadIdx.x;
     // K <= 16: each warp covers an 8 x 4 block of the bin (about as wide as
     // tall, like the inflated face bboxes it is culled against); K > 16: two
@@ -487,76 +492,61 @@ __global__ void __launch_bounds__(BS *BS) k_fine(FineArgs a) {
         const int off = a.offsets[bin];
         TopK<(KM > 0 ? KM : 1)> tk;
         SmemTopK stk;
-        // The bin's list is sorted front to back in segments of up to sort_cap
-        // entries (one segment unless the bin holds more faces than that).
-        // K <= 16: each segment is sorted in shared memory right before it is
-        // walked.  K > 16: every segment is sorted first and written back to
-        // the (block-owned) list, so that the same shared memory then holds
-        // the per-pixel lists.
         if constexpr (KM > 0) {
             tk.init();
         } else {
-            for (int seg = 0; seg < cnt; seg += a.sort_cap) {
-                const int m = min(a.sort_cap, cnt - seg);
-                sort_entries<BD>(s_sort, a.lists + off + seg, m);
-                for (int i = tid; i < m; i += BD) a.lists[off + seg + i] = s_sort[i];
-                __syncthreads();
-            }
-            stk.z = reinterpret_cast<float *>(s_sort) + tid * a.K;
-            stk.f = reinterpret_cast<int *>(s_sort) + BD * a.K + tid * a.K;
+            stk.z = reinterpret_cast<float *>(s_lists) + tid * a.K;
+            stk.f = reinterpret_cast<int *>(s_lists) + BD * a.K + tid * a.K;
             stk.stride = 1;
             stk.K = a.K;
             stk.init();
         }
-        for (int seg = 0; seg < cnt; seg += a.sort_cap) {
-            const int m = min(a.sort_cap, cnt - seg);
-            if constexpr (KM > 0) sort_entries<BD>(s_sort, a.lists + off + seg, m);
-            const unsigned long long *ent = (KM > 0) ? s_sort : a.lists + off + seg;
-            // Chunks of BD faces, front to back: every lane walks the staged
-            // faces in order.  Faces are culled 32 at a time for the whole
-            // warp: lane j tests face jb + j against the rectangle spanned by
-            // the warp's pixel centres and against the warp's largest K-th
-            // depth; one ballot names the faces the warp walks pixel by pixel.
-            // A face is skipped by a lane when its bbox misses the pixel or its
-            // nearest corner lies behind the lane's K-th depth.  Once a warp's
-            // largest K-th depth lies in front of the next face, the rest of
-            // the segment is behind all its lanes, and the block stops when
-            // that holds for every warp.
+        auto kth = [&]() {
+            if constexpr (KM > 0) return tk.z[KM - 1];
+            else return stk.thr();
+        };
+        auto warp_kth = [&]() {
+            return __int_as_float(__reduce_max_sync(0xffffffffu, valid ? __float_as_int(kth()) : 0));
+        };
+        // The bin's faces in front-to-back windows (two warps' worth is not
+        // worth ordering; without depth culling the order buys nothing).
+        // Chunks of BD faces are staged; faces are culled 32 at a time for the
+        // whole warp: lane j tests face jb + j against the rectangle spanned
+        // by the warp's pixel centres and against the warp's largest K-th
+        // depth; one ballot names the faces the warp walks pixel by pixel.  A
+        // face is skipped by a lane when its bbox misses the pixel or its
+        // nearest corner lies behind the lane's K-th depth.  Once a warp's
+        // largest K-th depth falls into a bucket in front of the next face's,
+        // the rest of the window is behind all its lanes, and the block stops
+        // when everything left is behind every warp.
+        window_begin<BD>(s_win, a.lists + off, cnt, zcull && cnt > 64);
+        while (const int m = window_next<BD>(s_win)) {
             for (int base = 0; base < m; base += BD) {
                 const int mc = min(BD, m - base);
                 if (tid < mc) {
-                    const unsigned long long v = ent[base + tid];
-                    const int fid = (int)(unsigned)(v & 0xffffffffull);
-                    s_id[tid] = fid;
-                    s_key[tid] = __uint_as_float((unsigned)(v >> 32));
+                    const int fid = (int)(unsigned)(s_win.ent[base + tid] & 0xffffffffull);
                     const float4 *src = reinterpret_cast<const float4 *>(a.rec + fid);
-                    FaceRec R;
-                    R.a = __ldg(src + kRecA);
-                    R.b = __ldg(src + kRecB);
-                    R.c = __ldg(src + kRecC);
-                    R.d = __ldg(src + kRecD);
-                    R.e = __ldg(src + kRecE);
-                    R.h = __ldg(src + kRecH);
-                    s_rec[tid] = R;
+                    s_rec[tid][0] = __ldg(src + kRecA);
+                    s_rec[tid][1] = __ldg(src + kRecB);
+                    s_rec[tid][2] = __ldg(src + kRecD);
+                    s_rec[tid][3] = __ldg(src + kRecE);
+                    s_rec[tid][4] = __ldg(src + kRecH);
+                    s_box[tid] = __ldg(src + kRecC);
                 }
                 __syncthreads();
                 bool warp_done = false;
                 for (int jb = 0; jb < mc; jb += 32) {
-                    float thr;
-                    if constexpr (KM > 0) thr = tk.z[KM - 1];
-                    else thr = stk.thr();
-                    const float wthr =
-                        __int_as_float(__reduce_max_sync(0xffffffffu, valid ? __float_as_int(thr) : 0));
-                    if (zcull && s_key[jb] > wthr) {
+                    const float wthr = warp_kth();
+                    if (zcull && s_win.rank(wthr) < s_win.rank(entry_key(s_win.ent[base + jb]))) {
                         warp_done = true;
                         break;
                     }
                     const int jl = jb + lane;
                     bool hit = false;
                     if (jl < mc) {
-                        const float4 bb = s_rec[jl].c;
+                        const float4 bb = s_box[jl];
                         hit = bb.x <= wx1 && bb.y >= wx0 && bb.z <= wy1 && bb.w >= wy0 &&
-                              !(zcull && s_key[jl] > wthr);
+                              !(zcull && entry_key(s_win.ent[base + jl]) > wthr);
                     }
                     unsigned mask = __ballot_sync(0xffffffffu, hit);
                     while (mask) {
@@ -564,19 +554,18 @@ __global__ void __launch_bounds__(BS *BS) k_fine(FineArgs a) {
                         mask &= mask - 1;
                         if (!valid) continue;
                         FaceRec R;
-                        R.c = s_rec[jj].c;
+                        R.c = s_box[jj];
                         if (!in_bbox(R, p)) continue;
-                        if constexpr (KM > 0) thr = tk.z[KM - 1];
-                        else thr = stk.thr();
-                        if (zcull && s_key[jj] > thr) continue;
-                        R.a = s_rec[jj].a;
-                        R.b = s_rec[jj].b;
-                        R.d = s_rec[jj].d;
-                        R.e = s_rec[jj].e;
-                        R.h = s_rec[jj].h;
+                        const unsigned long long e = s_win.ent[base + jj];
+                        if (zcull && entry_key(e) > kth()) continue;
+                        R.a = s_rec[jj][0];
+                        R.b = s_rec[jj][1];
+                        R.d = s_rec[jj][2];
+                        R.e = s_rec[jj][3];
+                        R.h = s_rec[jj][4];
                         float z;
                         if (face_key_nobbox(R, p, fl, z)) {
-                            const int fid = s_id[jj];
+                            const int fid = (int)(unsigned)(e & 0xffffffffull);
                             if constexpr (KM > 0) {
                                 if (tk.admits(z, fid)) tk.insert(z, fid);
                             } else {
@@ -585,17 +574,10 @@ __global__ void __launch_bounds__(BS *BS) k_fine(FineArgs a) {
                         }
                     }
                 }
-                if (!warp_done && zcull && base + BD < m) {
-                    float thr;
-                    if constexpr (KM > 0) thr = tk.z[KM - 1];
-                    else thr = stk.thr();
-                    const float wthr =
-                        __int_as_float(__reduce_max_sync(0xffffffffu, valid ? __float_as_int(thr) : 0));
-                    warp_done = __uint_as_float((unsigned)(ent[base + BD] >> 32)) > wthr;
-                }
+                // a warp past the window's last useful face is done with the window
                 if (__syncthreads_and(warp_done)) break;
             }
-            __syncthreads();
+            if (__syncthreads_and(zcull && s_win.rest_behind(warp_kth()))) break;
         }
         if constexpr (KM > 0) {
             if (valid) write_pixel_vec<KM, BL>(a.out, ((int64_t)n * a.S + r) * a.S + c, a.K, tk, a.rec, p, fl, a.blend);
@@ -603,20 +585,21 @@ __global__ void __launch_bounds__(BS *BS) k_fine(FineArgs a) {
             // K > 16: the block writes its tile slot by slot: consecutive
             // threads take consecutive output slots of a tile row (coalesced),
             // each recomputing its slot's barycentrics and distance
-            s_id[tid] = valid ? stk.n : 0;
+            __shared__ int s_held[BD];
+            s_held[tid] = valid ? stk.n : 0;
             __syncthreads();
             const int K = a.K;
             const int rows = min(BS, a.S - by * BS), cols = min(BS, a.S - bx * BS);
             const int per_row = cols * K;
-            const float *lz = reinterpret_cast<const float *>(s_sort);
-            const int *lf = reinterpret_cast<const int *>(s_sort) + BD * K;
+            const float *lz = reinterpret_cast<const float *>(s_lists);
+            const int *lf = reinterpret_cast<const int *>(s_lists) + BD * K;
             for (int i = tid; i < rows * per_row; i += BD) {
                 const int ry = i / per_row, rem = i - ry * per_row;
                 const int cx = rem / K, k = rem - cx * K;
                 const int t = ry * BS + cx;
                 const int rr = by * BS + ry, cc = bx * BS + cx;
                 const int64_t sl = (((int64_t)n * a.S + rr) * a.S + cc) * K + k;
-                if (k < s_id[t]) {
+                if (k < s_held[t]) {
                     const int f = lf[t * K + k];
                     FaceRec R;
                     const float4 *src = reinterpret_cast<const float4 *>(a.rec + f);
@@ -712,8 +695,7 @@ static int km_for(int K) {
 template <int KM, int BS, bool BL>
 static cudaError_t launch_fine_t(const FineArgs &a, cudaStream_t st) {
     constexpr int BD = BS * BS;
-    // the sort buffer; KM == 0: the same memory then holds the per-thread lists
-    const size_t dyn = std::max((size_t)a.sort_cap * 8, (KM > 0) ? (size_t)0 : (size_t)BD * a.K * 8);
+    const size_t dyn = (KM > 0) ? (size_t)0 : (size_t)BD * a.K * 8;
     auto kern = k_fine<KM, BS, BL>;
     cudaError_t e = cudaSuccess;
     if (dyn > 0) {  // static + dynamic above 48 KB needs the opt-in
