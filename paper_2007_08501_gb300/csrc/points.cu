@@ -200,8 +200,8 @@ __device__ __forceinline__ void pt_write(const PtArgs &a, int64_t pix, const Top
     }
 #pragma unroll
     for (int k = 0; k < KM; ++k) {
-        if (k >= a.K) break;
-        pt_slot(a, s0 + k, tk.f[k], tk.z[k], p);
+        if (k < KM - a.K) continue;
+        pt_slot(a, s0 + k - (KM - a.K), tk.f[k], tk.z[k], p);
     }
 }
 
@@ -250,7 +250,7 @@ __global__ void __launch_bounds__(BS *BS) k_pfine(PtArgs a) {
         TopK<(KM > 0 ? KM : 1)> tk;
         SmemTopK stk;
         if constexpr (KM > 0) {
-            tk.init();
+            tk.init(a.K);
         } else {
             // every segment sorted first and written back, then the same shared
             // memory holds the per-pixel lists (rows of K per thread)
@@ -366,7 +366,7 @@ __global__ void __launch_bounds__(256) k_pnaive(PtArgs a, int n) {
     TopK<(KM > 0 ? KM : 1)> tk;
     SmemTopK stk;
     if constexpr (KM > 0) {
-        tk.init();
+        tk.init(a.K);
     } else {
         stk.z = reinterpret_cast<float *>(s_dyn) + threadIdx.x;
         stk.f = reinterpret_cast<int *>(s_dyn) + blockDim.x * a.K + threadIdx.x;

@@ -420,15 +420,29 @@ __device__ __forceinline__ bool key_less(float za, int fa, float zb, int fb) {
     return za < zb || (za == zb && fa < fb);
 }
 
-// Register-resident top-K (KM slots, sorted ascending).  Slots beyond the
-// runtime K are kept too: the first K of the top KM are the top K.
+// Register-resident top-K, sorted ascending: the last K of KM slots (the ones
+// before them hold -inf and never move), so z[KM - 1] is the K-th depth for
+// every K <= KM and culls as early.
 template <int KM>
 struct TopK {
     float z[KM];
     int f[KM];
-    __device__ __forceinline__ void init() {
+    __device__ __forceinline__ void init(int K) {
+        const float inf = __int_as_float(0x7f800000);
 #pragma unroll
-        for (int k = 0; k < KM; ++k) { z[k] = __int_as_float(0x7f800000); f[k] = 0x7fffffff; }
+        for (int k = 0; k < KM; ++k) {
+            const bool unused = k < KM - K;
+            z[k] = unused ? -inf : inf;
+            f[k] = unused ? -1 : 0x7fffffff;
+        }
+    }
+    // nearest entry (slot KM - K)
+    __device__ __forceinline__ void first(int K, float &zz, int &ff) const {
+        zz = z[0];
+        ff = f[0];
+#pragma unroll
+        for (int k = 1; k < KM; ++k)
+            if (k == KM - K) { zz = z[k]; ff = f[k]; }
     }
     __device__ __forceinline__ bool admits(float zz, int ff) const { return key_less(zz, ff, z[KM - 1], f[KM - 1]); }
     __device__ __forceinline__ void insert(float zz, int ff) {

@@ -299,11 +299,16 @@ __device__ __forceinline__ void write_pixel(const FineOut &o, int64_t pix, int K
                                             const FineBlend &bl) {
     const int64_t s0 = pix * (int64_t)K;
     FwdBlend fb;
-    if constexpr (BL) fb.begin(bl, tk.f[0] != 0x7fffffff, tk.z[0]);
+    if constexpr (BL) {
+        float z0;
+        int f0;
+        tk.first(K, z0, f0);
+        fb.begin(bl, f0 != 0x7fffffff, z0);
+    }
 #pragma unroll
     for (int k = 0; k < KM; ++k) {
-        if (k >= K) break;
-        const int64_t s = s0 + k;
+        if (k < KM - K) continue;
+        const int64_t s = s0 + k - (KM - K);
         const int f = tk.f[k];
         const bool store = !BL || bl.frag;
         if (f == 0x7fffffff) {
@@ -493,7 +498,7 @@ __global__ void __launch_bounds__(BS *BS) k_fine(FineArgs a) {
         TopK<(KM > 0 ? KM : 1)> tk;
         SmemTopK stk;
         if constexpr (KM > 0) {
-            tk.init();
+            tk.init(a.K);
         } else {
             stk.z = reinterpret_cast<float *>(s_lists) + tid * a.K;
             stk.f = reinterpret_cast<int *>(s_lists) + BD * a.K + tid * a.K;
@@ -648,7 +653,7 @@ __global__ void __launch_bounds__(256) k_naive(NaiveArgs a, int n) {
     TopK<(KM > 0 ? KM : 1)> tk;
     SmemTopK stk;
     if constexpr (KM > 0) {
-        tk.init();
+        tk.init(a.K);
     } else {
         stk.z = reinterpret_cast<float *>(s_dyn) + threadIdx.x;
         stk.f = reinterpret_cast<int *>(s_dyn) + blockDim.x * a.K + threadIdx.x;
