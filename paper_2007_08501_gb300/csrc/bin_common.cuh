@@ -165,6 +165,28 @@ __device__ __forceinline__ void sort_entries_regs(unsigned long long *s_sort, co
     __syncthreads();
 }
 
+// Bitonic sort of n2 (a power of two) entries in shared memory.
+template <int BD>
+__device__ __forceinline__ void bitonic_shared(unsigned long long *s_sort, int n2) {
+    const int tid = threadIdx.x;
+#pragma unroll 1
+    for (int k2 = 2; k2 <= n2; k2 <<= 1) {
+#pragma unroll 1
+        for (int j2 = k2 >> 1; j2 > 0; j2 >>= 1) {
+            for (int i = tid; i < (n2 >> 1); i += BD) {
+                const int lo = ((i & ~(j2 - 1)) << 1) | (i & (j2 - 1));
+                const int hi = lo + j2;
+                const unsigned long long x = s_sort[lo], y = s_sort[hi];
+                if ((x > y) == ((lo & k2) == 0)) {
+                    s_sort[lo] = y;
+                    s_sort[hi] = x;
+                }
+            }
+            __syncthreads();
+        }
+    }
+}
+
 // Sorts m <= sort-buffer bin entries (64-bit keys) from src into s_sort,
 // ascending; every thread of the block (BD threads) must call it.  A segment
 // that fits one entry per thread sorts in registers: partners closer than 32
@@ -209,23 +231,7 @@ __device__ __forceinline__ void sort_entries(unsigned long long *s_sort, const u
     }
     for (int i = tid; i < n2; i += BD) s_sort[i] = i < m ? src[i] : ~0ull;
     __syncthreads();
-    // bitonic sort in shared memory (padding entries sort last)
-#pragma unroll 1
-    for (int k2 = 2; k2 <= n2; k2 <<= 1) {
-#pragma unroll 1
-        for (int j2 = k2 >> 1; j2 > 0; j2 >>= 1) {
-            for (int i = tid; i < (n2 >> 1); i += BD) {
-                const int lo = ((i & ~(j2 - 1)) << 1) | (i & (j2 - 1));
-                const int hi = lo + j2;
-                const unsigned long long x = s_sort[lo], y = s_sort[hi];
-                if ((x > y) == ((lo & k2) == 0)) {
-                    s_sort[lo] = y;
-                    s_sort[hi] = x;
-                }
-            }
-            __syncthreads();
-        }
-    }
+    bitonic_shared<BD>(s_sort, n2);
 }
 
 // ---------------------------------------------------------------------------
@@ -269,6 +275,7 @@ struct WindowState {
     int seg;         // >= 0: next piece of the list (unordered, or a level-1 bucket that does not fit)
     int deep, plain;
     int sorted;      // level whose buckets order the current window, -1: none
+    int base;        // entries of that level in front of the current window
 };
 
 template <int WIN>
@@ -383,6 +390,7 @@ struct WindowLoader : WindowState {
             __syncthreads();
         }
         sorted = level;
+        base = s.pre[level][b];
         return n;
     }
 
@@ -456,6 +464,7 @@ __device__ __forceinline__ void window_begin(WindowShared<WIN> &s, const unsigne
         s.st.deep = 0;
         s.st.plain = !ordered;
         s.st.sorted = -1;
+        s.st.base = 0;
     }
     __syncthreads();
 }
