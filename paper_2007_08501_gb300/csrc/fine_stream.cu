@@ -17,10 +17,12 @@
 //
 // A pixel whose unsettled candidates outgrow the ring (rare on smooth meshes;
 // common on strongly deformed ones, whose tilted faces lie far behind their
-// nearest corner) is queued with its 8 x 4 block; a second pass walks the
-// queued blocks again for those pixels only, with a ring of 64 entries, at
-// least K, which cannot overflow.  Its shared memory (64 KB per block of 4
-// warps) is paid only by the blocks that need it.
+// nearest corner) keeps the ones behind the ring's in a second ring of its own
+// in local memory, drawn back as the first drains; only those pixels touch it.
+// Walking their blocks a second time, with 64 entries of shared memory per
+// pixel, took 4.7 of the 16.4 ms of a forward and backward of 20 views (512 px,
+// K = 50, 81,920 faces, a sixth of the pixels outgrowing the ring); with the
+// local ring those take 12.2 ms.
 //
 // The fine pass writes each slot as one 64-bit key: (depth bits << 32) | face
 // id, or -1 for an empty slot, into pix_to_face.  k_frag_attr, one thread per
@@ -38,9 +40,9 @@
 
 namespace mr {
 
-// unsettled candidates a pixel keeps on chip: first pass, second pass (>= K)
-constexpr int kRing1 = 16, kRing2 = 64;
-constexpr int kWarps1 = 8, kWarps2 = 4;  // warps per block of each pass
+// unsettled candidates a pixel keeps on chip, and beyond those (16 + 64 > K)
+constexpr int kRing = 16, kSpill = 64;
+constexpr int kStreamWarps = 8;
 
 __device__ __forceinline__ long long pack_key(float z, int f) {
     return (long long)(((unsigned long long)__float_as_uint(z) << 32) | (unsigned)f);
@@ -97,13 +99,9 @@ __device__ __forceinline__ bool rect_beyond_edge(const float4 &ra, const float4 
     return out && sliver <= 64.f;
 }
 
-// First pass (SECOND = false): every item, a ring of RING = 16 per pixel,
-// WARPS = 8 warps per block.  Pixels whose unsettled candidates outgrow it are
-// queued, per item, as a lane mask.  Second pass (SECOND = true): the queued
-// items again, only their queued lanes, with a ring of RING = 64 >= K, which
-// cannot overflow (a pixel never holds more than K - settled candidates).
-template <int BS, int RING, int WARPS, bool SECOND>
-__global__ void __launch_bounds__(WARPS * 32, SECOND ? 3 : 4) k_fine_stream(FineArgs a) {
+template <int BS>
+__global__ void __launch_bounds__(kStreamWarps * 32, 4) k_fine_stream(FineArgs a) {
+    constexpr int RING = kRing, WARPS = kStreamWarps;
     constexpr int SUB = BS * BS / 32;  // 8 x 4 pixel blocks per bin
     // per warp: the rings ([slot][lane]), depths then face ids
     extern __shared__ float s_ring[];
@@ -113,26 +111,13 @@ __global__ void __launch_bounds__(WARPS * 32, SECOND ? 3 : 4) k_fine_stream(Fine
     EvalFlags fl = a.fl;
     const int nb2 = a.nb * a.nb;
     const int K = a.K;
-    const long long total = SECOND ? 0ll : (long long)a.items * SUB;
+    const long long total = (long long)a.items * SUB;
     const float kInf = __int_as_float(0x7f800000);
     while (true) {
         long long item = 0;
-        unsigned lanes = 0xffffffffu;  // the lanes this pass takes
-        if constexpr (SECOND) {
-            unsigned long long e = 0ull;
-            if (lane == 0) {
-                const unsigned j = atomicAdd(a.redo_head, 1u);
-                e = j < *a.redo_q ? a.redo_items[j] : ~0ull;
-            }
-            e = __shfl_sync(0xffffffffu, e, 0);
-            if (e == ~0ull) break;
-            item = (long long)(e >> 32);
-            lanes = (unsigned)e;
-        } else {
-            if (lane == 0) item = (long long)atomicAdd(a.queue, 1u);
-            item = __shfl_sync(0xffffffffu, item, 0);
-            if (item >= total) break;
-        }
+        if (lane == 0) item = (long long)atomicAdd(a.queue, 1u);
+        item = __shfl_sync(0xffffffffu, item, 0);
+        if (item >= total) break;
         const int qb = (int)(item / SUB), sub = (int)(item - (long long)qb * SUB);
         const int bin = a.order ? __ldg(a.order + qb) : qb;  // longest bins first
         const int n = bin / nb2, rem = bin - n * nb2;
@@ -140,7 +125,7 @@ __global__ void __launch_bounds__(WARPS * 32, SECOND ? 3 : 4) k_fine_stream(Fine
         const int r = by * BS + (sub / (BS / 8)) * 4 + (lane >> 3);
         const int c = bx * BS + (sub % (BS / 8)) * 8 + (lane & 7);
         fl.znear = __ldg(a.cams + 16 * n + 13);
-        const bool valid = (r < a.S) && (c < a.S) && ((lanes >> lane) & 1u);
+        const bool valid = (r < a.S) && (c < a.S);
         const PixC p = pixel_centre(r, c, a.S);
         float wx0 = 1.f, wx1 = -1.f, wy0 = 1.f, wy1 = -1.f;
         {
@@ -158,15 +143,17 @@ __global__ void __launch_bounds__(WARPS * 32, SECOND ? 3 : 4) k_fine_stream(Fine
         // the bin's list, sorted front to back by k_sort_bins
         const unsigned long long *ent = a.lists + a.offsets[bin];
         const int64_t s0 = (((int64_t)n * a.S + r) * a.S + c) * K;
-        int head = 0, nr = 0, nfin = 0;           // ring head, unsettled entries, settled slots
+        int head = 0, nr = 0, nfin = 0;           // ring head, its entries, settled slots
+        unsigned long long spill[kSpill];         // entries behind a full ring, as packed keys
+        int shead = 0, ns = 0;                    // (ns > 0 only while nr == RING)
         float kth_z = kInf;                       // K-th entry while the list is full
         int kth_f = 0x7fffffff;
-        bool redo = false;
+        bool spilled = false;
         auto settle = [&](float z, int f) { a.out.pix_to_face[s0 + nfin] = pack_key(z, f); ++nfin; };
         for (int jb = 0; jb < cnt; jb += 32) {
-            // a lane that is done (or invalid, or left for the redo) needs no more faces
-            const bool live = valid && !redo && nfin < K;
-            const float thr = !live ? 0.f : (nfin + nr >= K ? kth_z : kInf);
+            // a lane that is done (or invalid) needs no more faces
+            const bool live = valid && nfin < K;
+            const float thr = !live ? 0.f : (nfin + nr + ns >= K ? kth_z : kInf);
             const float wthr = __int_as_float(__reduce_max_sync(0xffffffffu, __float_as_int(thr)));
             const int jl = jb + lane;
             int fid = 0;
@@ -202,9 +189,9 @@ __global__ void __launch_bounds__(WARPS * 32, SECOND ? 3 : 4) k_fine_stream(Fine
                 R.c.y = __shfl_sync(0xffffffffu, bb.y, src);
                 R.c.z = __shfl_sync(0xffffffffu, bb.z, src);
                 R.c.w = __shfl_sync(0xffffffffu, bb.w, src);
-                if (!valid || redo || nfin >= K) continue;
+                if (!valid || nfin >= K) continue;
                 if (!in_bbox(R, p)) continue;
-                const bool full = nfin + nr >= K;
+                const bool full = nfin + nr + ns >= K;
                 if (full && fkey > kth_z) continue;  // its depth is at least its key
                 const float4 *rs = reinterpret_cast<const float4 *>(a.rec + f);
                 R.a = __ldg(rs + kRecA);
@@ -222,14 +209,44 @@ __global__ void __launch_bounds__(WARPS * 32, SECOND ? 3 : 4) k_fine_stream(Fine
                     if (!(fz < fkey)) break;
                     settle(fz, rf[h][lane]);
                     ++head;
-                    --nr;
+                    if (ns > 0) {           // the freed place (the new tail) takes the next one
+                        const unsigned long long e = spill[shead & (kSpill - 1)];
+                        rz[h][lane] = entry_key(e);
+                        rf[h][lane] = (int)(unsigned)e;
+                        ++shead;
+                        --ns;
+                    } else {
+                        --nr;
+                    }
                 }
-                if (full) --nr;             // the K-th entry is displaced (nr >= 1: not done)
-                if (nr == RING) {           // no room: this pixel goes to the second pass
-                    redo = true;
-                    continue;
+                if (full) {                 // the K-th entry is displaced (there is one: not done)
+                    if (ns > 0) --ns;
+                    else --nr;
                 }
-                int pos = nr;               // insertion from the tail (arrivals are nearly sorted)
+                if (nr == RING) {
+                    spilled = true;
+                    const int hl = (head + RING - 1) & (RING - 1);
+                    const unsigned long long e = (unsigned long long)pack_key(z, f);
+                    const unsigned long long last = (unsigned long long)pack_key(rz[hl][lane], rf[hl][lane]);
+                    if (e < last) {         // the ring's last moves behind it
+                        --shead;
+                        spill[shead & (kSpill - 1)] = last;
+                        ++ns;
+                        --nr;
+                    } else {
+                        int pos = ns;
+                        while (pos > 0) {
+                            const unsigned long long o = spill[(shead + pos - 1) & (kSpill - 1)];
+                            if (o < e) break;
+                            spill[(shead + pos) & (kSpill - 1)] = o;
+                            --pos;
+                        }
+                        spill[(shead + pos) & (kSpill - 1)] = e;
+                        ++ns;
+                    }
+                }
+                const bool placed = nr == RING;  // behind the ring
+                int pos = placed ? 0 : nr;  // insertion from the tail (arrivals are nearly sorted)
                 while (pos > 0) {
                     const int hp = (head + pos - 1) & (RING - 1);
                     const float pz = rz[hp][lane];
@@ -240,36 +257,35 @@ __global__ void __launch_bounds__(WARPS * 32, SECOND ? 3 : 4) k_fine_stream(Fine
                     rf[hq][lane] = pf;
                     --pos;
                 }
-                const int hq = (head + pos) & (RING - 1);
-                rz[hq][lane] = z;
-                rf[hq][lane] = f;
-                ++nr;
-                if (nfin + nr >= K) {
+                if (!placed) {
+                    const int hq = (head + pos) & (RING - 1);
+                    rz[hq][lane] = z;
+                    rf[hq][lane] = f;
+                    ++nr;
+                }
+                if (nfin + nr + ns >= K) {
                     const int hl = (head + nr - 1) & (RING - 1);
                     kth_z = rz[hl][lane];
                     kth_f = rf[hl][lane];
+                    if (ns > 0) {
+                        const unsigned long long e = spill[(shead + ns - 1) & (kSpill - 1)];
+                        kth_z = entry_key(e);
+                        kth_f = (int)(unsigned)e;
+                    }
                 }
             }
         }
-        // everything left in the ring is settled; empty slots get -1
-        if (valid && !redo) {
-            while (nr > 0) {
-                const int h = head & (RING - 1);
-                settle(rz[h][lane], rf[h][lane]);
-                ++head;
-                --nr;
+        // everything left is settled; empty slots get -1
+        if (valid) {
+            for (; nr > 0; --nr, ++head) settle(rz[head & (RING - 1)][lane], rf[head & (RING - 1)][lane]);
+            for (; ns > 0; --ns, ++shead) {
+                const unsigned long long e = spill[shead & (kSpill - 1)];
+                settle(entry_key(e), (int)(unsigned)e);
             }
             for (int k = nfin; k < K; ++k) a.out.pix_to_face[s0 + k] = -1ll;
         }
-        // pixels whose unsettled candidates outgrew the ring: queued for the
-        // second pass (each item at most once, so the queue never fills)
-        if constexpr (!SECOND) {
-            const unsigned todo = __ballot_sync(0xffffffffu, valid && redo);
-            if (todo && lane == 0) {
-                atomicAdd(a.redo_count, (unsigned)__popc(todo));
-                a.redo_items[atomicAdd(a.redo_q, 1u)] = ((unsigned long long)item << 32) | todo;
-            }
-        }
+        const unsigned n_spilled = __popc(__ballot_sync(0xffffffffu, spilled));
+        if (n_spilled && lane == 0) atomicAdd(a.spilled, n_spilled);
     }
 }
 
@@ -373,32 +389,15 @@ static cudaError_t launch_sort_bins(const FineArgs &a, cudaStream_t st) {
 
 template <int BS>
 static cudaError_t launch_fine_stream_t(const FineArgs &a, cudaStream_t st) {
-    // first pass: every 8 x 4 block of every bin
-    {
-        auto kern = k_fine_stream<BS, kRing1, kWarps1, false>;
-        const size_t dyn = (size_t)2 * kWarps1 * kRing1 * 32 * sizeof(float);  // 32 KB
-        int bps = 0;
-        cudaError_t e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&bps, kern, kWarps1 * 32, dyn);
-        if (e != cudaSuccess) return e;
-        const long long warps = (long long)a.items * (BS * BS / 32);
-        const long long need = (warps + kWarps1 - 1) / kWarps1;
-        const int grid =
-            (int)std::max(1LL, std::min<long long>(need, (long long)mr_host::num_sms() * std::max(1, bps)));
-        kern<<<grid, kWarps1 * 32, dyn, st>>>(a);
-        if ((e = cudaGetLastError()) != cudaSuccess) return e;
-    }
-    // second pass: the queued blocks (their count is on the device; warps stop
-    // at the end of the queue)
-    auto kern = k_fine_stream<BS, kRing2, kWarps2, true>;
-    const size_t dyn = (size_t)2 * kWarps2 * kRing2 * 32 * sizeof(float);  // 64 KB
-    cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)dyn);
-    if (e != cudaSuccess) return e;
+    auto kern = k_fine_stream<BS>;
+    const size_t dyn = (size_t)2 * kStreamWarps * kRing * 32 * sizeof(float);  // 32 KB
     int bps = 0;
-    e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&bps, kern, kWarps2 * 32, dyn);
+    cudaError_t e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&bps, kern, kStreamWarps * 32, dyn);
     if (e != cudaSuccess) return e;
-    const long long need = ((long long)a.items * (BS * BS / 32) + kWarps2 - 1) / kWarps2;
+    const long long warps = (long long)a.items * (BS * BS / 32);
+    const long long need = (warps + kStreamWarps - 1) / kStreamWarps;
     const int grid = (int)std::max(1LL, std::min<long long>(need, (long long)mr_host::num_sms() * std::max(1, bps)));
-    kern<<<grid, kWarps2 * 32, dyn, st>>>(a);
+    kern<<<grid, kStreamWarps * 32, dyn, st>>>(a);
     return cudaGetLastError();
 }
 
