@@ -335,6 +335,31 @@ typedef struct {
 } rast_bin_layout;
 MESHRAST_API int rast_workspace_bin_layout(const rast_params *p, int64_t V, int64_t F, rast_bin_layout *out);
 
+/* ---- silhouette rendering on packed slots -------------------------------
+ * rast_blend_fwd / blend_rast_bwd for the silhouette blend where the caller
+ * wants the image and the vertex gradients, not the Fragment data: 8 bytes per
+ * slot that holds a face instead of 28 per slot, and the backward reads the
+ * face records the forward staged.  The image is rast_blend_fwd's (K <= 16 bit
+ * for bit; above, the product over a pixel's slots in the same tree order).
+ *   slots   uint64 (N, S, S, K): opaque, 16-byte aligned
+ *   keep    (N, S, S): product of 1 - prob over the pixel's slots
+ *   staged  rast_staged_bytes(F) bytes, 16-byte aligned, kept unchanged until
+ *           the backward
+ *   scratch (F, 12) floats of the backward, 16-byte aligned
+ * sil_packed tells whether the parameters have this form (binned, F < 2^30,
+ * and K <= 16 or max_faces_per_bin <= 8192 with clipped barycentrics or no
+ * blur); without it both return MESHRAST_ERR_UNSUPPORTED.  The workspace is
+ * that of rast_workspace_bytes; sil_bwd needs none. */
+MESHRAST_API size_t rast_staged_bytes(int64_t F);
+MESHRAST_API int sil_packed(const rast_params *p, int64_t V, int64_t F);
+MESHRAST_API int sil_fwd(const rast_params *p, const blend_params *bp, const float *verts, int64_t V,
+                         const int64_t *faces, int64_t F, const int64_t *first_face, const int64_t *num_faces,
+                         const float *cams, uint64_t *slots, float *keep, float *image, void *staged,
+                         void *workspace, size_t workspace_bytes, void *stream);
+MESHRAST_API int sil_bwd(const rast_params *p, const blend_params *bp, int64_t V, const int64_t *faces, int64_t F,
+                         const float *cams, const uint64_t *slots, const float *keep, const void *staged,
+                         const float *grad_image, float *scratch, float *grad_verts, void *stream);
+
 /* ---- forward without a caller-supplied workspace -------------------------
  * Not part of the paper's method; it exists for callers that cannot allocate
  * device memory at all -- for example a plugin inside a host application

@@ -177,6 +177,34 @@ class _Render(torch.autograd.Function):
         return gv, gc, None, None, None, None, None, None, None
 
 
+class _RenderSilhouette(torch.autograd.Function):
+    """The silhouette blend on packed slots: 8 bytes per slot that holds a face
+    go to the backward instead of the Fragment data, with the staged face
+    records.  ``colors`` do not enter."""
+
+    @staticmethod
+    def forward(ctx, verts, colors, faces, first_face, num_faces, cams, p, bp, ws):
+        N, S, K = p.N, p.image_size, p.faces_per_pixel
+        dev, V, F = verts.device, verts.shape[0], faces.shape[0]
+        buf = ws.get(p, V, F)
+        slots = torch.empty((N, S, S, K), dtype=torch.int64, device=dev)
+        keep = torch.empty((N, S, S), dtype=torch.float32, device=dev)
+        img = torch.empty((N, S, S, 4), dtype=torch.float32, device=dev)
+        staged = torch.empty(ops.rast_staged_bytes(F), dtype=torch.uint8, device=dev)
+        ops.sil_fwd(p, bp, verts, faces, first_face, num_faces, cams, slots, keep, img, staged, buf)
+        ctx.save_for_backward(verts, faces, first_face, num_faces, cams, slots, keep, staged)
+        ctx.p, ctx.bp = p, bp
+        return img
+
+    @staticmethod
+    def backward(ctx, g_img):
+        verts, faces, _, _, cams, slots, keep, staged = ctx.saved_tensors
+        gv = torch.empty_like(verts)
+        scratch = torch.empty((faces.shape[0], 12), dtype=torch.float32, device=verts.device)
+        ops.sil_bwd(ctx.p, ctx.bp, verts, faces, cams, slots, keep, staged, g_img.contiguous(), scratch, gv)
+        return gv, None, None, None, None, None, None, None, None
+
+
 def render_meshes(verts, faces, first_face, num_faces, cams, raster: RasterSettings, blend: BlendSettings,
                   colors=None, ws: Workspace = None):
     """RGBA image (N, S, S, 4) of a packed mesh batch: rasterize, then blend;
@@ -186,6 +214,11 @@ def render_meshes(verts, faces, first_face, num_faces, cams, raster: RasterSetti
         ws = Workspace(verts.device)
     if blend.rgb and colors is None:
         raise ValueError("rgb blending needs per-vertex colours")
+    if not blend.rgb:
+        p = raster.params(first_face.shape[0])
+        if ops.sil_packed(p, verts.shape[0], faces.shape[0]):
+            return _RenderSilhouette.apply(verts.contiguous(), colors, faces.contiguous(), first_face.contiguous(),
+                                           num_faces.contiguous(), cams.contiguous(), p, blend.params(), ws)
     if colors is None:
         colors = torch.zeros(0, 3, device=verts.device)
     return _Render.apply(verts.contiguous(), colors.contiguous(), faces.contiguous(), first_face.contiguous(),

@@ -9,6 +9,7 @@
 #include "meshrast.h"
 #include "rast_common.cuh"
 #include "rast_internal.h"
+#include "sil.cuh"
 
 namespace mr_host {
 
@@ -108,9 +109,25 @@ size_t rast_workspace_bytes(const rast_params *p, int64_t V, int64_t F) {
     return L.bytes;
 }
 
+// The faces' records and images: in the workspace, or in a buffer of the
+// caller's that outlives the call (the backward then need not stage again).
+struct Staged {
+    mr::FaceRec *rec;
+    int *face_mesh;
+};
+
+static Staged staged_in_ws(char *ws, const WsLayout &L) {
+    return {reinterpret_cast<mr::FaceRec *>(ws + L.records), reinterpret_cast<int *>(ws + L.face_mesh)};
+}
+
+static Staged staged_in(void *buf, int64_t F) {
+    char *b = static_cast<char *>(buf);
+    return {reinterpret_cast<mr::FaceRec *>(b), reinterpret_cast<int *>(b + (size_t)F * sizeof(mr::FaceRec))};
+}
+
 static int stage(const rast_params *p, const float *verts, int64_t V, const int64_t *faces, int64_t F,
                  const int64_t *first_face, const int64_t *num_faces, const float *cams, char *ws,
-                 const WsLayout &L, int do_count, cudaStream_t st) {
+                 const WsLayout &L, const Staged &sg, int do_count, cudaStream_t st) {
     mr::StageArgs a;
     a.verts = verts;
     a.V = V;
@@ -125,8 +142,8 @@ static int stage(const rast_params *p, const float *verts, int64_t V, const int6
     a.bin = p->bin_size > 0 ? p->bin_size : 1;
     a.nb = (int)L.nb;
     a.do_count = do_count;
-    a.rec = reinterpret_cast<mr::FaceRec *>(ws + L.records);
-    a.face_mesh = reinterpret_cast<int *>(ws + L.face_mesh);
+    a.rec = sg.rec;
+    a.face_mesh = sg.face_mesh;
     a.counts = do_count ? reinterpret_cast<int *>(ws + L.counts) : nullptr;
     a.status = reinterpret_cast<unsigned *>(ws + L.status);
     return mr::launch_stage(a, st) == cudaSuccess ? MESHRAST_OK : MESHRAST_ERR_CUDA;
@@ -138,12 +155,31 @@ static int check_ws(const rast_params *p, int64_t V, int64_t F, void *ws, size_t
     return MESHRAST_OK;
 }
 
+// Large K: the front-to-back streaming fine pass, when every bin's list is
+// sorted as one piece (capacity <= 8192) and a candidate's depth is never
+// below its face's nearest corner (clipped barycentrics, or no blur);
+// Fragment attributes (and the silhouette blend) in a pass of their own.
+static bool streams(const rast_params *p, int64_t NB) {
+    const bool zcull = p->clip_barycentric_coords || !(p->blur_radius > 0.f);
+    // (work items: 32-pixel blocks of every bin, counted by a 32-bit queue)
+    const bool items_fit = NB * (int64_t)(p->bin_size * p->bin_size / 32) < 0x7fffffffLL;
+    return p->faces_per_pixel > 16 && zcull && p->max_faces_per_bin <= 8192 && items_fit;
+}
+
+// Whether the silhouette can be kept as packed slots: binned, by a pass that
+// writes them (the block pass for K <= 16, the streaming pass above).
+static bool packed_path(const rast_params *p, int64_t F) {
+    if (p->bin_size <= 0 || F >= mr::kSilMaxFaces) return false;
+    const int64_t nb = (p->image_size + p->bin_size - 1) / p->bin_size;
+    return mr::fine_blends(p->faces_per_pixel, false) || streams(p, (int64_t)p->N * nb * nb);
+}
+
 // Forward rasterization; with `blend` set, the fine pass also applies the blend
 // (register path, K <= 16) and *blended tells whether it did.
 static int forward(const rast_params *p, const float *verts, int64_t V, const int64_t *faces, int64_t F,
                    const int64_t *first_face, const int64_t *num_faces, const float *cams, int64_t *pix_to_face,
                    float *zbuf, float *bary, float *dists, void *workspace, size_t workspace_bytes, void *stream,
-                   const mr::FineBlend *blend, bool *blended) {
+                   const mr::FineBlend *blend, bool *blended, void *staged = nullptr) {
     if (blended) *blended = false;
     if (!mr_host::check_params(p, V, F)) return MESHRAST_ERR_INVALID_ARG;
     if (mr_host::unsupported(p)) return MESHRAST_ERR_UNSUPPORTED;
@@ -155,7 +191,8 @@ static int forward(const rast_params *p, const float *verts, int64_t V, const in
     // no Fragment data at all: only when the fine pass itself blends the silhouette
     const bool no_frag = !pix_to_face && !zbuf && !bary && !dists;
     const bool fine_blend = blend && binned && mr::fine_blends((int)K, blend->rgb != 0);
-    if (slots > 0 && (!pix_to_face || !zbuf || !bary || !dists) && !(no_frag && fine_blend))
+    const bool packed = blend && blend->slots;  // (the caller has checked packed_path)
+    if (slots > 0 && !packed && (!pix_to_face || !zbuf || !bary || !dists) && !(no_frag && fine_blend))
         return MESHRAST_ERR_INVALID_ARG;
     WsLayout L;
     int rc = check_ws(p, V, F, workspace, workspace_bytes, &L);
@@ -167,7 +204,8 @@ static int forward(const rast_params *p, const float *verts, int64_t V, const in
     if (binned && L.NB > 0) {
         if (cudaMemsetAsync(ws + L.counts, 0, (size_t)L.NB * 4, st) != cudaSuccess) return MESHRAST_ERR_CUDA;
     }
-    rc = stage(p, verts, V, faces, F, first_face, num_faces, cams, ws, L, binned ? 1 : 0, st);
+    const Staged sg = staged ? staged_in(staged, F) : staged_in_ws(ws, L);
+    rc = stage(p, verts, V, faces, F, first_face, num_faces, cams, ws, L, sg, binned ? 1 : 0, st);
     if (rc) return rc;
     mr::EvalFlags fl;
     fl.persp = p->perspective_correct;
@@ -177,7 +215,7 @@ static int forward(const rast_params *p, const float *verts, int64_t V, const in
     mr::FineOut out{pix_to_face, zbuf, bary, dists};
     if (!binned) {
         mr::NaiveArgs a;
-        a.rec = reinterpret_cast<const mr::FaceRec *>(ws + L.records);
+        a.rec = sg.rec;
         a.cams = cams;
         a.first_face = first_face;
         a.num_faces = num_faces;
@@ -188,15 +226,7 @@ static int forward(const rast_params *p, const float *verts, int64_t V, const in
         a.out = out;
         return mr::launch_naive(a, p->N, st) == cudaSuccess ? MESHRAST_OK : MESHRAST_ERR_CUDA;
     }
-    // Large K: the front-to-back streaming fine pass, when every bin's list is
-    // sorted as one piece (capacity <= 8192) and a candidate's depth is never
-    // below its face's nearest corner (clipped barycentrics, or no blur);
-    // Fragment attributes (and the silhouette blend) in a pass of their own.
-    const bool zcull = p->clip_barycentric_coords || !(p->blur_radius > 0.f);
-    // (work items: 32-pixel blocks of every bin, counted by a 32-bit queue)
-    const bool items_fit = L.NB * (int64_t)(p->bin_size * p->bin_size / 32) < 0x7fffffffLL;
-    const bool streaming =
-        K > 16 && zcull && p->max_faces_per_bin <= 8192 && items_fit && pix_to_face && zbuf && bary && dists;
+    const bool streaming = streams(p, L.NB) && (packed || (pix_to_face && zbuf && bary && dists));
     // The block fine pass takes bins longest first.  The streaming pass keeps
     // the natural (image, bin) order: its items are small, and consecutive
     // items of one image keep that image's face records and lists in L2.
@@ -220,8 +250,8 @@ static int forward(const rast_params *p, const float *verts, int64_t V, const in
     sa.F = F;
     if (mr::launch_scan(sa, st) != cudaSuccess) return MESHRAST_ERR_CUDA;
     mr::FillArgs fa;
-    fa.rec = reinterpret_cast<const mr::FaceRec *>(ws + L.records);
-    fa.face_mesh = reinterpret_cast<const int *>(ws + L.face_mesh);
+    fa.rec = sg.rec;
+    fa.face_mesh = sg.face_mesh;
     fa.F = F;
     fa.S = (int)S;
     fa.bin = p->bin_size;
@@ -232,7 +262,7 @@ static int forward(const rast_params *p, const float *verts, int64_t V, const in
     fa.lists = reinterpret_cast<unsigned long long *>(ws + L.lists);
     if (mr::launch_fill(fa, st) != cudaSuccess) return MESHRAST_ERR_CUDA;
     mr::FineArgs ka;
-    ka.rec = reinterpret_cast<const mr::FaceRec *>(ws + L.records);
+    ka.rec = sg.rec;
     ka.cams = cams;
     ka.lists = reinterpret_cast<unsigned long long *>(ws + L.lists);
     ka.eff = reinterpret_cast<const int *>(ws + L.eff);
@@ -247,7 +277,12 @@ static int forward(const rast_params *p, const float *verts, int64_t V, const in
     ka.fl = fl;
     ka.out = out;
     std::memset(&ka.blend, 0, sizeof(ka.blend));
+    if (packed) {
+        ka.blend = *blend;
+        if (blended) *blended = true;
+    }
     if (streaming) {
+        if (packed) ka.out.pix_to_face = reinterpret_cast<int64_t *>(blend->slots);  // the keys, before they are packed
         int cap = 256;
         while (cap < p->max_faces_per_bin) cap <<= 1;
         ka.sort_cap = cap;
@@ -263,11 +298,13 @@ static int forward(const rast_params *p, const float *verts, int64_t V, const in
         fa2.fl = fl;
         fa2.sigma = blend ? blend->sigma : 1.f;
         fa2.image = (blend && !blend->rgb) ? blend->image : nullptr;
+        fa2.slots = packed ? blend->slots : nullptr;
+        fa2.keep = packed ? blend->keep : nullptr;
         if (fa2.image && blended) *blended = true;
         return mr::launch_frag_attr(fa2, st) == cudaSuccess ? MESHRAST_OK : MESHRAST_ERR_CUDA;
     }
     ka.sort_cap = 0;
-    if (fine_blend) {
+    if (fine_blend && !packed) {
         ka.blend = *blend;
         ka.blend.frag = no_frag ? 0 : 1;
         if (blended) *blended = true;
@@ -303,7 +340,7 @@ int rast_mesh_bwd(const rast_params *p, const float *verts, int64_t V, const int
     if (V > 0 && cudaMemsetAsync(grad_verts, 0, (size_t)V * 3 * sizeof(float), st) != cudaSuccess)
         return MESHRAST_ERR_CUDA;
     if (slots == 0 || (!grad_zbuf && !grad_bary && !grad_dists)) return MESHRAST_OK;
-    rc = stage(p, verts, V, faces, F, first_face, num_faces, cams, ws, L, 0, st);
+    rc = stage(p, verts, V, faces, F, first_face, num_faces, cams, ws, L, staged_in_ws(ws, L), 0, st);
     if (rc) return rc;
     mr::RastBwdArgs a;
     a.rec = reinterpret_cast<const mr::FaceRec *>(ws + L.records);
@@ -500,7 +537,7 @@ int blend_rast_bwd(const rast_params *p, const blend_params *bp, const float *ve
     if (rgb && V > 0 && cudaMemsetAsync(grad_vert_colors, 0, (size_t)V * 3 * sizeof(float), st) != cudaSuccess)
         return MESHRAST_ERR_CUDA;
     if (slots == 0) return MESHRAST_OK;
-    rc = stage(p, verts, V, faces, F, first_face, num_faces, cams, ws, L, 0, st);
+    rc = stage(p, verts, V, faces, F, first_face, num_faces, cams, ws, L, staged_in_ws(ws, L), 0, st);
     if (rc) return rc;
     mr::BlendArgs a;
     fill_blend(a, bp, N, S, K, pix_to_face, zbuf, bary, dists, faces, F, vert_colors, V);
@@ -525,6 +562,79 @@ int blend_rast_bwd(const rast_params *p, const blend_params *bp, const float *ve
     r.fl.blur = p->blur_radius;
     r.fl.znear = 0.f;
     return mr::launch_blend_rast_bwd(a, r, st) == cudaSuccess ? MESHRAST_OK : MESHRAST_ERR_CUDA;
+}
+
+size_t rast_staged_bytes(int64_t F) {
+    return F < 0 || F >= 0x7fffffffLL ? 0 : mr_host::align256((size_t)F * (sizeof(mr::FaceRec) + sizeof(int)) + 1);
+}
+
+int sil_packed(const rast_params *p, int64_t V, int64_t F) {
+    return mr_host::check_params(p, V, F) && !mr_host::unsupported(p) && packed_path(p, F) ? 1 : 0;
+}
+
+int sil_fwd(const rast_params *p, const blend_params *bp, const float *verts, int64_t V, const int64_t *faces,
+            int64_t F, const int64_t *first_face, const int64_t *num_faces, const float *cams, uint64_t *slots,
+            float *keep, float *image, void *staged, void *workspace, size_t workspace_bytes, void *stream) {
+    if (!mr_host::check_params(p, V, F)) return MESHRAST_ERR_INVALID_ARG;
+    if (mr_host::unsupported(p)) return MESHRAST_ERR_UNSUPPORTED;
+    int rc = check_blend(bp, p->N, p->image_size, p->faces_per_pixel);
+    if (rc) return rc;
+    if (bp->mode != MESHRAST_BLEND_SIL) return MESHRAST_ERR_INVALID_ARG;
+    if (!packed_path(p, F)) return MESHRAST_ERR_UNSUPPORTED;
+    if (p->N > 0 && (!slots || !keep || !image || !aligned16(slots) || !aligned16(image)))
+        return MESHRAST_ERR_INVALID_ARG;
+    if (!staged || !aligned16(staged)) return MESHRAST_ERR_INVALID_ARG;
+    mr::FineBlend fbl;
+    std::memset(&fbl, 0, sizeof(fbl));
+    fbl.on = 1;
+    fbl.sigma = bp->sigma;
+    fbl.gamma = bp->gamma;
+    fbl.znear = bp->znear;
+    fbl.zfar = bp->zfar;
+    fbl.eps = bp->eps;
+    fbl.F = F;
+    fbl.image = image;
+    fbl.slots = reinterpret_cast<unsigned long long *>(slots);
+    fbl.keep = keep;
+    return forward(p, verts, V, faces, F, first_face, num_faces, cams, nullptr, nullptr, nullptr, nullptr, workspace,
+                   workspace_bytes, stream, &fbl, nullptr, staged);
+}
+
+int sil_bwd(const rast_params *p, const blend_params *bp, int64_t V, const int64_t *faces, int64_t F,
+            const float *cams, const uint64_t *slots, const float *keep, const void *staged, const float *grad_image,
+            float *scratch, float *grad_verts, void *stream) {
+    if (!mr_host::check_params(p, V, F)) return MESHRAST_ERR_INVALID_ARG;
+    if (mr_host::unsupported(p)) return MESHRAST_ERR_UNSUPPORTED;
+    int rc = check_blend(bp, p->N, p->image_size, p->faces_per_pixel);
+    if (rc) return rc;
+    if (!packed_path(p, F)) return MESHRAST_ERR_UNSUPPORTED;
+    if (V > 0 && !grad_verts) return MESHRAST_ERR_INVALID_ARG;
+    cudaStream_t st = reinterpret_cast<cudaStream_t>(stream);
+    if (V > 0 && cudaMemsetAsync(grad_verts, 0, (size_t)V * 3 * sizeof(float), st) != cudaSuccess)
+        return MESHRAST_ERR_CUDA;
+    if (p->N == 0 || F == 0 || V == 0) return MESHRAST_OK;
+    if (!faces || !cams || !slots || !keep || !staged || !grad_image || !scratch || !aligned16(scratch) ||
+        !aligned16(staged))
+        return MESHRAST_ERR_INVALID_ARG;
+    if (cudaMemsetAsync(scratch, 0, (size_t)F * 12 * sizeof(float), st) != cudaSuccess) return MESHRAST_ERR_CUDA;
+    const Staged sg = staged_in(const_cast<void *>(staged), F);
+    mr::SilBwdArgs a;
+    a.rec = sg.rec;
+    a.face_mesh = sg.face_mesh;
+    a.faces = faces;
+    a.cams = cams;
+    a.slots = reinterpret_cast<const unsigned long long *>(slots);
+    a.keep = keep;
+    a.grad_image = grad_image;
+    a.acc = reinterpret_cast<float4 *>(scratch);
+    a.grad_verts = grad_verts;
+    a.F = F;
+    a.V = V;
+    a.N = p->N;
+    a.S = p->image_size;
+    a.K = p->faces_per_pixel;
+    a.sigma = bp->sigma;
+    return mr::launch_sil_bwd(a, st) == cudaSuccess ? MESHRAST_OK : MESHRAST_ERR_CUDA;
 }
 
 int rast_query_status(const void *workspace, uint32_t *status, void *stream) {

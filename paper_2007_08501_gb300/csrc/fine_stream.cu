@@ -28,7 +28,9 @@
 // id, or -1 for an empty slot, into pix_to_face.  k_frag_attr, one thread per
 // slot (consecutive slots on consecutive threads: coalesced), expands it into
 // pix_to_face, zbuf, barycentrics and distance, and applies the silhouette
-// blend (Algorithm 1) when asked.
+// blend (Algorithm 1) when asked.  For packed silhouette slots (sil.cuh) the fine
+// pass leaves the slots behind a pixel's last alone and its count in the pixel's
+// image word, and k_sil_attr turns the keys into packed slots in place.
 #include <cuda_runtime.h>
 
 #include <algorithm>
@@ -37,6 +39,7 @@
 #include "blend_common.cuh"
 #include "rast_common.cuh"
 #include "rast_internal.h"
+#include "sil.cuh"
 
 namespace mr {
 
@@ -99,7 +102,7 @@ __device__ __forceinline__ bool rect_beyond_edge(const float4 &ra, const float4 
     return out && sliver <= 64.f;
 }
 
-template <int BS>
+template <int BS, bool PACKED>
 __global__ void __launch_bounds__(kStreamWarps * 32, 4) k_fine_stream(FineArgs a) {
     constexpr int RING = kRing, WARPS = kStreamWarps;
     constexpr int SUB = BS * BS / 32;  // 8 x 4 pixel blocks per bin
@@ -282,7 +285,11 @@ __global__ void __launch_bounds__(kStreamWarps * 32, 4) k_fine_stream(FineArgs a
                 const unsigned long long e = spill[shead & (kSpill - 1)];
                 settle(entry_key(e), (int)(unsigned)e);
             }
-            for (int k = nfin; k < K; ++k) a.out.pix_to_face[s0 + k] = -1ll;
+            if constexpr (PACKED) {
+                reinterpret_cast<int *>(a.blend.image)[4 * (((int64_t)n * a.S + r) * a.S + c)] = nfin;
+            } else {
+                for (int k = nfin; k < K; ++k) a.out.pix_to_face[s0 + k] = -1ll;
+            }
         }
         const unsigned n_spilled = __popc(__ballot_sync(0xffffffffu, spilled));
         if (n_spilled && lane == 0) atomicAdd(a.spilled, n_spilled);
@@ -372,6 +379,56 @@ __global__ void __launch_bounds__(256, 6) k_frag_attr(FragAttrArgs a) {
     }
 }
 
+// The same for packed silhouette slots: 8 bytes read and written per slot that
+// holds a face (28 and every slot above), no barycentrics.
+// 20 views at 512 px, K = 50: 2.77 -> 2.08 ms.
+__global__ void __launch_bounds__(256, 6) k_sil_attr(FragAttrArgs a) {
+    __shared__ float s_keep[256];
+    const int K = a.K, S = a.S;
+    const int PB = 256 / K;
+    const int t = threadIdx.x, lane = t & 31;
+    const unsigned SS = (unsigned)S * (unsigned)S;
+    const unsigned q0 = blockIdx.x * (unsigned)PB;
+    const int lp = (int)__fdividef((float)t + 0.5f, (float)K);  // t / K (t < 256: exact)
+    const int k = t - lp * K;
+    const unsigned qi = q0 + (unsigned)lp;
+    const int64_t pix0 = (int64_t)blockIdx.y * SS + q0;
+    float keep = 1.f;
+    if (lp < PB && qi < SS) {
+        const int64_t pix = pix0 + lp, s = pix * K + k;
+        const int cnt = reinterpret_cast<const int *>(a.image)[4 * pix];
+        if (k == cnt) a.slots[s] = kSilEnd;
+        if (k < cnt) {
+            const unsigned long long v = a.slots[s];
+            const int f = (int)(unsigned)v;
+            const float4 *src = reinterpret_cast<const float4 *>(a.rec + f);
+            FaceRec R;
+            R.a = __ldg(src + kRecA);
+            R.b = __ldg(src + kRecB);
+            R.d = __ldg(src + kRecD);
+            const int r = (int)div_small(qi, (unsigned)S, a.magic_S), c = (int)qi - r * S;
+            int edge;
+            const float d = face_distance(R, pixel_centre(r, c, S), edge);
+            keep = __frcp_rn(1.f + expf(-d * a.inv_sigma));
+            a.slots[s] = sil_pack(d, f, edge);
+        }
+    }
+    // as above; the counts have been read once every thread is here
+    s_keep[t] = keep;
+    __syncthreads();
+    for (int q = t >> 5; q < PB; q += 8) {
+        float m = 1.f;
+        if (lane < K) m = s_keep[q * K + lane];
+        if (lane + 32 < K) m *= s_keep[q * K + lane + 32];
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1) m *= __shfl_xor_sync(0xffffffffu, m, o);
+        if (lane == 0 && q0 + (unsigned)q < SS) {
+            a.keep[pix0 + q] = m;
+            reinterpret_cast<float4 *>(a.image)[pix0 + q] = make_float4(0.f, 0.f, 0.f, 1.f - m);
+        }
+    }
+}
+
 // ---------------------------------------------------------------------------
 // launchers
 // ---------------------------------------------------------------------------
@@ -387,9 +444,9 @@ static cudaError_t launch_sort_bins(const FineArgs &a, cudaStream_t st) {
     return cudaGetLastError();
 }
 
-template <int BS>
+template <int BS, bool PACKED>
 static cudaError_t launch_fine_stream_t(const FineArgs &a, cudaStream_t st) {
-    auto kern = k_fine_stream<BS>;
+    auto kern = k_fine_stream<BS, PACKED>;
     const size_t dyn = (size_t)2 * kStreamWarps * kRing * 32 * sizeof(float);  // 32 KB
     int bps = 0;
     cudaError_t e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&bps, kern, kStreamWarps * 32, dyn);
@@ -404,8 +461,9 @@ static cudaError_t launch_fine_stream_t(const FineArgs &a, cudaStream_t st) {
 cudaError_t launch_fine_stream(const FineArgs &a, int bin, cudaStream_t st) {
     cudaError_t e = launch_sort_bins(a, st);
     if (e != cudaSuccess) return e;
-    if (bin == 8) return launch_fine_stream_t<8>(a, st);
-    if (bin == 16) return launch_fine_stream_t<16>(a, st);
+    const bool packed = a.blend.slots != nullptr;
+    if (bin == 8) return packed ? launch_fine_stream_t<8, true>(a, st) : launch_fine_stream_t<8, false>(a, st);
+    if (bin == 16) return packed ? launch_fine_stream_t<16, true>(a, st) : launch_fine_stream_t<16, false>(a, st);
     return cudaErrorInvalidValue;
 }
 
@@ -420,7 +478,8 @@ cudaError_t launch_frag_attr(const FragAttrArgs &a, cudaStream_t st) {
     b.inv_sigma = 1.f / a.sigma;
     b.magic_S = (unsigned)((0x100000000ull + (unsigned)a.S - 1) / (unsigned)a.S);
     const dim3 grid((unsigned)(((int64_t)a.S * a.S + PB - 1) / PB), (unsigned)N);
-    if (a.image) k_frag_attr<true><<<grid, 256, 0, st>>>(b);
+    if (a.slots) k_sil_attr<<<grid, 256, 0, st>>>(b);
+    else if (a.image) k_frag_attr<true><<<grid, 256, 0, st>>>(b);
     else k_frag_attr<false><<<grid, 256, 0, st>>>(b);
     return cudaGetLastError();
 }

@@ -22,6 +22,7 @@
 #include "rast_internal.h"
 #include "blend_common.cuh"
 #include "bin_common.cuh"
+#include "sil.cuh"
 
 namespace mr {
 
@@ -405,6 +406,35 @@ __device__ __forceinline__ void write_pixel_vec(const FineOut &o, int64_t pix, i
     if constexpr (BL) fb.end(bl, pix);
 }
 
+// A pixel's packed silhouette slots, and Algorithm 1 on them (the arithmetic
+// and order of FwdBlend).
+template <int KM>
+__device__ __forceinline__ void write_pixel_packed(const FineBlend &bl, int64_t pix, int K, const TopK<KM> &tk,
+                                                   const FaceRec *rec, const PixC &p) {
+    unsigned long long *out = bl.slots + pix * K;
+    float keep = 1.f;
+#pragma unroll
+    for (int k = 0; k < KM; ++k) {
+        if (k < KM - K) continue;
+        const int f = tk.f[k], j = k - (KM - K);
+        if (f == 0x7fffffff) {
+            out[j] = kSilEnd;
+            break;
+        }
+        FaceRec R;
+        const float4 *src = reinterpret_cast<const float4 *>(rec + f);
+        R.a = __ldg(src + kRecA);
+        R.b = __ldg(src + kRecB);
+        R.d = __ldg(src + kRecD);
+        int edge;
+        const float d = face_distance(R, p, edge);
+        keep *= sigmoidf_(d / bl.sigma);
+        out[j] = sil_pack(d, f, edge);
+    }
+    bl.keep[pix] = keep;
+    reinterpret_cast<float4 *>(bl.image)[pix] = make_float4(0.f, 0.f, 0.f, 1.f - keep);
+}
+
 // ---------------------------------------------------------------------------
 // fine pass: persistent blocks, one bin (bin x bin pixels = block) per item
 // ---------------------------------------------------------------------------
@@ -412,7 +442,8 @@ __device__ __forceinline__ void write_pixel_vec(const FineOut &o, int64_t pix, i
 // of it, and at 8 KB the blocks an SM holds stay limited by registers
 constexpr int fine_window(int BS) { return BS >= 16 ? 1024 : 512; }
 
-template <int KM, int BS, bool BL>
+// OUT: 0 Fragment data, 1 with the silhouette blend, 2 packed silhouette slots with it
+template <int KM, int BS, int OUT>
 __global__ void __launch_bounds__(BS *BS) k_fine(FineArgs a) {
     constexpr int BD = BS * BS;
     constexpr int WIN = fine_window(BS);
@@ -552,7 +583,12 @@ __global__ void __launch_bounds__(BS *BS) k_fine(FineArgs a) {
             if (__syncthreads_and(zcull && s_win.rest_behind(warp_kth()))) break;
         }
         if constexpr (KM > 0) {
-            if (valid) write_pixel_vec<KM, BL>(a.out, ((int64_t)n * a.S + r) * a.S + c, a.K, tk, a.rec, p, fl, a.blend);
+            const int64_t pix = ((int64_t)n * a.S + r) * a.S + c;
+            if constexpr (OUT == 2) {
+                if (valid) write_pixel_packed<KM>(a.blend, pix, a.K, tk, a.rec, p);
+            } else {
+                if (valid) write_pixel_vec<KM, OUT == 1>(a.out, pix, a.K, tk, a.rec, p, fl, a.blend);
+            }
         } else {
             // K > 16: the block writes its tile slot by slot: consecutive
             // threads take consecutive output slots of a tile row (coalesced),
@@ -748,11 +784,11 @@ static int km_for(int K) {
     return 0;  // shared-memory lists
 }
 
-template <int KM, int BS, bool BL>
+template <int KM, int BS, int OUT>
 static cudaError_t launch_fine_t(const FineArgs &a, cudaStream_t st) {
     constexpr int BD = BS * BS;
     const size_t dyn = (KM > 0) ? (size_t)0 : (size_t)BD * a.K * 8;
-    auto kern = k_fine<KM, BS, BL>;
+    auto kern = k_fine<KM, BS, OUT>;
     cudaError_t e = cudaSuccess;
     if (dyn > 0) {  // static + dynamic above 48 KB needs the opt-in
         e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)dyn);
@@ -773,19 +809,17 @@ bool fine_blends(int K, bool rgb) { return km_for(K) > 0 && !rgb; }
 
 cudaError_t launch_fine(const FineArgs &a, int bin, cudaStream_t st) {
     const int km = km_for(a.K);
-    const bool bl = a.blend.on != 0;
-#define MR_FINE(KM_)                                                          \
-    if (km == KM_) {                                                          \
-        if (bin == 8) return bl ? launch_fine_t<KM_, 8, true>(a, st)          \
-                                : launch_fine_t<KM_, 8, false>(a, st);        \
-        if (bin == 16) return bl ? launch_fine_t<KM_, 16, true>(a, st)        \
-                                 : launch_fine_t<KM_, 16, false>(a, st);      \
-    }
-    MR_FINE(1) MR_FINE(2) MR_FINE(4) MR_FINE(8) MR_FINE(16)
+    const int out = a.blend.on ? (a.blend.slots ? 2 : 1) : 0;
+#define MR_FINE(KM_, BS_)                                                              \
+    if (km == KM_ && bin == BS_)                                                       \
+        return out == 2   ? launch_fine_t<KM_, BS_, 2>(a, st)                          \
+               : out == 1 ? launch_fine_t<KM_, BS_, 1>(a, st) : launch_fine_t<KM_, BS_, 0>(a, st);
+    MR_FINE(1, 8) MR_FINE(2, 8) MR_FINE(4, 8) MR_FINE(8, 8) MR_FINE(16, 8)
+    MR_FINE(1, 16) MR_FINE(2, 16) MR_FINE(4, 16) MR_FINE(8, 16) MR_FINE(16, 16)
 #undef MR_FINE
     if (km == 0) {
-        if (bin == 8) return launch_fine_t<0, 8, false>(a, st);
-        if (bin == 16) return launch_fine_t<0, 16, false>(a, st);
+        if (bin == 8) return launch_fine_t<0, 8, 0>(a, st);
+        if (bin == 16) return launch_fine_t<0, 16, 0>(a, st);
     }
     return cudaErrorInvalidValue;
 }

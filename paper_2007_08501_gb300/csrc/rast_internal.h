@@ -66,6 +66,10 @@ struct FineBlend {
     const float *colors;
     int64_t F, V;
     float *image;
+    // packed silhouette slots (instead of Fragment data; sil.cuh) and the
+    // product of 1 - prob per pixel; NULL elsewhere
+    unsigned long long *slots;
+    float *keep;
 };
 
 struct FineArgs {
@@ -97,6 +101,23 @@ struct FragAttrArgs {
     float *image;     // non-NULL: silhouette blend (Algorithm 1) into (P, 4)
     unsigned magic_S; // ceil(2^32 / S), set by the launcher
     float inv_sigma;  // 1 / sigma, set by the launcher
+    unsigned long long *slots;  // non-NULL: packed slots in and out (sil.cuh), and the
+    float *keep;                //   product of 1 - prob per pixel
+};
+
+// Backward of the packed silhouette.
+struct SilBwdArgs {
+    const FaceRec *rec;
+    const int *face_mesh;
+    const int64_t *faces;
+    const float *cams;
+    const unsigned long long *slots;
+    const float *keep, *grad_image;
+    float4 *acc;        // 3 per face: edge i's (dL/d first corner, dL/d second corner), NDC x, y
+    float *grad_verts;
+    int64_t F, V;
+    int N, S, K;
+    float sigma;
 };
 
 struct NaiveArgs {
@@ -150,6 +171,7 @@ cudaError_t launch_naive(const NaiveArgs &a, int N, cudaStream_t st);
 // large K: front-to-back streaming fine pass + attribute pass (fine_stream.cu)
 cudaError_t launch_fine_stream(const FineArgs &a, int bin, cudaStream_t st);
 cudaError_t launch_frag_attr(const FragAttrArgs &a, cudaStream_t st);
+cudaError_t launch_sil_bwd(const SilBwdArgs &a, cudaStream_t st);
 cudaError_t launch_rast_bwd(const RastBwdArgs &a, int N, cudaStream_t st);
 cudaError_t launch_blend_fwd(const BlendArgs &a, cudaStream_t st);
 cudaError_t launch_blend_bwd(const BlendArgs &a, cudaStream_t st);

@@ -34,7 +34,7 @@ BLEND_RGB = 1
 EXPORTED = ("rast_workspace_bytes", "rast_mesh_fwd", "rast_mesh_bwd", "blend_fwd", "blend_bwd",
             "rast_query_status", "rast_bin_occupancy", "rast_strerror", "rast_mesh_fwd_static",
             "rast_query_static_status", "rast_workspace_bin_layout", "meshrast_fma_probe",
-            "blend_rast_bwd", "rast_blend_fwd",
+            "blend_rast_bwd", "rast_blend_fwd", "rast_staged_bytes", "sil_packed", "sil_fwd", "sil_bwd",
             "pts_workspace_bytes", "pts_rasterize_fwd", "pts_rasterize_bwd", "pts_composite_fwd",
             "pts_composite_bwd", "pts_bin_occupancy", "shade_fwd", "shade_bwd",
             "knn_workspace_bytes", "knn_index_workspace_bytes", "knn_points", "knn_points_bwd", "chamfer_fwd", "chamfer_bwd")
@@ -119,6 +119,14 @@ def load(build_if_missing: bool = False):
     L.rast_blend_fwd.restype = ctypes.c_int
     L.blend_rast_bwd.argtypes = [P, B, vp, i64, vp, i64, vp, vp, vp, vp, vp, vp, vp, vp, vp, vp, vp, vp, sz, vp]
     L.blend_rast_bwd.restype = ctypes.c_int
+    L.rast_staged_bytes.argtypes = [i64]
+    L.rast_staged_bytes.restype = sz
+    L.sil_packed.argtypes = [P, i64, i64]
+    L.sil_packed.restype = ctypes.c_int
+    L.sil_fwd.argtypes = [P, B, vp, i64, vp, i64, vp, vp, vp, vp, vp, vp, vp, vp, sz, vp]
+    L.sil_fwd.restype = ctypes.c_int
+    L.sil_bwd.argtypes = [P, B, i64, vp, i64, vp, vp, vp, vp, vp, vp, vp, vp]
+    L.sil_bwd.restype = ctypes.c_int
     L.rast_query_status.argtypes = [vp, ctypes.POINTER(ctypes.c_uint32), vp]
     L.rast_query_status.restype = ctypes.c_int
     L.rast_bin_occupancy.argtypes = [P, i64, i64, vp, ctypes.POINTER(ctypes.c_int32),
@@ -415,6 +423,48 @@ def blend_rast_bwd(p, bp, verts, faces, first_face, num_faces, cams, pix_to_face
         _ptr(grad_verts, torch.float32, "grad_verts"), _ptr(grad_vert_colors, torch.float32, "grad_vert_colors"),
         _ptr(workspace, None, "workspace"), workspace.numel() * workspace.element_size(), _stream(stream))
     _check(rc, "blend_rast_bwd")
+
+
+def rast_staged_bytes(F: int) -> int:
+    return int(load().rast_staged_bytes(int(F)))
+
+
+def sil_packed(p, V: int, F: int) -> bool:
+    """Whether sil_fwd / sil_bwd take these parameters."""
+    return bool(load().sil_packed(ctypes.byref(p), int(V), int(F)))
+
+
+def sil_fwd(p, bp, verts, faces, first_face, num_faces, cams, slots, keep, image, staged, workspace, stream=None):
+    """Silhouette image, packed slots and staged records of a mesh batch."""
+    _batch_inputs(p.N, verts, faces, first_face, num_faces, cams)
+    _slots(p.N, p.image_size, p.faces_per_pixel, (("slots", slots),))
+    _image(keep, p.N, p.image_size, 1, "keep")
+    _image(image, p.N, p.image_size, 4, "image")
+    _atleast(staged, rast_staged_bytes(faces.shape[0]), "staged")
+    rc = load().sil_fwd(
+        ctypes.byref(p), ctypes.byref(bp), _ptr(verts, torch.float32, "verts"), verts.shape[0],
+        _ptr(faces, torch.int64, "faces"), faces.shape[0],
+        _ptr(first_face, torch.int64, "first_face"), _ptr(num_faces, torch.int64, "num_faces"),
+        _ptr(cams, torch.float32, "cams"), _ptr(slots, torch.int64, "slots"), _ptr(keep, torch.float32, "keep"),
+        _ptr(image, torch.float32, "image"), _ptr(staged, torch.uint8, "staged"),
+        _ptr(workspace, None, "workspace"), workspace.numel() * workspace.element_size(), _stream(stream))
+    _check(rc, "sil_fwd")
+
+
+def sil_bwd(p, bp, verts, faces, cams, slots, keep, staged, grad_image, scratch, grad_verts, stream=None):
+    _batch_inputs(p.N, verts, faces, None, None, cams)
+    _slots(p.N, p.image_size, p.faces_per_pixel, (("slots", slots),))
+    _image(keep, p.N, p.image_size, 1, "keep")
+    _image(grad_image, p.N, p.image_size, 4, "grad_image")
+    _atleast(staged, rast_staged_bytes(faces.shape[0]), "staged")
+    _atleast(scratch, 12 * faces.shape[0], "scratch")
+    _atleast(grad_verts, _n(verts), "grad_verts")
+    rc = load().sil_bwd(
+        ctypes.byref(p), ctypes.byref(bp), verts.shape[0], _ptr(faces, torch.int64, "faces"), faces.shape[0],
+        _ptr(cams, torch.float32, "cams"), _ptr(slots, torch.int64, "slots"), _ptr(keep, torch.float32, "keep"),
+        _ptr(staged, torch.uint8, "staged"), _ptr(grad_image, torch.float32, "grad_image"),
+        _ptr(scratch, torch.float32, "scratch"), _ptr(grad_verts, torch.float32, "grad_verts"), _stream(stream))
+    _check(rc, "sil_bwd")
 
 
 def rast_query_status(workspace, stream=None) -> int:
