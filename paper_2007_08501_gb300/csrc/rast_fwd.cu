@@ -441,10 +441,12 @@ __device__ __forceinline__ void write_pixel_packed(const FineBlend &bl, int64_t 
 // entries per window of the bin's list: a window of the usual bin is the whole
 // of it, and at 8 KB the blocks an SM holds stay limited by registers
 constexpr int fine_window(int BS) { return BS >= 16 ? 1024 : 512; }
+// blocks of 256 threads per SM: 64, 80 and 128 registers hold the lists and the face test
+constexpr int fine_blocks(int KM) { return KM <= 4 ? 4 : KM == 8 ? 3 : 2; }
 
 // OUT: 0 Fragment data, 1 with the silhouette blend, 2 packed silhouette slots with it
 template <int KM, int BS, int OUT>
-__global__ void __launch_bounds__(BS *BS) k_fine(FineArgs a) {
+__global__ void __launch_bounds__(BS *BS, fine_blocks(KM) * 256 / (BS * BS)) k_fine(FineArgs a) {
     constexpr int BD = BS * BS;
     constexpr int WIN = fine_window(BS);
     __shared__ float4 s_rec[BD][5];  // a, b, d, e, h of the staged records; boxes apart, lanes read them side by side
