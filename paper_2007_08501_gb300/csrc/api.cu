@@ -262,6 +262,7 @@ static int forward(const rast_params *p, const float *verts, int64_t V, const in
     fa.lists = reinterpret_cast<unsigned long long *>(ws + L.lists);
     if (mr::launch_fill(fa, st) != cudaSuccess) return MESHRAST_ERR_CUDA;
     mr::FineArgs ka;
+    std::memset(&ka, 0, sizeof(ka));
     ka.rec = sg.rec;
     ka.cams = cams;
     ka.lists = reinterpret_cast<unsigned long long *>(ws + L.lists);
@@ -276,7 +277,6 @@ static int forward(const rast_params *p, const float *verts, int64_t V, const in
     ka.K = (int)K;
     ka.fl = fl;
     ka.out = out;
-    std::memset(&ka.blend, 0, sizeof(ka.blend));
     if (packed) {
         ka.blend = *blend;
         if (blended) *blended = true;
@@ -286,7 +286,9 @@ static int forward(const rast_params *p, const float *verts, int64_t V, const in
         int cap = 256;
         while (cap < p->max_faces_per_bin) cap <<= 1;
         ka.sort_cap = cap;
+        if (packed) ka.inv_sigma = 1.f / blend->sigma;
         if (mr::launch_fine_stream(ka, p->bin_size, st) != cudaSuccess) return MESHRAST_ERR_CUDA;
+        if (packed) return MESHRAST_OK;
         mr::FragAttrArgs fa2;
         fa2.rec = ka.rec;
         fa2.out = out;
@@ -298,12 +300,9 @@ static int forward(const rast_params *p, const float *verts, int64_t V, const in
         fa2.fl = fl;
         fa2.sigma = blend ? blend->sigma : 1.f;
         fa2.image = (blend && !blend->rgb) ? blend->image : nullptr;
-        fa2.slots = packed ? blend->slots : nullptr;
-        fa2.keep = packed ? blend->keep : nullptr;
         if (fa2.image && blended) *blended = true;
         return mr::launch_frag_attr(fa2, st) == cudaSuccess ? MESHRAST_OK : MESHRAST_ERR_CUDA;
     }
-    ka.sort_cap = 0;
     if (fine_blend && !packed) {
         ka.blend = *blend;
         ka.blend.frag = no_frag ? 0 : 1;

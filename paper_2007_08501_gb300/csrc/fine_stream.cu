@@ -28,9 +28,10 @@
 // id, or -1 for an empty slot, into pix_to_face.  k_frag_attr, one thread per
 // slot (consecutive slots on consecutive threads: coalesced), expands it into
 // pix_to_face, zbuf, barycentrics and distance, and applies the silhouette
-// blend (Algorithm 1) when asked.  For packed silhouette slots (sil.cuh) the fine
-// pass leaves the slots behind a pixel's last alone and its count in the pixel's
-// image word, and k_sil_attr turns the keys into packed slots in place.
+// blend (Algorithm 1) when asked.  For packed silhouette slots (sil.cuh) each
+// warp packs and blends its pixels itself once they are settled: as a pass of its
+// own that took 2.1 ms of 20 views at 512 px, K = 50 (a block for every five
+// pixels, most of them empty); here it adds 1.0 ms to the fine pass's 4.2.
 #include <cuda_runtime.h>
 
 #include <algorithm>
@@ -285,10 +286,43 @@ __global__ void __launch_bounds__(kStreamWarps * 32, 4) k_fine_stream(FineArgs a
                 const unsigned long long e = spill[shead & (kSpill - 1)];
                 settle(entry_key(e), (int)(unsigned)e);
             }
-            if constexpr (PACKED) {
-                reinterpret_cast<int *>(a.blend.image)[4 * (((int64_t)n * a.S + r) * a.S + c)] = nfin;
-            } else {
+            if constexpr (!PACKED)
                 for (int k = nfin; k < K; ++k) a.out.pix_to_face[s0 + k] = -1ll;
+        }
+        if constexpr (PACKED) {
+            // The warp packs its own 32 pixels' slots, one pixel at a time over
+            // the lanes: the keys are still in L2 and the faces' records in L1.
+            float keep = 1.f;
+            __syncwarp();
+            for (unsigned todo = __ballot_sync(0xffffffffu, valid && nfin > 0); todo; todo &= todo - 1) {
+                const int src = __ffs(todo) - 1;
+                const int cnt = __shfl_sync(0xffffffffu, nfin, src);
+                unsigned long long *slots = a.blend.slots + __shfl_sync(0xffffffffu, s0, src);
+                const PixC q = {__shfl_sync(0xffffffffu, p.xh, src), __shfl_sync(0xffffffffu, p.xl, src),
+                                __shfl_sync(0xffffffffu, p.yh, src), __shfl_sync(0xffffffffu, p.yl, src)};
+                float m = 1.f;
+                for (int k = lane; k < cnt; k += 32) {
+                    const int f = (int)(unsigned)__ldcg(slots + k);
+                    const float4 *rp = reinterpret_cast<const float4 *>(a.rec + f);
+                    FaceRec R;
+                    R.a = __ldg(rp + kRecA);
+                    R.b = __ldg(rp + kRecB);
+                    R.d = __ldg(rp + kRecD);
+                    int edge;
+                    const float d = face_distance(R, q, edge);
+                    m *= __frcp_rn(1.f + expf(-d * a.inv_sigma));  // 1 - prob = sigmoid(d / sigma)
+                    slots[k] = sil_pack(d, f, edge);
+                }
+                // Algorithm 1: alpha = 1 - prod_k (1 - prob_k), in k_frag_attr's tree order
+#pragma unroll
+                for (int o = 16; o > 0; o >>= 1) m *= __shfl_xor_sync(0xffffffffu, m, o);
+                if (lane == src) keep = m;
+            }
+            if (valid) {
+                if (nfin < K) a.blend.slots[s0 + nfin] = kSilEnd;
+                const int64_t pix = ((int64_t)n * a.S + r) * a.S + c;
+                a.blend.keep[pix] = keep;
+                reinterpret_cast<float4 *>(a.blend.image)[pix] = make_float4(0.f, 0.f, 0.f, 1.f - keep);
             }
         }
         const unsigned n_spilled = __popc(__ballot_sync(0xffffffffu, spilled));
@@ -379,56 +413,6 @@ __global__ void __launch_bounds__(256, 6) k_frag_attr(FragAttrArgs a) {
     }
 }
 
-// The same for packed silhouette slots: 8 bytes read and written per slot that
-// holds a face (28 and every slot above), no barycentrics.
-// 20 views at 512 px, K = 50: 2.77 -> 2.08 ms.
-__global__ void __launch_bounds__(256, 6) k_sil_attr(FragAttrArgs a) {
-    __shared__ float s_keep[256];
-    const int K = a.K, S = a.S;
-    const int PB = 256 / K;
-    const int t = threadIdx.x, lane = t & 31;
-    const unsigned SS = (unsigned)S * (unsigned)S;
-    const unsigned q0 = blockIdx.x * (unsigned)PB;
-    const int lp = (int)__fdividef((float)t + 0.5f, (float)K);  // t / K (t < 256: exact)
-    const int k = t - lp * K;
-    const unsigned qi = q0 + (unsigned)lp;
-    const int64_t pix0 = (int64_t)blockIdx.y * SS + q0;
-    float keep = 1.f;
-    if (lp < PB && qi < SS) {
-        const int64_t pix = pix0 + lp, s = pix * K + k;
-        const int cnt = reinterpret_cast<const int *>(a.image)[4 * pix];
-        if (k == cnt) a.slots[s] = kSilEnd;
-        if (k < cnt) {
-            const unsigned long long v = a.slots[s];
-            const int f = (int)(unsigned)v;
-            const float4 *src = reinterpret_cast<const float4 *>(a.rec + f);
-            FaceRec R;
-            R.a = __ldg(src + kRecA);
-            R.b = __ldg(src + kRecB);
-            R.d = __ldg(src + kRecD);
-            const int r = (int)div_small(qi, (unsigned)S, a.magic_S), c = (int)qi - r * S;
-            int edge;
-            const float d = face_distance(R, pixel_centre(r, c, S), edge);
-            keep = __frcp_rn(1.f + expf(-d * a.inv_sigma));
-            a.slots[s] = sil_pack(d, f, edge);
-        }
-    }
-    // as above; the counts have been read once every thread is here
-    s_keep[t] = keep;
-    __syncthreads();
-    for (int q = t >> 5; q < PB; q += 8) {
-        float m = 1.f;
-        if (lane < K) m = s_keep[q * K + lane];
-        if (lane + 32 < K) m *= s_keep[q * K + lane + 32];
-#pragma unroll
-        for (int o = 16; o > 0; o >>= 1) m *= __shfl_xor_sync(0xffffffffu, m, o);
-        if (lane == 0 && q0 + (unsigned)q < SS) {
-            a.keep[pix0 + q] = m;
-            reinterpret_cast<float4 *>(a.image)[pix0 + q] = make_float4(0.f, 0.f, 0.f, 1.f - m);
-        }
-    }
-}
-
 // ---------------------------------------------------------------------------
 // launchers
 // ---------------------------------------------------------------------------
@@ -478,8 +462,7 @@ cudaError_t launch_frag_attr(const FragAttrArgs &a, cudaStream_t st) {
     b.inv_sigma = 1.f / a.sigma;
     b.magic_S = (unsigned)((0x100000000ull + (unsigned)a.S - 1) / (unsigned)a.S);
     const dim3 grid((unsigned)(((int64_t)a.S * a.S + PB - 1) / PB), (unsigned)N);
-    if (a.slots) k_sil_attr<<<grid, 256, 0, st>>>(b);
-    else if (a.image) k_frag_attr<true><<<grid, 256, 0, st>>>(b);
+    if (a.image) k_frag_attr<true><<<grid, 256, 0, st>>>(b);
     else k_frag_attr<false><<<grid, 256, 0, st>>>(b);
     return cudaGetLastError();
 }

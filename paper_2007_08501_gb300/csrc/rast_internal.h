@@ -81,7 +81,8 @@ struct FineArgs {
     unsigned *queue;
     unsigned *spilled;          // large-K streaming pass: pixels whose unsettled candidates outgrew the ring
     int items, nb, S, K;
-    int sort_cap;  // bin entries sorted at a time (power of two)
+    int sort_cap;  // streaming pass: bin entries sorted at a time (power of two)
+    float inv_sigma;  // streaming pass with packed slots: 1 / sigma
     EvalFlags fl;
     FineOut out;
     FineBlend blend;
@@ -101,8 +102,6 @@ struct FragAttrArgs {
     float *image;     // non-NULL: silhouette blend (Algorithm 1) into (P, 4)
     unsigned magic_S; // ceil(2^32 / S), set by the launcher
     float inv_sigma;  // 1 / sigma, set by the launcher
-    unsigned long long *slots;  // non-NULL: packed slots in and out (sil.cuh), and the
-    float *keep;                //   product of 1 - prob per pixel
 };
 
 // Backward of the packed silhouette.
