@@ -251,9 +251,10 @@ struct RareQueue {
 
 // NDC corner gradients g[9] of face R (corner-0-relative record) through the
 // projection Jacobian and R^T of camera cam to world space: atomics into
-// grad_verts at the face's three vertices.
+// grad_verts at the face's three vertices (`pairs` as in red_add_row).
 __device__ __forceinline__ void scatter_corner_grads(const FaceRec &R, const float *cam, const int64_t *faces,
-                                                     int64_t f, const float (&g)[9], float *grad_verts) {
+                                                     int64_t f, const float (&g)[9], float *grad_verts,
+                                                     bool pairs) {
     const float fo = cam[12];
     const float v0x = R.a.x + R.a.z, v0y = R.a.y + R.a.w;
     const float Px[3] = {0.f, R.b.x, R.b.z}, Py[3] = {0.f, R.b.y, R.b.w};
@@ -265,11 +266,9 @@ __device__ __forceinline__ void scatter_corner_grads(const FaceRec &R, const flo
         const float gxv = g[3 * i] * fo * iz[i];
         const float gyv = g[3 * i + 1] * fo * iz[i];
         const float gzv = g[3 * i + 2] - (g[3 * i] * xn + g[3 * i + 1] * yn) * iz[i];
-        const int64_t vi = __ldg(faces + 3 * f + i);
-        float *gv = grad_verts + 3 * vi;
-        atomicAdd(gv + 0, cam[0] * gxv + cam[3] * gyv + cam[6] * gzv);
-        atomicAdd(gv + 1, cam[1] * gxv + cam[4] * gyv + cam[7] * gzv);
-        atomicAdd(gv + 2, cam[2] * gxv + cam[5] * gyv + cam[8] * gzv);
+        const float gw[3] = {cam[0] * gxv + cam[3] * gyv + cam[6] * gzv, cam[1] * gxv + cam[4] * gyv + cam[7] * gzv,
+                             cam[2] * gxv + cam[5] * gyv + cam[8] * gzv};
+        red_add_row<3>(grad_verts, __ldg(faces + 3 * f + i), gw, pairs);
     }
 }
 
@@ -301,7 +300,7 @@ __device__ __forceinline__ void flush_rare_slots(const RareQueue &q, const FaceR
             g[3 * j + 1] = gy[j];
             g[3 * j + 2] = gZ[j];
         }
-        scatter_corner_grads(R, cams + 16 * e.nf, faces, e.f, g, grad_verts);
+        scatter_corner_grads(R, cams + 16 * e.nf, faces, e.f, g, grad_verts, ((uintptr_t)grad_verts & 7u) == 0);
     }
 }
 

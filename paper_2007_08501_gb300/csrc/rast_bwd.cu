@@ -12,62 +12,68 @@
 #include "rast_common.cuh"
 #include "rast_internal.h"
 #include "rast_adjoint.cuh"
+#include "tile_sort.cuh"
 
 namespace mr {
 
-// One block = a 16 x 16 pixel tile of one image; each thread loops over its
-// pixel's K slots.  For every k the warp (2 rows x 16 pixels) sums the corner
-// gradients of lanes that hold the same face, and one lane per face applies
-// the projection Jacobian and R^T and issues the atomics.
+// One block = a 16 x 16 pixel tile of one image, kTileSlots slots per pixel at
+// a time, by face over the tile (tile_sort.cuh).  Bound by instructions (the
+// adjoint itself, ~700 per slot).  8 meshes of 5,120 faces, 256 px, K = 8: 110 -> 105
+// us.
 __global__ void __launch_bounds__(256) k_rast_bwd(RastBwdArgs a) {
-    // each warp covers an 8 x 4 block of the 16 x 16 tile: neighbouring pixels
-    // share faces, so the warp's grouping by face finds more peers
-    const int tx = ((threadIdx.x >> 5) & 1) * 8 + (threadIdx.x & 7), ty = (threadIdx.x >> 6) * 4 + ((threadIdx.x >> 3) & 3);
     const int n = blockIdx.z;
-    const int r = blockIdx.y * 16 + ty, c = blockIdx.x * 16 + tx;
-    const bool valid = (r < a.S) && (c < a.S);
-    const PixC p = pixel_centre(r, c, a.S);
-    const int64_t pix = ((int64_t)n * a.S + r) * a.S + c;
+    int tx, ty;
+    tile_xy(threadIdx.x, tx, ty);
+    const int row = blockIdx.y * 16 + ty, col = blockIdx.x * 16 + tx;
+    const int64_t s0 = row < a.S && col < a.S ? (((int64_t)n * a.S + row) * a.S + col) * a.K : -1;
+    __shared__ TileSort s_sorted;
     __shared__ RareSlot s_rare[kRareCap];
     __shared__ int s_nrare;
     if (threadIdx.x == 0) s_nrare = 0;
-    __syncthreads();
     const RareQueue rq{s_rare, &s_nrare};
-    for (int k = 0; k < a.K; ++k) {
-        const int64_t s = pix * a.K + k;
-        int64_t f = valid ? a.pix_to_face[s] : -1;
-        if (f >= a.F) f = -1;  // an id outside the batch contributes nothing
-        int nf = (f >= 0) ? a.face_mesh[f] : -1;
-        if (nf < 0) f = -1;
-        float g[9];
+    const bool pairs = ((uintptr_t)a.grad_verts & 7u) == 0;
+    for (int kb = 0; kb < a.K; kb += kTileSlots) {
+        const int cnt = tile_sort(s_sorted, [&](int k) {
+            const int64_t f = s0 >= 0 && kb + k < a.K ? __ldg(a.pix_to_face + s0 + kb + k) : -1;
+            return f >= 0 && f < a.F ? (int)f : -1;  // an id outside the batch contributes nothing
+        });
+        for (int i = threadIdx.x; i < ((cnt + 31) & ~31); i += 256) {
+            int key = -1, nf = -1;
+            float g[9];
 #pragma unroll
-        for (int j = 0; j < 9; ++j) g[j] = 0.f;
-        FaceRec R;
-        if (f >= 0) {
-            const float4 *src = reinterpret_cast<const float4 *>(a.rec + f);
-            R.a = __ldg(src + kRecA);
-            R.b = __ldg(src + kRecB);
-            R.c = __ldg(src + kRecC);
-            R.d = __ldg(src + kRecD);
-            R.e = __ldg(src + kRecE);
-            const float gz = a.grad_zbuf ? a.grad_zbuf[s] : 0.f;
-            const float gd = a.grad_dists ? a.grad_dists[s] : 0.f;
-            float gb0 = 0.f, gb1 = 0.f, gb2 = 0.f;
-            if (a.grad_bary) {
-                gb0 = a.grad_bary[3 * s];
-                gb1 = a.grad_bary[3 * s + 1];
-                gb2 = a.grad_bary[3 * s + 2];
+            for (int j = 0; j < 9; ++j) g[j] = 0.f;
+            FaceRec R;
+            if (i < cnt) {
+                const int e = s_sorted.order[i];
+                int px, py;
+                tile_xy(e & 255, px, py);
+                const int r = blockIdx.y * 16 + py, c = blockIdx.x * 16 + px;
+                const int64_t s = (((int64_t)n * a.S + r) * a.S + c) * a.K + kb + (e >> 8);
+                const int f = (int)__ldg(a.pix_to_face + s);
+                nf = __ldg(a.face_mesh + f);
+                const float gz = a.grad_zbuf ? __ldg(a.grad_zbuf + s) : 0.f;
+                const float gd = a.grad_dists ? __ldg(a.grad_dists + s) : 0.f;
+                float gb0 = 0.f, gb1 = 0.f, gb2 = 0.f;
+                if (a.grad_bary) {
+                    gb0 = __ldg(a.grad_bary + 3 * s);
+                    gb1 = __ldg(a.grad_bary + 3 * s + 1);
+                    gb2 = __ldg(a.grad_bary + 3 * s + 2);
+                }
+                if (nf >= 0 && (gz != 0.f || gd != 0.f || gb0 != 0.f || gb1 != 0.f || gb2 != 0.f)) {
+                    key = f;
+                    const float4 *src = reinterpret_cast<const float4 *>(a.rec + f);
+                    R.a = __ldg(src + kRecA);
+                    R.b = __ldg(src + kRecB);
+                    R.d = __ldg(src + kRecD);
+                    R.e = __ldg(src + kRecE);
+                    slot_corner_grads(R, pixel_centre(r, c, a.S), a.fl, gz, gd, gb0, gb1, gb2, g, rq, f, nf,
+                                      (py << 4) | px);
+                }
             }
-            if (gz != 0.f || gd != 0.f || gb0 != 0.f || gb1 != 0.f || gb2 != 0.f)
-                slot_corner_grads(R, p, a.fl, gz, gd, gb0, gb1, gb2, g, rq, (int)f, nf, (ty << 4) | tx);
-            else
-                f = -1;
+            if (run_sum<9>(key, g) && key >= 0)
+                scatter_corner_grads(R, a.cams + 16 * nf, a.faces, key, g, a.grad_verts, pairs);
         }
-        const int key = (int)f;
-        const unsigned peers = __match_any_sync(0xffffffffu, key);
-        group_sum<9>(peers, g);
-        if (key >= 0 && (int)(threadIdx.x & 31) == __ffs(peers) - 1)
-            scatter_corner_grads(R, a.cams + 16 * nf, a.faces, f, g, a.grad_verts);  // once per face and warp
+        __syncthreads();
     }
     flush_rare_slots(rq, a.rec, a.cams, a.faces, a.grad_verts, a.S, a.fl);
 }
