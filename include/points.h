@@ -95,6 +95,26 @@ MESHRAST_API int pts_composite_bwd(const pts_params *p, int32_t mode, const int6
                                    const float *features, int64_t P, int32_t D, const float *grad_image,
                                    float *grad_dists, float *grad_features, void *stream);
 
+/* Rasterization and compositing in one call, and their two adjoints, where the
+ * caller wants the image and the gradients, not the Fragment data (binned
+ * parameters only, else MESHRAST_ERR_UNSUPPORTED): 8 bytes per slot that holds
+ * a point.
+ *   slots   uint64 (N, S, S, K): opaque, 16-byte aligned
+ *   staged  pts_staged_bytes(P) bytes, 16-byte aligned, kept unchanged until
+ *           the backward
+ *   scratch of the backward, 16-byte aligned: 4, 8 or 12 floats per point for
+ *           D <= 2, <= 6, <= 8
+ * grad_points and grad_features are overwritten. */
+MESHRAST_API size_t pts_staged_bytes(int64_t P);
+MESHRAST_API int pts_render_fwd(const pts_params *p, int32_t mode, const float *points, int64_t P,
+                                const int64_t *first_point, const int64_t *num_points, const float *cams,
+                                const float *features, int32_t D, uint64_t *slots, float *image, void *staged,
+                                void *workspace, size_t workspace_bytes, void *stream);
+MESHRAST_API int pts_render_bwd(const pts_params *p, int32_t mode, int64_t P, const float *cams,
+                                const float *features, int32_t D, const uint64_t *slots, const void *staged,
+                                const float *grad_image, float *scratch, float *grad_points, float *grad_features,
+                                void *stream);
+
 /* Waits for the stream, then reports the bin occupancy of the last binned
  * pts_rasterize_fwd on this workspace (largest bin count, sum of counts). */
 MESHRAST_API int pts_bin_occupancy(const pts_params *p, int64_t P, const void *workspace, int32_t *max_count,

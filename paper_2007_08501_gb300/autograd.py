@@ -273,12 +273,46 @@ class _RenderPoints(torch.autograd.Function):
         return gp, gf, None, None, None, None, None
 
 
+class _RenderPointsPacked(torch.autograd.Function):
+    """The same on packed slots: 8 bytes per slot that holds a point go to the
+    backward instead of the Fragment data, with the staged point records."""
+
+    @staticmethod
+    def forward(ctx, points, features, first_point, num_points, cams, settings, ws):
+        N, P = first_point.shape[0], points.shape[0]
+        S, K = settings.image_size, settings.points_per_pixel
+        p = settings.params(N)
+        n = ops.pts_workspace_bytes(p, P)
+        if ws.buf is None or ws.buf.numel() < n:
+            ws.buf = torch.empty(n, dtype=torch.uint8, device=points.device)
+        slots = torch.empty((N, S, S, K), dtype=torch.int64, device=points.device)
+        img = torch.empty((N, S, S, features.shape[1]), dtype=torch.float32, device=points.device)
+        staged = torch.empty(ops.pts_staged_bytes(P), dtype=torch.uint8, device=points.device)
+        ops.pts_render_fwd(p, settings.mode, points, first_point, num_points, cams, features, slots, img, staged,
+                           ws.buf)
+        ctx.save_for_backward(points, features, cams, slots, staged)
+        ctx.p, ctx.mode = p, settings.mode
+        return img
+
+    @staticmethod
+    def backward(ctx, g_img):
+        points, features, cams, slots, staged = ctx.saved_tensors
+        gp, gf = torch.empty_like(points), torch.empty_like(features)
+        scratch = torch.empty(points.shape[0] * ops.pts_scratch_width(features.shape[1]), dtype=torch.float32,
+                              device=points.device)
+        ops.pts_render_bwd(ctx.p, ctx.mode, points, cams, features, slots, staged, g_img.contiguous(), scratch, gp, gf)
+        return gp, gf, None, None, None, None, None
+
+
 def render_points(points, features, first_point, num_points, cams, settings: PointSettings, ws: Workspace = None):
     """(N, S, S, D) image of a packed batch of point clouds: K nearest splats per
     pixel, Alpha or Norm compositing; differentiable in points and features."""
     if ws is None:
         ws = Workspace(points.device)
-    return _RenderPoints.apply(points.contiguous(), features.contiguous(), first_point.contiguous(),
+    fn = _RenderPoints
+    if settings.bin_size > 0 and features.dim() == 2 and features.shape[0] == points.shape[0]:
+        fn = _RenderPointsPacked
+    return fn.apply(points.contiguous(), features.contiguous(), first_point.contiguous(),
                                num_points.contiguous(), cams.contiguous(), settings, ws)
 
 

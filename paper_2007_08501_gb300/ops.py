@@ -36,7 +36,8 @@ EXPORTED = ("rast_workspace_bytes", "rast_mesh_fwd", "rast_mesh_bwd", "blend_fwd
             "rast_query_static_status", "rast_workspace_bin_layout", "meshrast_fma_probe",
             "blend_rast_bwd", "rast_blend_fwd", "rast_staged_bytes", "sil_packed", "sil_fwd", "sil_bwd",
             "pts_workspace_bytes", "pts_rasterize_fwd", "pts_rasterize_bwd", "pts_composite_fwd",
-            "pts_composite_bwd", "pts_bin_occupancy", "shade_fwd", "shade_bwd",
+            "pts_composite_bwd", "pts_bin_occupancy", "pts_staged_bytes", "pts_render_fwd", "pts_render_bwd",
+             "shade_fwd", "shade_bwd",
             "knn_workspace_bytes", "knn_index_workspace_bytes", "knn_points", "knn_points_bwd", "chamfer_fwd", "chamfer_bwd")
 
 SHADE_FLAT, SHADE_GOURAUD, SHADE_PHONG = 0, 1, 2
@@ -157,6 +158,12 @@ def load(build_if_missing: bool = False):
     L.pts_composite_fwd.restype = ctypes.c_int
     L.pts_composite_bwd.argtypes = [Q, ctypes.c_int32, vp, vp, vp, i64, ctypes.c_int32, vp, vp, vp, vp]
     L.pts_composite_bwd.restype = ctypes.c_int
+    L.pts_staged_bytes.argtypes = [i64]
+    L.pts_staged_bytes.restype = sz
+    L.pts_render_fwd.argtypes = [Q, ctypes.c_int32, vp, i64, vp, vp, vp, vp, ctypes.c_int32, vp, vp, vp, vp, sz, vp]
+    L.pts_render_fwd.restype = ctypes.c_int
+    L.pts_render_bwd.argtypes = [Q, ctypes.c_int32, i64, vp, vp, ctypes.c_int32, vp, vp, vp, vp, vp, vp, vp]
+    L.pts_render_bwd.restype = ctypes.c_int
     L.pts_bin_occupancy.argtypes = [Q, i64, vp, ctypes.POINTER(ctypes.c_int32), ctypes.POINTER(ctypes.c_int64), vp]
     L.pts_bin_occupancy.restype = ctypes.c_int
     L.rast_strerror.argtypes = [ctypes.c_int]
@@ -579,6 +586,57 @@ def pts_composite_bwd(p, mode, idx, dists, features, grad_image, grad_dists, gra
                                   _ptr(grad_dists, torch.float32, "grad_dists"),
                                   _ptr(grad_features, torch.float32, "grad_features"), _stream(stream))
     _check(rc, "pts_composite_bwd")
+
+
+def pts_staged_bytes(P: int) -> int:
+    return int(load().pts_staged_bytes(int(P)))
+
+
+def _pts_features(points, features):
+    if features.dim() != 2 or features.shape[0] != points.shape[0]:
+        raise MeshRastError("features must be (P, D)")
+
+
+def pts_render_fwd(p, mode, points, first_point, num_points, cams, features, slots, image, staged, workspace,
+                   stream=None):
+    """Image, packed slots and staged records of a batch of point clouds."""
+    _batch_inputs(p.N, points, None, first_point, num_points, cams, "points")
+    _pts_features(points, features)
+    _slots(p.N, p.image_size, p.points_per_pixel, (("slots", slots),))
+    _image(image, p.N, p.image_size, features.shape[1], "image")
+    _atleast(staged, pts_staged_bytes(points.shape[0]), "staged")
+    rc = load().pts_render_fwd(
+        ctypes.byref(p), int(mode), _ptr(points, torch.float32, "points"), points.shape[0],
+        _ptr(first_point, torch.int64, "first_point"), _ptr(num_points, torch.int64, "num_points"),
+        _ptr(cams, torch.float32, "cams"), _ptr(features, torch.float32, "features"), features.shape[1],
+        _ptr(slots, torch.int64, "slots"), _ptr(image, torch.float32, "image"), _ptr(staged, torch.uint8, "staged"),
+        _ptr(workspace, None, "workspace"), workspace.numel() * workspace.element_size(), _stream(stream))
+    _check(rc, "pts_render_fwd")
+
+
+def pts_scratch_width(D: int) -> int:
+    """Floats of pts_render_bwd's scratch per point."""
+    return 4 if D <= 2 else 8 if D <= 6 else 12
+
+
+def pts_render_bwd(p, mode, points, cams, features, slots, staged, grad_image, scratch, grad_points, grad_features,
+                   stream=None):
+    P = points.shape[0]
+    _pts_features(points, features)
+    _atleast(cams, 16 * p.N, "cams")
+    _slots(p.N, p.image_size, p.points_per_pixel, (("slots", slots),))
+    _image(grad_image, p.N, p.image_size, features.shape[1], "grad_image")
+    _atleast(staged, pts_staged_bytes(P), "staged")
+    _atleast(scratch, P * pts_scratch_width(features.shape[1]), "scratch")
+    _atleast(grad_points, 3 * P, "grad_points")
+    _atleast(grad_features, features.numel(), "grad_features")
+    rc = load().pts_render_bwd(
+        ctypes.byref(p), int(mode), P, _ptr(cams, torch.float32, "cams"), _ptr(features, torch.float32, "features"),
+        features.shape[1], _ptr(slots, torch.int64, "slots"), _ptr(staged, torch.uint8, "staged"),
+        _ptr(grad_image, torch.float32, "grad_image"), _ptr(scratch, torch.float32, "scratch"),
+        _ptr(grad_points, torch.float32, "grad_points"), _ptr(grad_features, torch.float32, "grad_features"),
+        _stream(stream))
+    _check(rc, "pts_render_bwd")
 
 
 def pts_bin_occupancy(p, P, workspace, stream=None):
