@@ -20,8 +20,9 @@ __device__ __forceinline__ int find_mesh(const int64_t *first_face, int N, int64
 // or -1.  Thread 0 looks up the block's first element once; threads whose
 // element lies in that image's range skip their own binary search.  Every
 // thread of the block must call it (it synchronises the block).
+// `block`: image of the block's first element, or -1.
 __device__ __forceinline__ int block_find_mesh(const int64_t *first, const int64_t *num, int N, int64_t count,
-                                               int64_t i) {
+                                               int64_t i, int &block) {
     __shared__ int s_n;
     __shared__ long long s_lo, s_hi;
     if (threadIdx.x == 0) {
@@ -32,6 +33,7 @@ __device__ __forceinline__ int block_find_mesh(const int64_t *first, const int64
         s_hi = n0 >= 0 ? first[n0] + num[n0] : 0;
     }
     __syncthreads();
+    block = s_n;
     if (i >= count) return -1;
     if (s_n >= 0 && i >= s_lo && i < s_hi) return s_n;
     const int n = find_mesh(first, N, i);
@@ -95,6 +97,62 @@ __device__ __forceinline__ void bin_rect_box(const float4 &box, int S, int bin, 
 __device__ __forceinline__ void bin_rect(const FaceRec &R, int S, int bin, int &bx0, int &bx1, int &by0,
                                          int &by1) {
     bin_rect_box(R.c, S, bin, bx0, bx1, by0, by1);
+}
+
+// The warp's (element, bin) pairs, one bin per lane and step: f(key) with key -1
+// for lanes whose rectangle is done.  Every lane of the warp calls it.
+template <class F>
+__device__ __forceinline__ void for_bins(int n, int nb, int bx0, int bx1, int by0, int by1, const F &f) {
+    const int cnt = max(0, bx1 - bx0 + 1) * max(0, by1 - by0 + 1);
+    const int wmax = __reduce_max_sync(0xffffffffu, cnt);
+    int bx = bx0, row = (n * nb + by0) * nb;
+    for (int i = 0; i < wmax; ++i) {
+        f(i < cnt ? row + bx : -1);
+        if (++bx > bx1) { bx = bx0; row += nb; }
+    }
+}
+
+// Adds the warp's pairs to the bins' counts, equal bins of a step as one.
+__device__ __forceinline__ void count_bins(int *counts, int n, int nb, int bx0, int bx1, int by0, int by1) {
+    const int lane = threadIdx.x & 31;
+    for_bins(n, nb, bx0, bx1, by0, by1, [&](int key) {
+        const unsigned grp = __match_any_sync(0xffffffffu, key);
+        if (key >= 0 && lane == __ffs(grp) - 1) atomicAdd(counts + key, __popc(grp));
+    });
+}
+
+// Appends `entry` to the lists of the element's bins (up to eff entries each
+// from offsets), four steps' cursor additions in flight at a time: one at a
+// time, each waited for its round trip to L2 (1.3M faces in 14M pairs: MRFILL).
+__device__ __forceinline__ void fill_bins(unsigned long long *lists, int *cursor, const int *eff, const int *offsets,
+                                          unsigned long long entry, int n, int nb, int bx0, int bx1, int by0, int by1) {
+    constexpr int U = 4;
+    const int lane = threadIdx.x & 31;
+    const unsigned lt = (1u << lane) - 1u;
+    const int cnt = max(0, bx1 - bx0 + 1) * max(0, by1 - by0 + 1);
+    const int wmax = __reduce_max_sync(0xffffffffu, cnt);
+    int bx = bx0, row = (n * nb + by0) * nb;
+    for (int i = 0; i < wmax; i += U) {
+        int key[U], base[U], room[U], off[U];
+        unsigned grp[U];
+#pragma unroll
+        for (int u = 0; u < U; ++u) {
+            key[u] = i + u < cnt ? row + bx : -1;
+            if (++bx > bx1) { bx = bx0; row += nb; }
+            grp[u] = __match_any_sync(0xffffffffu, key[u]);
+            base[u] = room[u] = off[u] = 0;
+            if (key[u] >= 0) {
+                if (lane == __ffs(grp[u]) - 1) base[u] = atomicAdd(cursor + key[u], __popc(grp[u]));
+                room[u] = eff[key[u]];
+                off[u] = offsets[key[u]];
+            }
+        }
+#pragma unroll
+        for (int u = 0; u < U; ++u) {
+            const int slot = __shfl_sync(0xffffffffu, base[u], __ffs(grp[u]) - 1) + __popc(grp[u] & lt);
+            if (key[u] >= 0 && slot < room[u]) lists[off[u] + slot] = entry;
+        }
+    }
 }
 
 // Bitonic sort of N2 = BD * E entries, E consecutive entries per thread in

@@ -82,13 +82,17 @@ __device__ __forceinline__ float splat_d(const float4 &a, const PixC &p) {
 // ---------------------------------------------------------------------------
 __global__ void __launch_bounds__(256) k_pstage(PtArgs a, int do_count) {
     const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+    __shared__ float s_cam[16];
     PtRec R;
     R.a = make_float4(0.f, 0.f, 0.f, 0.f);
     R.b = make_float4(__int_as_float(0x7f800000), 0.f, 0.f, 0.f);
-    int n = block_find_mesh(a.first, a.num, a.N, a.P, i);
+    int block;
+    int n = block_find_mesh(a.first, a.num, a.N, a.P, i, block);
+    if (threadIdx.x < 16 && block >= 0) s_cam[threadIdx.x] = a.cams[16 * block + threadIdx.x];
+    __syncthreads();
     if (i < a.P) {
         if (n >= 0) {
-            const float *cam = a.cams + 16 * n;
+            const float *cam = n == block ? s_cam : a.cams + 16 * n;
             const float px = a.points[3 * i], py = a.points[3 * i + 1], pz = a.points[3 * i + 2];
             if (!(isfinite(px) && isfinite(py) && isfinite(pz))) {
                 set_status(a.status, MESHRAST_ST_NONFINITE);
@@ -112,16 +116,7 @@ __global__ void __launch_bounds__(256) k_pstage(PtArgs a, int do_count) {
     if (!do_count) return;
     int bx0 = 1, bx1 = 0, by0 = 1, by1 = 0;
     if (n >= 0) bin_rect_box(splat_box(R, a.radius), a.S, a.bin, bx0, bx1, by0, by1);
-    const int nbx = max(0, bx1 - bx0 + 1), nby = max(0, by1 - by0 + 1);
-    const int cnt = nbx * nby;
-    const int wmax = __reduce_max_sync(0xffffffffu, cnt);
-    const int lane = threadIdx.x & 31;
-    for (int j = 0; j < wmax; ++j) {
-        int key = -1;
-        if (j < cnt) key = (n * a.nb + by0 + j / nbx) * a.nb + bx0 + j % nbx;
-        const unsigned grp = __match_any_sync(0xffffffffu, key);
-        if (key >= 0 && lane == __ffs(grp) - 1) atomicAdd(a.counts + key, __popc(grp));
-    }
+    count_bins(a.counts, n, a.nb, bx0, bx1, by0, by1);
 }
 
 __global__ void __launch_bounds__(256) k_pfill(PtArgs a) {
@@ -137,27 +132,10 @@ __global__ void __launch_bounds__(256) k_pfill(PtArgs a) {
     }
     int bx0 = 1, bx1 = 0, by0 = 1, by1 = 0;
     if (n >= 0) bin_rect_box(splat_box(R, a.radius), a.S, a.bin, bx0, bx1, by0, by1);
-    const int nbx = max(0, bx1 - bx0 + 1), nby = max(0, by1 - by0 + 1);
-    const int cnt = nbx * nby;
     // depth bits (positive float) in the high word: integer order = front to back, ties by id
     const unsigned long long entry =
         n >= 0 ? (((unsigned long long)__float_as_uint(R.b.x) << 32) | (unsigned)i) : 0ull;
-    const int wmax = __reduce_max_sync(0xffffffffu, cnt);
-    const int lane = threadIdx.x & 31;
-    const unsigned lt = (1u << lane) - 1u;
-    for (int j = 0; j < wmax; ++j) {
-        int key = -1;
-        if (j < cnt) key = (n * a.nb + by0 + j / nbx) * a.nb + bx0 + j % nbx;
-        const unsigned grp = __match_any_sync(0xffffffffu, key);
-        const int leader = __ffs(grp) - 1;
-        int base = 0;
-        if (key >= 0 && lane == leader) base = atomicAdd(a.cursor + key, __popc(grp));
-        base = __shfl_sync(0xffffffffu, base, leader);
-        if (key >= 0) {
-            const int slot = base + __popc(grp & lt);
-            if (slot < a.eff[key]) a.lists[a.offsets[key] + slot] = entry;
-        }
-    }
+    fill_bins(a.lists, a.cursor, a.eff, a.offsets, entry, n, a.nb, bx0, bx1, by0, by1);
 }
 
 // ---------------------------------------------------------------------------

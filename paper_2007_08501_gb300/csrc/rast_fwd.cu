@@ -29,8 +29,32 @@ namespace mr {
 // ---------------------------------------------------------------------------
 // staging
 // ---------------------------------------------------------------------------
-// Build the record of face f; returns the mesh index or -1 when culled.
-__device__ int stage_face(const StageArgs &a, int64_t f, int n, FaceRec &R) {
+// A block's faces share most of their corners (256 faces of a mesh touch some
+// 150 vertices, 768 corners): each distinct vertex is projected once, in
+// double-float, found through a hash of its index in shared memory.  Bound by
+// instructions: 1.3M faces, 1,310,720 x 3 corners: MRSTAGE
+constexpr int kStageTable = 1024;  // > 3 x 256 corners
+struct StageTable {
+    int key[kStageTable];          // vertex, -1 free
+    float x[6][kStageTable];       // X, Y, Z as hi, lo
+    unsigned short list[3 * 256];  // occupied places
+    unsigned char bad[kStageTable];
+    int n;
+};
+
+__device__ __forceinline__ int stage_place(StageTable &t, int v) {
+    unsigned h = ((unsigned)v * 2654435761u) >> 22;
+    while (true) {
+        const int seen = atomicCAS(&t.key[h], -1, v);
+        if (seen == -1) t.list[atomicAdd(&t.n, 1)] = (unsigned short)h;
+        if (seen == -1 || seen == v) return (int)h;
+        h = (h + 1) & (kStageTable - 1);  // (at most 768 of 1,024 are taken)
+    }
+}
+
+// Build the record of face f; returns the mesh index or -1 when culled.  Every
+// thread of the block calls it; `block` is the image whose corners are shared.
+__device__ int stage_face(const StageArgs &a, StageTable &t, int64_t f, int n, int block, FaceRec &R) {
     const float kInf = __int_as_float(0x7f800000);
     R.a = make_float4(0.f, 0.f, 0.f, 0.f);
     R.b = make_float4(0.f, 0.f, 0.f, 0.f);
@@ -38,22 +62,59 @@ __device__ int stage_face(const StageArgs &a, int64_t f, int n, FaceRec &R) {
     R.d = make_float4(0.f, 1.f, 1.f, 1.f);
     R.e = make_float4(0.f, 0.f, 0.f, 0.f);
     R.h = make_float4(0.f, 0.f, 0.f, 0.f);
-    if (n < 0) return -1;
+    reinterpret_cast<int4 *>(t.key)[threadIdx.x] = make_int4(-1, -1, -1, -1);
+    if (threadIdx.x == 0) t.n = 0;
+    __syncthreads();
     unsigned bad = 0;
-    int64_t vi[3];
+    int64_t vi[3] = {0, 0, 0};
+    int at[3] = {0, 0, 0};
+    if (n >= 0) {
 #pragma unroll
-    for (int i = 0; i < 3; ++i) {
-        vi[i] = a.faces[3 * f + i];
-        if (vi[i] < 0 || vi[i] >= a.V) bad |= MESHRAST_ST_BAD_INDEX;
+        for (int i = 0; i < 3; ++i) {
+            vi[i] = a.faces[3 * f + i];
+            if (vi[i] < 0 || vi[i] >= a.V) bad |= MESHRAST_ST_BAD_INDEX;
+        }
+        if (!bad && n == block)
+            for (int i = 0; i < 3; ++i) at[i] = stage_place(t, (int)vi[i]);
     }
+    __syncthreads();
+    for (int j = threadIdx.x; j < t.n; j += 256) {
+        const int h = t.list[j];
+        const float *v = a.verts + 3 * (int64_t)t.key[h];
+        const float px = v[0], py = v[1], pz = v[2];
+        t.bad[h] = !(isfinite(px) && isfinite(py) && isfinite(pz));
+        df X, Y, Z;
+        project_corner(a.cams + 16 * block, px, py, pz, X, Y, Z);
+        t.x[0][h] = X.hi;
+        t.x[1][h] = X.lo;
+        t.x[2][h] = Y.hi;
+        t.x[3][h] = Y.lo;
+        t.x[4][h] = Z.hi;
+        t.x[5][h] = Z.lo;
+    }
+    __syncthreads();
+    if (n < 0) return -1;
     if (bad) { set_status(a.status, bad); return -1; }
     const float *cam = a.cams + 16 * n;
     df X[3], Y[3], Z[3];
 #pragma unroll
     for (int i = 0; i < 3; ++i) {
-        float px = a.verts[3 * vi[i]], py = a.verts[3 * vi[i] + 1], pz = a.verts[3 * vi[i] + 2];
-        if (!(isfinite(px) && isfinite(py) && isfinite(pz))) bad |= MESHRAST_ST_NONFINITE;
-        project_corner(cam, px, py, pz, X[i], Y[i], Z[i]);
+        df x, y, z;
+        if (n == block) {
+            const int h = at[i];
+            if (t.bad[h]) bad |= MESHRAST_ST_NONFINITE;
+            x = {t.x[0][h], t.x[1][h]};
+            y = {t.x[2][h], t.x[3][h]};
+            z = {t.x[4][h], t.x[5][h]};
+        } else {  // a block across two images
+            const float *v = a.verts + 3 * vi[i];
+            const float px = v[0], py = v[1], pz = v[2];
+            if (!(isfinite(px) && isfinite(py) && isfinite(pz))) bad |= MESHRAST_ST_NONFINITE;
+            project_corner(cam, px, py, pz, x, y, z);
+        }
+        X[i] = x;
+        Y[i] = y;
+        Z[i] = z;
     }
     if (bad) { set_status(a.status, bad); return -1; }
     const float znear = cam[13];
@@ -88,10 +149,12 @@ __device__ int stage_face(const StageArgs &a, int64_t f, int n, FaceRec &R) {
 
 __global__ void __launch_bounds__(256) k_stage(StageArgs a) {
     const int64_t f = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+    __shared__ __align__(16) StageTable s_table;
     FaceRec R;
-    int n = block_find_mesh(a.first_face, a.num_faces, a.N, a.F, f);
+    int block;
+    int n = block_find_mesh(a.first_face, a.num_faces, a.N, a.F, f, block);
+    n = stage_face(a, s_table, f, n, block, R);
     if (f < a.F) {
-        n = stage_face(a, f, n, R);
         float4 *dst = reinterpret_cast<float4 *>(a.rec + f);
         dst[kRecA] = R.a;
         dst[kRecB] = R.b;
@@ -102,19 +165,9 @@ __global__ void __launch_bounds__(256) k_stage(StageArgs a) {
         if (a.face_mesh) a.face_mesh[f] = n;
     }
     if (!a.do_count) return;
-    // warp-aggregated bin counting; every lane of the warp takes part
     int bx0 = 1, bx1 = 0, by0 = 1, by1 = 0;
     if (n >= 0) bin_rect(R, a.S, a.bin, bx0, bx1, by0, by1);
-    const int nbx = max(0, bx1 - bx0 + 1), nby = max(0, by1 - by0 + 1);
-    const int cnt = nbx * nby;
-    const int wmax = __reduce_max_sync(0xffffffffu, cnt);
-    const int lane = threadIdx.x & 31;
-    for (int i = 0; i < wmax; ++i) {
-        int key = -1;
-        if (i < cnt) key = (n * a.nb + by0 + i / nbx) * a.nb + bx0 + i % nbx;
-        unsigned grp = __match_any_sync(0xffffffffu, key);
-        if (key >= 0 && lane == __ffs(grp) - 1) atomicAdd(a.counts + key, __popc(grp));
-    }
+    count_bins(a.counts, n, a.nb, bx0, bx1, by0, by1);
 }
 
 // ---------------------------------------------------------------------------
@@ -271,24 +324,7 @@ __global__ void __launch_bounds__(256) k_fill(FillArgs a) {
     int bx0 = 1, bx1 = 0, by0 = 1, by1 = 0;
     if (n >= 0) bin_rect(R, a.S, a.bin, bx0, bx1, by0, by1);
     const unsigned long long entry = n >= 0 ? bin_entry(face_zmin(R), (int)f) : 0ull;
-    const int nbx = max(0, bx1 - bx0 + 1), nby = max(0, by1 - by0 + 1);
-    const int cnt = nbx * nby;
-    const int wmax = __reduce_max_sync(0xffffffffu, cnt);
-    const int lane = threadIdx.x & 31;
-    const unsigned lt = (1u << lane) - 1u;
-    for (int i = 0; i < wmax; ++i) {
-        int key = -1;
-        if (i < cnt) key = (n * a.nb + by0 + i / nbx) * a.nb + bx0 + i % nbx;
-        unsigned grp = __match_any_sync(0xffffffffu, key);
-        int leader = __ffs(grp) - 1;
-        int base = 0;
-        if (key >= 0 && lane == leader) base = atomicAdd(a.cursor + key, __popc(grp));
-        base = __shfl_sync(0xffffffffu, base, leader);
-        if (key >= 0) {
-            int slot = base + __popc(grp & lt);
-            if (slot < a.eff[key]) a.lists[a.offsets[key] + slot] = entry;
-        }
-    }
+    fill_bins(a.lists, a.cursor, a.eff, a.offsets, entry, n, a.nb, bx0, bx1, by0, by1);
 }
 
 // ---------------------------------------------------------------------------
