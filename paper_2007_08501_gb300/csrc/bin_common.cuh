@@ -16,17 +16,15 @@ __device__ __forceinline__ int find_mesh(const int64_t *first_face, int N, int64
     return ans;
 }
 
-// Image of element i of a packed batch (ranges first[n] .. first[n] + num[n]),
-// or -1.  Thread 0 looks up the block's first element once; threads whose
-// element lies in that image's range skip their own binary search.  Every
-// thread of the block must call it (it synchronises the block).
-// `block`: image of the block's first element, or -1.
-__device__ __forceinline__ int block_find_mesh(const int64_t *first, const int64_t *num, int N, int64_t count,
-                                               int64_t i, int &block) {
+// Image of a block's first element i0 of a packed batch (ranges first[n] ..
+// first[n] + num[n]) and that image's range; -1 and an empty range past the
+// end.  Thread 0 looks it up; every thread of the block must call it (it
+// synchronises the block).
+__device__ __forceinline__ void block_image(const int64_t *first, const int64_t *num, int N, int64_t count,
+                                            int64_t i0, int &block, int64_t &lo, int64_t &hi) {
     __shared__ int s_n;
     __shared__ long long s_lo, s_hi;
     if (threadIdx.x == 0) {
-        const int64_t i0 = (int64_t)blockIdx.x * blockDim.x;
         const int n0 = i0 < count ? find_mesh(first, N, i0) : -1;
         s_n = n0;
         s_lo = n0 >= 0 ? first[n0] : 0;
@@ -34,8 +32,14 @@ __device__ __forceinline__ int block_find_mesh(const int64_t *first, const int64
     }
     __syncthreads();
     block = s_n;
-    if (i >= count) return -1;
-    if (s_n >= 0 && i >= s_lo && i < s_hi) return s_n;
+    lo = s_lo;
+    hi = s_hi;
+}
+
+// Image of element i, or -1: the block's when i lies in its range, else by search.
+__device__ __forceinline__ int image_of(const int64_t *first, const int64_t *num, int N, int64_t i, int block,
+                                        int64_t lo, int64_t hi) {
+    if (block >= 0 && i >= lo && i < hi) return block;
     const int n = find_mesh(first, N, i);
     return (n >= 0 && i < first[n] + num[n]) ? n : -1;
 }
@@ -123,7 +127,8 @@ __device__ __forceinline__ void count_bins(int *counts, int n, int nb, int bx0, 
 
 // Appends `entry` to the lists of the element's bins (up to eff entries each
 // from offsets), four steps' cursor additions in flight at a time: one at a
-// time, each waited for its round trip to L2 (1.3M faces in 14M pairs: MRFILL).
+// time, each waited for its round trip to L2 (1.3M faces in 14M pairs: 107
+// -> 94 us).
 __device__ __forceinline__ void fill_bins(unsigned long long *lists, int *cursor, const int *eff, const int *offsets,
                                           unsigned long long entry, int n, int nb, int bx0, int bx1, int by0, int by1) {
     constexpr int U = 4;

@@ -420,10 +420,7 @@ static cudaError_t launch_sort_bins(const FineArgs &a, cudaStream_t st) {
     const size_t dyn = (size_t)a.sort_cap * 8;
     cudaError_t e = cudaFuncSetAttribute(k_sort_bins, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)dyn);
     if (e != cudaSuccess) return e;
-    int bps = 0;
-    e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&bps, k_sort_bins, 256, dyn);
-    if (e != cudaSuccess) return e;
-    const int grid = std::max(1, std::min<int>(a.items, mr_host::num_sms() * std::max(1, bps)));
+    const int grid = mr_host::queue_blocks(a.items, 8);
     k_sort_bins<<<grid, 256, dyn, st>>>(a);
     return cudaGetLastError();
 }
@@ -432,12 +429,8 @@ template <int BS, bool PACKED>
 static cudaError_t launch_fine_stream_t(const FineArgs &a, cudaStream_t st) {
     auto kern = k_fine_stream<BS, PACKED>;
     const size_t dyn = (size_t)2 * kStreamWarps * kRing * 32 * sizeof(float);  // 32 KB
-    int bps = 0;
-    cudaError_t e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&bps, kern, kStreamWarps * 32, dyn);
-    if (e != cudaSuccess) return e;
-    const long long warps = (long long)a.items * (BS * BS / 32);
-    const long long need = (warps + kStreamWarps - 1) / kStreamWarps;
-    const int grid = (int)std::max(1LL, std::min<long long>(need, (long long)mr_host::num_sms() * std::max(1, bps)));
+    const int64_t blocks = ((int64_t)a.items * (BS * BS / 32) + kStreamWarps - 1) / kStreamWarps;
+    const int grid = mr_host::queue_blocks(blocks, 4);
     kern<<<grid, kStreamWarps * 32, dyn, st>>>(a);
     return cudaGetLastError();
 }

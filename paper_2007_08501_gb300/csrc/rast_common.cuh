@@ -531,4 +531,11 @@ struct WsLayout {
 namespace mr_host {
 bool ws_layout(const rast_params *p, int64_t V, int64_t F, mr::WsLayout *L);
 int num_sms();
+// Blocks of a kernel whose blocks pull items from a queue: as many as can be
+// resident at most (the rest of the SM's limits may leave some waiting: they
+// find the queue empty and end), so that no launch asks for its occupancy.
+inline int queue_blocks(int64_t items, int per_sm) {
+    const int64_t most = (int64_t)num_sms() * per_sm;
+    return (int)(items < 1 ? 1 : items < most ? items : most);
+}
 }
