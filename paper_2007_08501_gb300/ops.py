@@ -200,12 +200,14 @@ def _ptr(t, dtype=None, name="tensor"):
         raise MeshRastError("%s must be %s, got %s" % (name, dtype, t.dtype))
     if not t.is_contiguous():
         raise MeshRastError("%s must be contiguous" % name)
-    return t.data_ptr() if t.numel() > 0 else None
+    return t.data_ptr() or None  # an empty tensor has no address
 
 
 def _stream(stream):
-    s = torch.cuda.current_stream() if stream is None else stream
-    return s.cuda_stream
+    if stream is None:
+        # the current stream's handle without building a torch.cuda.Stream around it
+        return torch._C._cuda_getCurrentRawStream(torch._C._cuda_getDevice())
+    return stream.cuda_stream
 
 
 # The C ABI trusts the sizes it derives from the parameters and the leading
@@ -245,27 +247,15 @@ def _image(t, N, S, C, name):
 
 def make_rast_params(N, image_size, K, blur_radius=0.0, bin_size=16, max_faces_per_bin=1024,
                      perspective_correct=True, clip_barycentric_coords=False, max_bin_entries=0):
-    p = rast_params()
-    p.N, p.image_size, p.faces_per_pixel = int(N), int(image_size), int(K)
-    p.bin_size, p.max_faces_per_bin = int(bin_size), int(max_faces_per_bin)
-    p.perspective_correct = int(bool(perspective_correct))
-    p.clip_barycentric_coords = int(bool(clip_barycentric_coords))
-    p.reserved = 0
-    p.blur_radius = float(blur_radius)
-    p.reserved_f = 0.0
-    p.max_bin_entries = int(max_bin_entries)
-    return p
+    return rast_params(int(N), int(image_size), int(K), int(bin_size), int(max_faces_per_bin),
+                       int(bool(perspective_correct)), int(bool(clip_barycentric_coords)), 0, float(blur_radius), 0.0,
+                       int(max_bin_entries))
 
 
 def make_blend_params(sigma=1e-4, gamma=1e-4, znear=0.1, zfar=100.0, bg=(1.0, 1.0, 1.0), eps=1e-10,
                       mode=BLEND_RGB):
-    b = blend_params()
-    b.sigma, b.gamma, b.znear, b.zfar = float(sigma), float(gamma), float(znear), float(zfar)
-    b.bg[0], b.bg[1], b.bg[2] = (float(x) for x in bg)
-    b.eps = float(eps)
-    b.mode = int(mode)
-    b.reserved = 0
-    return b
+    r, g, b = (float(x) for x in bg)
+    return blend_params(float(sigma), float(gamma), float(znear), float(zfar), (r, g, b), float(eps), int(mode), 0)
 
 
 # ---------------------------------------------------------------------------
