@@ -9,8 +9,8 @@
 //   k_scan      one block: clamp counts to capacity, exclusive scan -> offsets
 //   k_fill      one thread per face: warp-aggregated atomic append into lists
 //   k_fine      persistent blocks pull (image, bin) items from a global queue,
-//               stage each bin's face records in shared memory, keep a
-//               register-resident top-K per pixel, write the fragments
+//               walk each bin's faces front to back, keep a register-resident
+//               top-K per pixel, write the fragments
 // The plain form (bin_size 0) replaces scan/fill/fine by k_naive, every pixel
 // against every face of its image.
 #include <cuda_runtime.h>
@@ -487,8 +487,8 @@ template <int KM, int BS, int OUT>
 __global__ void __launch_bounds__(BS *BS, fine_blocks(KM) * 256 / (BS * BS)) k_fine(FineArgs a) {
     constexpr int BD = BS * BS;
     constexpr int WIN = fine_window(BS);
-    __shared__ float4 s_rec[BD][5];  // a, b, d, e, h of the staged records; boxes apart, lanes read them side by side
-    __shared__ float4 s_box[BD];
+    __shared__ float4 s_box[WIN];               // the window's bboxes: lanes read them side by side
+    __shared__ float4 s_rec[BD / 32][32][5];    // per warp: a, b, d, e, h of the faces it walks next
     __shared__ WindowShared<WIN> s_win;
     __shared__ int s_item;
     // K > 16: the per-thread lists
@@ -502,6 +502,7 @@ __global__ void __launch_bounds__(BS *BS, fine_blocks(KM) * 256 / (BS * BS)) k_f
     EvalFlags fl = a.fl;
     const bool zcull = fl.clip || !(fl.blur > 0.f);
     const int nb2 = a.nb * a.nb;
+    float4 (*const rec)[5] = s_rec[tid >> 5];
     while (true) {
         if (tid == 0) s_item = (int)atomicAdd(a.queue, 1u);
         __syncthreads();
@@ -553,72 +554,71 @@ __global__ void __launch_bounds__(BS *BS, fine_blocks(KM) * 256 / (BS * BS)) k_f
         };
         // The bin's faces in front-to-back windows (two warps' worth is not
         // worth ordering; without depth culling the order buys nothing).
-        // Chunks of BD faces are staged; faces are culled 32 at a time for the
-        // whole warp: lane j tests face jb + j against the rectangle spanned
-        // by the warp's pixel centres and against the warp's largest K-th
-        // depth; one ballot names the faces the warp walks pixel by pixel.  A
-        // face is skipped by a lane when its bbox misses the pixel or its
-        // nearest corner lies behind the lane's K-th depth.  Once a warp's
-        // largest K-th depth falls into a bucket in front of the next face's,
-        // the rest of the window is behind all its lanes, and the block stops
-        // when everything left is behind every warp.
+        // Within a window the warps go their own way.  Faces are culled 32 at
+        // a time for the whole warp: lane j tests face jb + j against the
+        // rectangle spanned by the warp's pixel centres and against the warp's
+        // largest K-th depth; one ballot names the faces the warp walks pixel
+        // by pixel, and their lanes bring the records to the warp's own part
+        // of shared memory.  A face is skipped
+        // by a lane when its bbox misses the pixel or its nearest corner lies
+        // behind the lane's K-th depth.  Once a warp's largest K-th depth
+        // falls into a bucket in front of the next face's, the rest of the
+        // window is behind all its lanes, and the block stops when everything
+        // left is behind every warp.  (Staging the records for the block, 256
+        // at a time, made all warps wait for the slowest at every 256: 700
+        // against 633 us at 1.3M faces, 1024 px, K = 8, 225 against 176 for 5
+        // meshes at 225 px; reading them from L1 one by one, 297 against 246
+        // where few faces reach a warp: 1.3M faces, K = 1, no blur.)
         window_begin<BD>(s_win, a.lists + off, cnt, zcull && cnt > 64);
         while (const int m = window_next<BD>(s_win)) {
-            for (int base = 0; base < m; base += BD) {
-                const int mc = min(BD, m - base);
-                if (tid < mc) {
-                    const int fid = (int)(unsigned)(s_win.ent[base + tid] & 0xffffffffull);
-                    const float4 *src = reinterpret_cast<const float4 *>(a.rec + fid);
-                    s_rec[tid][0] = __ldg(src + kRecA);
-                    s_rec[tid][1] = __ldg(src + kRecB);
-                    s_rec[tid][2] = __ldg(src + kRecD);
-                    s_rec[tid][3] = __ldg(src + kRecE);
-                    s_rec[tid][4] = __ldg(src + kRecH);
-                    s_box[tid] = __ldg(src + kRecC);
+            for (int i = tid; i < m; i += BD)
+                s_box[i] = __ldg(reinterpret_cast<const float4 *>(a.rec + (unsigned)s_win.ent[i]) + kRecC);
+            __syncthreads();
+            for (int jb = 0; jb < m; jb += 32) {
+                const float wthr = warp_kth();
+                if (zcull && s_win.rank(wthr) < s_win.rank(entry_key(s_win.ent[jb]))) break;
+                const int jl = jb + lane;
+                bool hit = false;
+                if (jl < m) {
+                    const float4 bb = s_box[jl];
+                    const unsigned long long e = s_win.ent[jl];
+                    hit = bb.x <= wx1 && bb.y >= wx0 && bb.z <= wy1 && bb.w >= wy0 && !(zcull && entry_key(e) > wthr);
+                    if (hit) {
+                        const float4 *src = reinterpret_cast<const float4 *>(a.rec + (unsigned)e);
+                        rec[lane][0] = __ldg(src + kRecA);
+                        rec[lane][1] = __ldg(src + kRecB);
+                        rec[lane][2] = __ldg(src + kRecD);
+                        rec[lane][3] = __ldg(src + kRecE);
+                        rec[lane][4] = __ldg(src + kRecH);
+                    }
                 }
-                __syncthreads();
-                bool warp_done = false;
-                for (int jb = 0; jb < mc; jb += 32) {
-                    const float wthr = warp_kth();
-                    if (zcull && s_win.rank(wthr) < s_win.rank(entry_key(s_win.ent[base + jb]))) {
-                        warp_done = true;
-                        break;
-                    }
-                    const int jl = jb + lane;
-                    bool hit = false;
-                    if (jl < mc) {
-                        const float4 bb = s_box[jl];
-                        hit = bb.x <= wx1 && bb.y >= wx0 && bb.z <= wy1 && bb.w >= wy0 &&
-                              !(zcull && entry_key(s_win.ent[base + jl]) > wthr);
-                    }
-                    unsigned mask = __ballot_sync(0xffffffffu, hit);
-                    while (mask) {
-                        const int jj = jb + __ffs(mask) - 1;
-                        mask &= mask - 1;
-                        if (!valid) continue;
-                        FaceRec R;
-                        R.c = s_box[jj];
-                        if (!in_bbox(R, p)) continue;
-                        const unsigned long long e = s_win.ent[base + jj];
-                        if (zcull && entry_key(e) > kth()) continue;
-                        R.a = s_rec[jj][0];
-                        R.b = s_rec[jj][1];
-                        R.d = s_rec[jj][2];
-                        R.e = s_rec[jj][3];
-                        R.h = s_rec[jj][4];
-                        float z;
-                        if (face_key_nobbox(R, p, fl, z)) {
-                            const int fid = (int)(unsigned)(e & 0xffffffffull);
-                            if constexpr (KM > 0) {
-                                if (tk.admits(z, fid)) tk.insert(z, fid);
-                            } else {
-                                if (stk.admits(z, fid)) stk.insert(z, fid);
-                            }
+                unsigned mask = __ballot_sync(0xffffffffu, hit);
+                __syncwarp();
+                while (mask) {
+                    const int j = __ffs(mask) - 1, jj = jb + j;
+                    mask &= mask - 1;
+                    if (!valid) continue;
+                    FaceRec R;
+                    R.c = s_box[jj];
+                    if (!in_bbox(R, p)) continue;
+                    const unsigned long long e = s_win.ent[jj];
+                    if (zcull && entry_key(e) > kth()) continue;
+                    const int fid = (int)(unsigned)e;
+                    R.a = rec[j][0];
+                    R.b = rec[j][1];
+                    R.d = rec[j][2];
+                    R.e = rec[j][3];
+                    R.h = rec[j][4];
+                    float z;
+                    if (face_key_nobbox(R, p, fl, z)) {
+                        if constexpr (KM > 0) {
+                            if (tk.admits(z, fid)) tk.insert(z, fid);
+                        } else {
+                            if (stk.admits(z, fid)) stk.insert(z, fid);
                         }
                     }
                 }
-                // a warp past the window's last useful face is done with the window
-                if (__syncthreads_and(warp_done)) break;
+                __syncwarp();
             }
             if (__syncthreads_and(zcull && s_win.rest_behind(warp_kth()))) break;
         }
@@ -633,7 +633,7 @@ __global__ void __launch_bounds__(BS *BS, fine_blocks(KM) * 256 / (BS * BS)) k_f
             // K > 16: the block writes its tile slot by slot: consecutive
             // threads take consecutive output slots of a tile row (coalesced),
             // each recomputing its slot's barycentrics and distance
-            __shared__ int s_held[BD];
+            int *const s_held = reinterpret_cast<int *>(s_win.ent);  // (the window is done)
             s_held[tid] = valid ? stk.n : 0;
             __syncthreads();
             const int K = a.K;
