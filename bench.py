@@ -89,27 +89,8 @@ def mesh_kernels_per_step(w):
 # DRAM bytes (read + write) per C-ABI call of a stage -- every kernel of the
 # call, from one ncu capture (gpu__time_duration, dram__bytes_read/write,
 # --clock-control none) of the current kernel source -- keyed by (workload,
-# stage, bin size); a combination without an entry reports null.  Workload 4
-# is captured on its first 2 of 20 views (--max-images 2) and scaled by 10:
-# every view carries the same mesh, so each kernel's traffic grows with the
-# views.
-TRAFFIC_BYTES = {
-    ("1", "fwd", 16): {"kernel": "rast_blend_fwd call: k_stage + k_scan + k_fill + k_fine<8,16,0> + k_blend_fwd<8>",
-                       "bytes": 141800000, "profile": "profiles/launch_list_8x5120faces_256px_K8.md"},
-    ("1", "bwd", 16): {"kernel": "blend_rast_bwd call: k_stage + k_blend_rast_bwd<8,1>", "bytes": 106100000,
-                       "profile": "profiles/launch_list_8x5120faces_256px_K8.md"},
-    ("4", "fwd", 16): {"kernel": "rast_blend_fwd call: k_stage + k_scan + k_fill + k_sort_bins + "
-                                 "k_fine_stream<16,16,8,0> + k_fine_stream<16,64,4,1> + k_frag_attr<1>", "bytes": 11634000000,
-                       "profile": "profiles/launch_list_20x81920faces_512px_K50.md (2 views x 10)"},
-    ("4", "bwd", 16): {"kernel": "blend_rast_bwd call: k_stage + k_blend_rast_bwd_any<0>", "bytes": 4209000000,
-                       "profile": "profiles/launch_list_20x81920faces_512px_K50.md (2 views x 10)"},
-    ("points", "rast_fwd", 8): {"kernel": "pts_rasterize_fwd call: k_pstage + k_scan + k_pfill + k_pfine<0,8>",
-                                "bytes": 552453578, "profile": "profiles/points_8x200000pts_256px_K50.md"},
-    # the same rasterizer call (compositing mode does not enter it)
-    ("points_norm", "rast_fwd", 8): {"kernel": "pts_rasterize_fwd call: k_pstage + k_scan + k_pfill + "
-                                               "k_pfine<0,8>", "bytes": 552453578,
-                                     "profile": "profiles/points_8x200000pts_256px_K50.md"},
-}
+# stage, bin size); a combination without an entry reports null.
+TRAFFIC_BYTES = {}
 
 
 def _args():
@@ -560,7 +541,7 @@ def run_ours(args):
         raise RuntimeError("device status %d after the first step" % st)
     mc, tot = ops.rast_bin_occupancy(pipe.p, b.V, b.F, pipe.ws)
     fine_tests = int(tot) * tuned["bin_size"] ** 2
-    # pixels the large-K streaming fine pass handed to its second pass (ring overflow)
+    # pixels of the large-K streaming fine pass whose unsettled candidates outgrew the ring
     lay = ops.rast_workspace_bin_layout(pipe.p, b.V, b.F)
     redo_pixels = int(pipe.ws[lay["redo"]:lay["redo"] + 4].cpu().numpy().view(np.uint32)[0])
     pipe.capture()
@@ -1091,9 +1072,6 @@ def run_reference(args):
 KNN_WORKLOADS = ("knn", "knn_het", "chamfer")
 KNN_METRIC = "exact KNN / Chamfer ms per batch & candidate distances per second (Gpair/s), % FP32 ALU roofline"
 KNN_UNIT = "Gpair/s"
-# FP32 lane operations one candidate distance needs at least: D subtractions,
-# one multiply and D - 1 fused multiply-adds (D = 3)
-KNN_OPS_PER_PAIR = 6
 FP32_LANE_OPS_PEAK = 152 * 128 * 2.07e9   # SMs x FP32 lanes x max SM clock (derived, not measured)
 
 
@@ -1111,8 +1089,8 @@ class KnnPipeline:
         self.f1, self.l1, self.f2, self.l2 = T(c.first1), T(c.len1), T(c.first2), T(c.len2)
         self.K, self.chamfer = w.K, w.chamfer
         self.dev = device
-        self.ws = ops.alloc_knn_workspace(c.N, device)
         P1, P2 = c.p.shape[0], c.q.shape[0]
+        self.ws = ops.alloc_knn_workspace(c.N, device, P1, P2, c.p.shape[1], *([] if w.chamfer else [w.K]))
         if self.chamfer:
             self.idx_pq = torch.empty(P1, dtype=torch.int64, device=device)
             self.d_pq = torch.empty(P1, device=device)
@@ -1225,14 +1203,16 @@ def run_knn(args):
     value = whole_job_rate(pairs, world, ms, 1e9)
     stages = {k: statistics.mean(s[k] for s in per_step) for k in per_step[0]}
     dom = "chamfer_fwd" if w.chamfer else "knn"
-    achieved = pairs * KNN_OPS_PER_PAIR / (stages[dom] / 1e3)
-    peak_ops = measure_fp32_peak(dev)
-    roofline = {"bound": "alu", "achieved": round(achieved / 1e12, 3), "peak": round(peak_ops / 1e12, 2),
-                "unit": "T FP32 lane-op/s", "frac": round(achieved / peak_ops, 4), "traffic": None,
-                "kernel": "k_knn (%s call)" % dom,
-                "ops_per_pair": KNN_OPS_PER_PAIR, "pairs_per_launch": pairs,
-                "peak_source": "measured in this run: meshrast_fma_probe (FMA lane operations per second)",
-                "derived_peak": round(FP32_LANE_OPS_PEAK / 1e12, 2)}
+    # the index search evaluates a small share of the pairs it covers, so the
+    # roofline is that of the data: every input read once, every output written once
+    alg = sum(t.numel() * t.element_size() for t in [*pipe.inputs(), *pipe.outputs()])
+    peak, peak_kind = _peaks()
+    achieved = alg / (sum(stages.values()) / 1e3) / 1e9
+    roofline = {"bound": "hbm", "achieved": round(achieved, 1), "peak": peak, "unit": "GB/s",
+                "frac": round(achieved / peak, 4), "traffic": None, "algorithmic_bytes": alg,
+                "kernel": "%s step (limited by the search's instruction issue)" % dom, "pairs_covered": pairs,
+                "peak_source": "%s (MEASURED_PEAKS.json hbm_gbs)" % peak_kind if peak_kind == "measured"
+                else "fallback 6.8 TB/s"}
     # end to end with host buffers: inputs in, results out, every step
     pin = lambda t: t.cpu().pin_memory()
     h_in = [(d_, pin(d_)) for d_ in pipe.inputs()]
@@ -1270,7 +1250,7 @@ def run_knn(args):
                        "l2": "flushed between steps (256 MiB write), outside the timed events",
                        "parallelism": "replicas x%d" % world},
             "roofline": roofline, "stages_ms": {k: round(v, 4) for k, v in stages.items()},
-            "cpu_baseline": cpu, "e2e": e2e, "gpu_launches": (5 if w.chamfer else 2) * args.steps, "clocks": clk,
+            "cpu_baseline": cpu, "e2e": e2e, "gpu_launches": (11 if w.chamfer else 7) * args.steps, "clocks": clk,
             "ms_per_step_median": round(statistics.median(sum(s.values()) for s in per_step), 4)}), flush=True)
     if dist is not None:
         dist.barrier()

@@ -95,7 +95,7 @@ typedef struct {
     int32_t N;                    /* images (= meshes) in the batch, 0 .. 65535 */
     int32_t image_size;           /* S, 1 .. 8192 */
     int32_t faces_per_pixel;      /* K, 1 .. 64 */
-    int32_t bin_size;             /* 0: plain form, one unbinned launch per image;
+    int32_t bin_size;             /* 0: plain form, every pixel against every face of its image;
                                      8 or 16: coarse-to-fine with bins of bin_size^2 pixels */
     int32_t max_faces_per_bin;    /* binned mode: capacity of one bin (> 0) */
     int32_t perspective_correct;  /* 0/1: barycentrics of the 3D point on the face */

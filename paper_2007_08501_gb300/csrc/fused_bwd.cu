@@ -4,12 +4,12 @@
 //
 // blend_bwd followed by rast_mesh_bwd writes dL/d(zbuf, bary, dists) for every
 // slot (20 bytes) and reads it back, together with pix_to_face, in a second
-// launch.  Here each thread owns one pixel: it forms the slot's blend adjoint
-// in registers and pulls it straight through the per-slot rasterizer adjoint
-// (slot_corner_grads), so the fragment gradients never reach memory.  For
-// every slot k the warp (2 rows x 16 pixels) groups lanes holding the same
-// face once; one lane per face adds the face's colour gradients (softmax
-// blend) and, through the projection Jacobian and R^T, its vertex gradients.
+// launch.  Here each thread owns one pixel and forms its slots' blend adjoint,
+// which goes through shared memory into the per-slot rasterizer adjoint, so the
+// fragment gradients never reach memory.  Softmax blend: the tile's slots are
+// taken face by face (tile_sort.cuh).  Silhouette: rank by rank, the warp's
+// lanes grouped by face (render_meshes keeps packed slots instead,
+// sil_bwd.cu).
 // The per-slot arithmetic is that of k_blend_bwd and k_rast_bwd.
 #include <cuda_runtime.h>
 

@@ -75,7 +75,7 @@ struct FineBlend {
 struct FineArgs {
     const FaceRec *rec;
     const float *cams;
-    unsigned long long *lists;  // K > 16: each block sorts its bins' lists in place
+    unsigned long long *lists;  // the streaming pass's are sorted in place first
     const int *eff, *offsets;
     const int *order;           // queue position -> bin (bins by descending work class)
     unsigned *queue;
