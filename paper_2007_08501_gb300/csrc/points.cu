@@ -293,8 +293,11 @@ __device__ __forceinline__ void pt_write(const PtArgs &a, int64_t pix, const Top
 // point covers 5 of a warp's 32 pixels.  8 clouds of 200,000 points, 256 px, K =
 // 50, bins of 8: 874 -> 275 us; 3 clouds of 9,000 at 100 px, K = 10, bins of 16:
 // 165 -> 36 us.
-constexpr int pfine_threads(int BS) { return BS == 16 ? 256 : 128; }
-constexpr int pfine_window(int BS) { return BS == 16 ? 512 : 1024; }
+// 256 threads also for the 64 pixels of a bin of 8: the ordering and the tile's
+// slots take them all, and 512 entries a window keep 5 blocks on an SM (8 x
+// 200,000 points, forward and backward: 128 threads and 1,024 entries 645 us, 256
+// and 1,024 584, 256 and 512 574, 64 and 512 736)
+constexpr int kPfineThreads = 256, kPfineWindow = 512;
 constexpr int kPtCount = 64;  // a bucket beyond this has its window sorted instead
 
 // Composites a pixel's points, ids and 1 - alpha in shared memory (the
@@ -323,8 +326,8 @@ __device__ __forceinline__ void pt_composite(const PtArgs &a, const int *ids, co
 // RENDER: the tile's pixels are composited and their points left as packed
 // slots, 8 bytes for each there is, in place of 16 for every slot.
 template <int BS, bool RENDER>
-__global__ void __launch_bounds__(pfine_threads(BS)) k_pfine(PtArgs a) {
-    constexpr int BD = pfine_threads(BS), WIN = pfine_window(BS), PX = BS * BS;
+__global__ void __launch_bounds__(kPfineThreads) k_pfine(PtArgs a) {
+    constexpr int BD = kPfineThreads, WIN = kPfineWindow, PX = BS * BS;
     __shared__ WindowShared<WIN> s_win;
     __shared__ int s_ids[WIN];             // the window's points, in order
     __shared__ unsigned s_bits[WIN / 32][PX];
@@ -1045,7 +1048,7 @@ static cudaError_t launch_pfill(const PtArgs &a, cudaStream_t st) {
 
 template <int BS, bool RENDER>
 static cudaError_t launch_pfine_t(const PtArgs &a, cudaStream_t st) {
-    constexpr int BD = pfine_threads(BS);
+    constexpr int BD = kPfineThreads;
     const size_t dyn = (size_t)BS * BS * (a.K | 1) * (RENDER ? 2 : 1) * sizeof(int);  // ids, and 1 - alpha
     auto kern = k_pfine<BS, RENDER>;
     if (dyn > 16 * 1024) {  // static + dynamic above 48 KB needs the opt-in
