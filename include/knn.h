@@ -19,7 +19,9 @@
  *   p2 (P2, D), first2 (N,), len2 (N,)   candidate clouds, same form
  * Query cloud i only sees candidate cloud i.  In each batch, first is
  * non-decreasing and the ranges are disjoint and inside the array;
- * len2[i] < 2^31.  Coordinates must be finite.
+ * len2[i] < 2^31.  Coordinates must be finite.  knn_points also answers clouds
+ * in any order and candidate ranges that overlap (one cloud shared by many
+ * query clouds), by scanning whatever the workspace.
  *
  * Distance and ranking: the squared Euclidean distance evaluated in fp32 as
  * s = dx_0 * dx_0, then s = fma(dx_c, dx_c, s) for c = 1 .. D-1 with

@@ -391,7 +391,9 @@ class _KnnPoints(torch.autograd.Function):
 def knn_points(p1, first1, len1, p2, first2, len2, K):
     """(dists (P1, K), idx (P1, K)): the K nearest rows of p2 (same cloud) to
     each row of p1, ascending squared distance; idx is -1 (dist +inf) past
-    the end of a small cloud.  Differentiable in p1 and p2 through dists."""
+    the end of a small cloud.  Differentiable in p1 and p2 through dists.
+    Clouds in ascending, disjoint ranges are the fast case; other orders, and
+    one candidate cloud shared by several query clouds, are answered too."""
     return _KnnPoints.apply(p1.contiguous(), p2.contiguous(), first1.contiguous(), len1.contiguous(),
                             first2.contiguous(), len2.contiguous(), int(K))
 

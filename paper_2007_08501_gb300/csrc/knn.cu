@@ -33,6 +33,7 @@
 
 #include "knn.h"
 #include "knn_index.h"
+#include "knn_plan.cuh"
 #include "meshrast.h"
 #include "rast_common.cuh"
 
@@ -63,44 +64,7 @@ struct KnnArgs {
 // ---------------------------------------------------------------------------
 __global__ void __launch_bounds__(1024) k_knn_plan(KnnArgs a) {
     const KnnProblem &P = a.pr[blockIdx.x];
-    __shared__ long long s_warp[32];
-    __shared__ long long s_carry;
-    if (threadIdx.x == 0) s_carry = 0;
-    __syncthreads();
-    const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
-    for (int base = 0; base < P.N; base += 1024) {
-        const int i = base + threadIdx.x;
-        long long v = 0;
-        if (i < P.N) {
-            const long long n = P.len1[i];
-            v = n > 0 ? (n + P.qpb - 1) / P.qpb : 0;
-        }
-        long long x = v;   // inclusive scan within the warp
-#pragma unroll
-        for (int o = 1; o < 32; o <<= 1) {
-            const long long y = __shfl_up_sync(0xffffffffu, x, o);
-            if (lane >= o) x += y;
-        }
-        if (lane == 31) s_warp[w] = x;
-        __syncthreads();
-        if (w == 0) {
-            long long t = s_warp[lane];
-#pragma unroll
-            for (int o = 1; o < 32; o <<= 1) {
-                const long long y = __shfl_up_sync(0xffffffffu, t, o);
-                if (lane >= o) t += y;
-            }
-            s_warp[lane] = t;   // inclusive over warps
-        }
-        __syncthreads();
-        const long long carry = s_carry;
-        const long long before = carry + (w > 0 ? s_warp[w - 1] : 0) + x - v;
-        if (i < P.N) P.tiles[i] = before;
-        __syncthreads();
-        if (threadIdx.x == 0) s_carry = carry + s_warp[31];
-        __syncthreads();
-    }
-    if (threadIdx.x == 0) P.tiles[P.N] = s_carry;
+    plan_tiles<1024>(P.len1, P.N, P.qpb, P.tiles);
 }
 
 // ---------------------------------------------------------------------------
@@ -792,7 +756,8 @@ MESHRAST_API int knn_points(const float *p1, int64_t P1, const int64_t *first1, 
     cudaStream_t st = reinterpret_cast<cudaStream_t>(stream);
     if (use_index(N, P1, P2, D, K, workspace_bytes)) {
         NnSide side[2];
-        if (nn_index_build(side, p1, P1, first1, len1, p2, P2, first2, len2, N, D, false,
+        if (nn_index_build(side, p1, P1, first1, len1, p2, P2, first2, len2, N, D, K, false,
+                           reinterpret_cast<long long *>(workspace),
                            reinterpret_cast<char *>(workspace) + ws_bytes(N), st) != cudaSuccess)
             return MESHRAST_ERR_CUDA;
         return nn_index_search(side[0], side[1], D, K, idx, dists, st) == cudaSuccess ? MESHRAST_OK : MESHRAST_ERR_CUDA;
@@ -849,7 +814,8 @@ MESHRAST_API int chamfer_fwd(const float *p, int64_t P1, const int64_t *first1, 
     }
     if (use_index(N, P1, P2, D, 1, workspace_bytes)) {
         NnSide side[2];
-        if (nn_index_build(side, p, P1, first1, len1, q, P2, first2, len2, N, D, true,
+        if (nn_index_build(side, p, P1, first1, len1, q, P2, first2, len2, N, D, 1, true,
+                           reinterpret_cast<long long *>(workspace),
                            reinterpret_cast<char *>(workspace) + ws_bytes(N), st) != cudaSuccess ||
             nn_index_search(side[0], side[1], D, 1, idx_pq, d_pq, st) != cudaSuccess ||
             nn_index_search(side[1], side[0], D, 1, idx_qp, d_qp, st) != cudaSuccess)

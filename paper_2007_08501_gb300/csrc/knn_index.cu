@@ -16,7 +16,16 @@
 // lists rank by (distance, row), so the visiting order does not matter and
 // the results are those of the scan.
 //
-//   k_nn_bounds   bounds of every cloud
+// The clouds' ranges decide where everything lies, and only the device knows
+// them: the first kernel checks that they are ascending and disjoint.  If they
+// are not, the building kernels leave everything alone and the search kernels
+// scan all candidates in place (a launch of knn.cu's scan behind every search,
+// to do nothing, cost 32 pairs of 1,000 and 50,000 points 14 of 384 us).  8
+// clouds of 30,000 points against one of 30,000: K = 1 2,299 us, K = 8 2,799; the
+// scan of knn.cu 1,810 and 3,729.
+//
+//   k_nn_bounds   bounds of every cloud; one more block per batch checks its
+//                 ranges and plans the tiles of such a scan
 //   k_nn_count    cell of every point and its rank there (warp-aggregated)
 //   k_nn_tiles    sums of kNnTile cells (clouds of more cells than that)
 //   k_nn_starts   exclusive scan of a cloud's cells
@@ -34,6 +43,7 @@
 #include <cstdint>
 
 #include "knn_index.h"
+#include "knn_plan.cuh"
 #include "rast_common.cuh"
 
 namespace mr {
@@ -53,8 +63,11 @@ __device__ __forceinline__ float dec(unsigned e) {
 }
 
 // Cloud and tile of block b when cloud i's tiles of 2^shift rows start at
-// (first[i] >> shift) + i.  False when the block has no rows.
+// (first[i] >> shift) + i.  False when the block has no rows, or the ranges are
+// unfit (the word is asked for first and looked at last: waiting for it on
+// entry cost each kernel 0.7 us).
 __device__ __forceinline__ bool tile_of(const NnSide &s, long long b, int shift, int &cloud, long long &row0, int &n) {
+    const int unfit = s.control->unfit;
     int lo = 0, hi = s.N;   // last i with start <= b
     while (hi - lo > 1) {
         const int mid = (lo + hi) >> 1;
@@ -64,7 +77,20 @@ __device__ __forceinline__ bool tile_of(const NnSide &s, long long b, int shift,
     cloud = lo;
     row0 = t << shift;
     n = (int)s.len[lo];
-    return t >= 0 && row0 < n;
+    return t >= 0 && row0 < n && !unfit;
+}
+
+// The same for a search kernel: with unfit ranges the tile of the scan's plan.
+__device__ __forceinline__ bool query_tile(const NnSide &s, long long b, int shift, int &cloud, long long &row0, int &n,
+                                           bool &scan) {
+    scan = false;
+    if (tile_of(s, b, shift, cloud, row0, n)) return true;
+    if (!s.control->unfit || b >= s.plan[s.N]) return false;
+    scan = true;
+    cloud = planned_cloud(s.plan, s.N, b);
+    row0 = (b - s.plan[cloud]) << shift;
+    n = (int)s.len[cloud];
+    return true;
 }
 
 template <int D>
@@ -77,10 +103,20 @@ __device__ __forceinline__ void load_point(const float *x, long long row, float 
 // building
 // ---------------------------------------------------------------------------
 // box[cloud]: enc(high) in 0..3, enc(-low) in 4..7, both by atomicMax from 0.
-// A block takes 4,096 rows, so that few atomics meet at a cloud's words.
+// A block takes 4,096 rows, so that few atomics meet at a cloud's words.  (It
+// runs beside the check of the ranges; unfit ones have it read rows of their own
+// clouds and write their clouds' words, nothing else.)
 template <int D>
 __global__ void __launch_bounds__(256) k_nn_bounds(NnSide a, NnSide b) {
     const NnSide &s = blockIdx.y ? b : a;
+    if (blockIdx.x == gridDim.x - 1) {
+        for (int i = threadIdx.x; i < s.N; i += 256) {
+            const long long f = s.first[i], n = s.len[i], next = i + 1 < s.N ? s.first[i + 1] : s.P;
+            if (f < 0 || n < 0 || n > s.P || f > next - n) s.control->unfit = 1;
+        }
+        if (s.plan) plan_tiles<256>(s.len, s.N, s.per, s.plan);
+        return;
+    }
     __shared__ unsigned s_m[2 * D];
     int cloud, n;
     long long row0;
@@ -402,6 +438,29 @@ struct Nearest {
 };
 
 constexpr int kLaneThreads = 128;
+constexpr int kLaneShift = 7, kWarpShift = 2;   // queries per block, as powers of two
+
+// Sorted candidate at global place `at` and its row.
+template <int D>
+__device__ __forceinline__ int load_leaf(const NnSide &s, long long at, float (&v)[D]) {
+    const float4 p = __ldg(s.pts + at);
+    const float x[4] = {p.x, p.y, p.z, p.w};
+#pragma unroll
+    for (int c = 0; c < D; ++c) v[c] = x[c];
+    return D < 4 ? __float_as_int(p.w) : s.row[at];
+}
+
+// Candidate of row `at`, for the scan; past the end one that is never inserted
+// (distance +inf or NaN).
+template <int D>
+__device__ __forceinline__ void load_row(const NnSide &s, long long first, int cn, int at, float (&v)[D]) {
+    if (at < cn) {
+        load_point<D>(s.x, first + at, v);
+    } else {
+#pragma unroll
+        for (int c = 0; c < D; ++c) v[c] = INFINITY;
+    }
+}
 
 // A query per lane.  The warp's 32 queries are neighbours on the curve; it
 // walks nodes and leaves in order of their distance to the queries' common
@@ -415,7 +474,8 @@ __global__ void __launch_bounds__(kLaneThreads, KM <= 8 ? 8 : 4) k_nn_lanes(NnQu
     __shared__ __align__(16) float s_c[kLaneThreads / 32][D + 1][32];
     int cloud, n;
     long long row0;
-    if (!tile_of(a.q, blockIdx.x, 7, cloud, row0, n)) return;
+    bool scan;
+    if (!query_tile(a.q, blockIdx.x, kLaneShift, cloud, row0, n, scan)) return;
     const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
     const long long pos = row0 + threadIdx.x;
     if (row0 + (w << 5) >= n) return;   // uniform for the warp; no block barrier below
@@ -425,12 +485,17 @@ __global__ void __launch_bounds__(kLaneThreads, KM <= 8 ? 8 : 4) k_nn_lanes(NnQu
     float q[D];
     int qrow = 0;
     {
-        const long long at = qfirst + (valid ? pos : n - 1);
-        const float4 p = __ldg(a.q.pts + at);
-        const float v[4] = {p.x, p.y, p.z, p.w};
+        const long long r = valid ? pos : n - 1, at = qfirst + r;
+        if (scan) {
+            load_point<D>(a.q.x, at, q);
+            qrow = (int)r;
+        } else {
+            const float4 p = __ldg(a.q.pts + at);
+            const float v[4] = {p.x, p.y, p.z, p.w};
 #pragma unroll
-        for (int c = 0; c < D; ++c) q[c] = v[c];
-        qrow = D < 4 ? __float_as_int(p.w) : a.q.row[at];
+            for (int c = 0; c < D; ++c) q[c] = v[c];
+            qrow = D < 4 ? __float_as_int(p.w) : a.q.row[at];
+        }
     }
     float glo[D], ghi[D];
 #pragma unroll
@@ -444,20 +509,12 @@ __global__ void __launch_bounds__(kLaneThreads, KM <= 8 ? 8 : 4) k_nn_lanes(NnQu
     const float4 *leafbox = a.c.leaf + 2 * ((cfirst >> 5) + cloud);
     const float4 *nodebox = a.c.node + 2 * ((cfirst >> 10) + cloud);
     auto thr = [&]() { return valid ? L.z[KM - 1] : -1.f; };
-    auto visit = [&](int leaf) {
-        const int at = leaf * kLeaf + lane;
-        __syncwarp();   // the previous leaf's candidates are done with
-        if (at < cn) {
-            const float4 p = __ldg(a.c.pts + cfirst + at);
-            const float v[4] = {p.x, p.y, p.z, p.w};
+    // the lane's own candidate of 32, offered to every lane's query
+    auto offer = [&](const float (&v)[D], int row) {
+        __syncwarp();   // the previous candidates are done with
 #pragma unroll
-            for (int c = 0; c < D; ++c) s_c[w][c][lane] = v[c];
-            s_c[w][D][lane] = D < 4 ? p.w : __int_as_float(a.c.row[cfirst + at]);
-        } else {
-#pragma unroll
-            for (int c = 0; c < D; ++c) s_c[w][c][lane] = INFINITY;   // distance +inf or NaN: never inserted
-            s_c[w][D][lane] = 0.f;
-        }
+        for (int c = 0; c < D; ++c) s_c[w][c][lane] = v[c];
+        s_c[w][D][lane] = __int_as_float(row);
         __syncwarp();
         if constexpr (KM == 1) {   // a running minimum, no mask
 #pragma unroll
@@ -495,8 +552,20 @@ __global__ void __launch_bounds__(kLaneThreads, KM <= 8 ? 8 : 4) k_nn_lanes(NnQu
             }
         }
     };
+    auto visit = [&](int leaf) {
+        const int at = leaf * kLeaf + lane;
+        float v[D];
+        int row = 0;
+        if (at < cn) {
+            row = load_leaf<D>(a.c, cfirst + at, v);
+        } else {
+#pragma unroll
+            for (int c = 0; c < D; ++c) v[c] = INFINITY;   // distance +inf or NaN: never inserted
+        }
+        offer(v, row);
+    };
     int seed = -1;
-    if (cn > 0) {
+    if (cn > 0 && !scan) {
         // the leaf where the middle query would lie: a first bound
         float m[D];
 #pragma unroll
@@ -506,7 +575,7 @@ __global__ void __launch_bounds__(kLaneThreads, KM <= 8 ? 8 : 4) k_nn_lanes(NnQu
         visit(seed);
     }
     unsigned bits;
-    for (int nb = 0; nb < nnode; nb += 32) {
+    for (int nb = 0; nb < nnode && !scan; nb += 32) {
         float nd = __uint_as_float(kDone);
         if (nb + lane < nnode) nd = box_dist<D>(load_box<D>(nodebox + 2 * (nb + lane)), glo, ghi);
         while (true) {
@@ -528,6 +597,36 @@ __global__ void __launch_bounds__(kLaneThreads, KM <= 8 ? 8 : 4) k_nn_lanes(NnQu
             }
         }
     }
+    if (scan) {
+        float v[D];
+        load_row<D>(a.c, cfirst, cn, lane, v);
+        for (int at = lane; at - lane < cn; at += 32) {
+            float next[D];   // asked for before the present ones are offered
+            load_row<D>(a.c, cfirst, cn, at + 32, next);
+            if constexpr (KM == 1 && D >= 3) {   // one load of shared memory per candidate, rows in order
+                float4 *s4 = reinterpret_cast<float4 *>(s_c[w]);
+                __syncwarp();
+                s4[lane] = make_float4(v[0], v[1], v[2], v[D - 1]);
+                __syncwarp();
+#pragma unroll
+                for (int j = 0; j < 32; ++j) {
+                    const float4 c4 = s4[j];
+                    const float x[4] = {c4.x, c4.y, c4.z, c4.w};
+                    float p[D];
+#pragma unroll
+                    for (int c = 0; c < D; ++c) p[c] = x[c];
+                    const float d = point_dist<D>(q, p);
+                    const bool take = d < L.z[0];
+                    L.z[0] = take ? d : L.z[0];
+                    L.f[0] = take ? at - lane + j : L.f[0];
+                }
+            } else {
+                offer(v, at);
+            }
+#pragma unroll
+            for (int c = 0; c < D; ++c) v[c] = next[c];
+        }
+    }
     if (!valid) return;
     const long long out = (qfirst + qrow) * a.K;
 #pragma unroll
@@ -546,7 +645,8 @@ template <int D>
 __global__ void __launch_bounds__(kLaneThreads) k_nn_warps(NnQuery a) {
     int cloud, n;
     long long row0;
-    if (!tile_of(a.q, blockIdx.x, 2, cloud, row0, n)) return;
+    bool scan;
+    if (!query_tile(a.q, blockIdx.x, kWarpShift, cloud, row0, n, scan)) return;
     const int lane = threadIdx.x & 31, K = a.K;
     const long long pos = row0 + (threadIdx.x >> 5);
     if (pos >= n) return;   // uniform for the warp; no block barrier below
@@ -554,7 +654,10 @@ __global__ void __launch_bounds__(kLaneThreads) k_nn_warps(NnQuery a) {
     const int cn = (int)a.c.len[cloud];
     float q[D];
     int qrow;
-    {
+    if (scan) {
+        load_point<D>(a.q.x, qfirst + pos, q);
+        qrow = (int)pos;
+    } else {
         const float4 p = __ldg(a.q.pts + qfirst + pos);
         const float v[4] = {p.x, p.y, p.z, p.w};
 #pragma unroll
@@ -566,19 +669,8 @@ __global__ void __launch_bounds__(kLaneThreads) k_nn_warps(NnQuery a) {
     const int nleaf = (cn + kLeaf - 1) / kLeaf, nnode = (cn + kNode - 1) / kNode;
     const float4 *leafbox = a.c.leaf + 2 * ((cfirst >> 5) + cloud);
     const float4 *nodebox = a.c.node + 2 * ((cfirst >> 10) + cloud);
-    auto visit = [&](int leaf) {
-        const int at = leaf * kLeaf + lane;
-        float d = INFINITY;
-        int f = INT_MAX;
-        if (at < cn) {
-            const float4 c4 = __ldg(a.c.pts + cfirst + at);
-            const float v[4] = {c4.x, c4.y, c4.z, c4.w};
-            float p[D];
-#pragma unroll
-            for (int c = 0; c < D; ++c) p[c] = v[c];
-            d = point_dist<D>(q, p);
-            f = D < 4 ? __float_as_int(c4.w) : a.c.row[cfirst + at];
-        }
+    // the lanes' 32 candidates, offered to the query
+    auto offer = [&](float d, int f) {
         if (K == 1) {
             if (!before(d, f, tz, tf)) { d = INFINITY; f = INT_MAX; }   // NaN as well
             const unsigned u = __float_as_uint(d), m = __reduce_min_sync(kAll, u);
@@ -606,28 +698,71 @@ __global__ void __launch_bounds__(kLaneThreads) k_nn_warps(NnQuery a) {
             tf = __shfl_sync(kAll, ef, K - 1);
         }
     };
-    int seed = -1;
-    if (cn > 0) {
-        seed = min(__ldg(a.c.start + (size_t)cloud * a.c.cells + cell_of<D>(a.c, cloud, q)) / kLeaf, nleaf - 1);
-        visit(seed);
-    }
-    unsigned bits;
-    for (int nb = 0; nb < nnode; nb += 32) {
-        float nd = __uint_as_float(kDone);
-        if (nb + lane < nnode) nd = box_dist<D>(load_box<D>(nodebox + 2 * (nb + lane)), q, q);
-        while (true) {
-            const int nl = nearest_lane(nd, bits);
-            if (bits == kDone || !(__uint_as_float(bits) <= tz)) break;
-            if (lane == nl) nd = __uint_as_float(kDone);
-            const int base = (nb + nl) * 32;
-            float ld = __uint_as_float(kDone);
-            if (base + lane < nleaf && base + lane != seed)
-                ld = box_dist<D>(load_box<D>(leafbox + 2 * (base + lane)), q, q);
+    auto visit = [&](int leaf) {
+        const int at = leaf * kLeaf + lane;
+        float d = INFINITY;
+        int f = INT_MAX;
+        if (at < cn) {
+            float v[D];
+            f = load_leaf<D>(a.c, cfirst + at, v);
+            d = point_dist<D>(q, v);
+        }
+        offer(d, f);
+    };
+    if (!scan) {
+        int seed = -1;
+        if (cn > 0) {
+            seed = min(__ldg(a.c.start + (size_t)cloud * a.c.cells + cell_of<D>(a.c, cloud, q)) / kLeaf, nleaf - 1);
+            visit(seed);
+        }
+        unsigned bits;
+        for (int nb = 0; nb < nnode; nb += 32) {
+            float nd = __uint_as_float(kDone);
+            if (nb + lane < nnode) nd = box_dist<D>(load_box<D>(nodebox + 2 * (nb + lane)), q, q);
             while (true) {
-                const int ll = nearest_lane(ld, bits);
+                const int nl = nearest_lane(nd, bits);
                 if (bits == kDone || !(__uint_as_float(bits) <= tz)) break;
-                if (lane == ll) ld = __uint_as_float(kDone);
-                visit(base + ll);
+                if (lane == nl) nd = __uint_as_float(kDone);
+                const int base = (nb + nl) * 32;
+                float ld = __uint_as_float(kDone);
+                if (base + lane < nleaf && base + lane != seed)
+                    ld = box_dist<D>(load_box<D>(leafbox + 2 * (base + lane)), q, q);
+                while (true) {
+                    const int ll = nearest_lane(ld, bits);
+                    if (bits == kDone || !(__uint_as_float(bits) <= tz)) break;
+                    if (lane == ll) ld = __uint_as_float(kDone);
+                    visit(base + ll);
+                }
+            }
+        }
+    } else if (K == 1) {   // each lane its own candidates, in order of their rows
+        float z = INFINITY;
+        int f = INT_MAX;
+#pragma unroll 4
+        for (int at = lane; at < cn; at += 32) {
+            float v[D];
+            load_point<D>(a.c.x, cfirst + at, v);
+            const float d = point_dist<D>(q, v);
+            f = d < z ? at : f;
+            z = d < z ? d : z;
+        }
+        const unsigned u = __float_as_uint(z), m = __reduce_min_sync(kAll, u);
+        if (m != 0x7f800000u) {
+            ef = __reduce_min_sync(kAll, u == m ? f : INT_MAX);
+            ez = __uint_as_float(m);
+        }
+    } else {
+        float v[2][D];   // two rounds ahead
+        load_row<D>(a.c, cfirst, cn, lane, v[0]);
+        load_row<D>(a.c, cfirst, cn, lane + 32, v[1]);
+        for (int at = lane; at - lane < cn; at += 32) {
+            float next[D];
+            load_row<D>(a.c, cfirst, cn, at + 64, next);
+            offer(point_dist<D>(q, v[0]), at);
+#pragma unroll
+            for (int c = 0; c < D; ++c) {
+                v[0][c] = v[1][c];
+                v[1][c] = next[c];
             }
         }
     }
@@ -676,12 +811,14 @@ void layout_side(NnSide &s, int64_t N, int64_t P, int D, char *ws, size_t &zero,
     off = up256(off + (size_t)((P >> 10) + N + 1) * 2 * sizeof(float4));
 }
 
-// both sides; the part to be zeroed first comes first.  Returns the total, `zero` its leading bytes.
+// both sides; the part to be zeroed first comes first, the control word at its head.  Returns the total,
+// `zero` its leading bytes.
 size_t layout(NnSide (&sides)[2], int64_t N, int64_t P1, int64_t P2, int D, char *ws, size_t &zero) {
     size_t z = 0, off = 0;
     for (int pass = 0; pass < 2; ++pass) {   // the first pass finds the length of the zeroed part
         off = z;
-        z = 0;
+        z = up256(sizeof(NnControl));
+        sides[0].control = sides[1].control = reinterpret_cast<NnControl *>(ws);
         layout_side(sides[0], N, P1, D, ws, z, off);
         layout_side(sides[1], N, P2, D, ws, z, off);
     }
@@ -696,7 +833,7 @@ cudaError_t build_t(NnSide (&s)[2], int64_t N, bool boxes1, size_t zero, char *w
     const int64_t P = std::max(s[0].P, s[1].P);
     const unsigned g12 = (unsigned)((P >> 12) + N), g10 = (unsigned)((P >> 10) + N), g8 = (unsigned)((P >> 8) + N);
     const unsigned gt = (unsigned)(N * std::max(s[0].tiles, s[1].tiles));
-    k_nn_bounds<D><<<dim3(g12, 2), 256, 0, st>>>(s[0], s[1]);
+    k_nn_bounds<D><<<dim3(g12 + 1, 2), 256, 0, st>>>(s[0], s[1]);
     k_nn_count<D><<<dim3(g8, 2), 256, 0, st>>>(s[0], s[1]);
     if (s[0].tiles > 1 || s[1].tiles > 1) k_nn_tiles<<<dim3(gt, 2), 1024, 0, st>>>(s[0], s[1]);
     k_nn_starts<<<dim3(gt, 2), 1024, 0, st>>>(s[0], s[1]);
@@ -709,10 +846,10 @@ cudaError_t build_t(NnSide (&s)[2], int64_t N, bool boxes1, size_t zero, char *w
 template <int D>
 cudaError_t search_t(const NnQuery &a, bool warps, cudaStream_t st) {
     if (warps) {
-        k_nn_warps<D><<<(unsigned)((a.q.P >> 2) + a.q.N), kLaneThreads, 0, st>>>(a);
+        k_nn_warps<D><<<(unsigned)((a.q.P >> kWarpShift) + a.q.N), kLaneThreads, 0, st>>>(a);
         return cudaGetLastError();
     }
-    const unsigned g = (unsigned)((a.q.P >> 7) + a.q.N);
+    const unsigned g = (unsigned)((a.q.P >> kLaneShift) + a.q.N);
     if (a.K <= 1) k_nn_lanes<D, 1><<<g, kLaneThreads, 0, st>>>(a);
     else if (a.K <= 2) k_nn_lanes<D, 2><<<g, kLaneThreads, 0, st>>>(a);
     else if (a.K <= 4) k_nn_lanes<D, 4><<<g, kLaneThreads, 0, st>>>(a);
@@ -762,9 +899,13 @@ size_t nn_index_bytes(int64_t N, int64_t P1, int64_t P2, int D) {
 
 cudaError_t nn_index_build(NnSide (&s)[2], const float *p1, int64_t P1, const int64_t *first1, const int64_t *len1,
                            const float *p2, int64_t P2, const int64_t *first2, const int64_t *len2, int64_t N, int D,
-                           bool boxes1, char *ws, cudaStream_t st) {
+                           int K, bool both_ways, long long *plans, char *ws, cudaStream_t st) {
     size_t zero;
     layout(s, N, P1, P2, D, ws, zero);
+    s[0].plan = plans;
+    s[0].per = 1 << (per_warp(P1, P2, K) ? kWarpShift : kLaneShift);
+    s[1].plan = both_ways ? plans + N + 1 : nullptr;
+    s[1].per = 1 << (per_warp(P2, P1, K) ? kWarpShift : kLaneShift);
     s[0].x = p1;
     s[0].first = first1;
     s[0].len = len1;
@@ -772,10 +913,10 @@ cudaError_t nn_index_build(NnSide (&s)[2], const float *p1, int64_t P1, const in
     s[1].first = first2;
     s[1].len = len2;
     switch (D) {
-        case 1: return build_t<1>(s, N, boxes1, zero, ws, st);
-        case 2: return build_t<2>(s, N, boxes1, zero, ws, st);
-        case 3: return build_t<3>(s, N, boxes1, zero, ws, st);
-        default: return build_t<4>(s, N, boxes1, zero, ws, st);
+        case 1: return build_t<1>(s, N, both_ways, zero, ws, st);
+        case 2: return build_t<2>(s, N, both_ways, zero, ws, st);
+        case 3: return build_t<3>(s, N, both_ways, zero, ws, st);
+        default: return build_t<4>(s, N, both_ways, zero, ws, st);
     }
 }
 

@@ -7,14 +7,24 @@
 
 namespace mr {
 
+// Written by the first kernel of a call.
+struct NnControl {
+    int unfit;   // the clouds' ranges are not ascending and disjoint
+};
+
 // One batch of clouds in sorted form.  Cloud i keeps its own row range of the
 // packed arrays, its leaves start at (first >> 5) + i and its nodes at
 // (first >> 10) + i: first is non-decreasing and the ranges are disjoint, so
-// these never collide and no prefix over the clouds is needed.
+// these never collide and no prefix over the clouds is needed.  Clouds in other
+// ranges -- in any order, or one candidate cloud shared by many query clouds --
+// are not sorted; the search then scans every candidate where it lies.
 struct NnSide {
     const float *x;
     const int64_t *first, *len;
     int64_t P;
+    NnControl *control;         // one for both batches
+    long long *plan;            // N + 1: the scan's tiles of this batch as queries (NULL: never queries)
+    int per;                    // queries of such a tile
     int N, bits, cells, tiles;  // cells = 2^(bits D) per cloud, tiles of kNnTile cells
     unsigned *box;              // N x 8: running bounds, order-preserving bits
     int *start;                 // N x cells: counts, then the first sorted position of each cell
@@ -35,10 +45,12 @@ struct NnQuery {
 // Whether searching through the index beats scanning every candidate.
 bool nn_index_wins(int64_t N, int64_t P1, int64_t P2, int K);
 size_t nn_index_bytes(int64_t N, int64_t P1, int64_t P2, int D);
-// Sides laid out in `ws` (nn_index_bytes), built on `st`: sides[0] the first batch, sides[1] the second.
+// Sides laid out in `ws` (nn_index_bytes), built on `st`: sides[0] the first batch, sides[1] the second.  The
+// first is searched for K neighbours; with `both_ways` the second is, too.  `plans`: 2 (N + 1) words.
 cudaError_t nn_index_build(NnSide (&sides)[2], const float *p1, int64_t P1, const int64_t *first1,
                            const int64_t *len1, const float *p2, int64_t P2, const int64_t *first2,
-                           const int64_t *len2, int64_t N, int D, bool boxes1, char *ws, cudaStream_t st);
+                           const int64_t *len2, int64_t N, int D, int K, bool both_ways, long long *plans, char *ws,
+                           cudaStream_t st);
 cudaError_t nn_index_search(const NnSide &q, const NnSide &c, int D, int K, int64_t *idx, float *dists,
                             cudaStream_t st);
 
