@@ -329,6 +329,18 @@ struct KeyMap {
 
 __device__ __forceinline__ float entry_key(unsigned long long e) { return __uint_as_float((unsigned)(e >> 32)); }
 
+// Keys of either sign (points where znear is below 0) are kept in the order of
+// their values: the sign bit set on positive ones, all bits turned on negative.
+__device__ __forceinline__ unsigned signed_key_bits(float z) {
+    const unsigned u = __float_as_uint(z);
+    return (u & 0x80000000u) ? ~u : (u | 0x80000000u);
+}
+template <bool SIGNED>
+__device__ __forceinline__ float key_of_bits(unsigned u) {
+    if (SIGNED) u = (u & 0x80000000u) ? (u ^ 0x80000000u) : ~u;
+    return __uint_as_float(u);
+}
+
 // Where a block is in its bin's list; the same in every thread.
 struct WindowState {
     const unsigned long long *list;
@@ -341,8 +353,11 @@ struct WindowState {
     int base;        // entries of that level in front of the current window
 };
 
-template <int WIN>
+template <int WIN, bool SIGNED = false>
 struct WindowShared {
+    static __device__ __forceinline__ float key(unsigned long long e) {
+        return key_of_bits<SIGNED>((unsigned)(e >> 32));
+    }
     unsigned long long ent[WIN];      // the current window
     int pre[2][kBuckets + 1];         // entries before each bucket, per level
     int cur[kBuckets];
@@ -362,10 +377,11 @@ struct WindowShared {
     }
 };
 
-template <int BD, int WIN>
+template <int BD, int WIN, bool SIGNED>
 struct WindowLoader : WindowState {
-    WindowShared<WIN> &s;
-    __device__ __forceinline__ WindowLoader(WindowShared<WIN> &sh) : WindowState(sh.st), s(sh) {}
+    using Shared = WindowShared<WIN, SIGNED>;
+    Shared &s;
+    __device__ __forceinline__ WindowLoader(Shared &sh) : WindowState(sh.st), s(sh) {}
 
     __device__ __forceinline__ bool mine(float key, int level) const { return level == 0 || map[0](key) == b0; }
 
@@ -377,10 +393,10 @@ struct WindowLoader : WindowState {
         if (tid == 0) { s.lo = 0xffffffffu; s.hi = 0u; }
         for (int b = tid; b < kBuckets; b += BD) s.cur[b] = 0;
         __syncthreads();
-        unsigned lo = 0xffffffffu, hi = 0u;  // keys are positive: bits order like values
+        unsigned lo = 0xffffffffu, hi = 0u;  // the bits order like the values
         for (int i = tid; i < cnt; i += BD) {
             const unsigned long long e = __ldg(list + i);
-            if (!mine(entry_key(e), level)) continue;
+            if (!mine(Shared::key(e), level)) continue;
             lo = min(lo, (unsigned)(e >> 32));
             hi = max(hi, (unsigned)(e >> 32));
         }
@@ -389,12 +405,12 @@ struct WindowLoader : WindowState {
         if ((tid & 31) == 0) { atomicMin(&s.lo, lo); atomicMax(&s.hi, hi); }
         __syncthreads();
         KeyMap m;
-        m.lo = __uint_as_float(s.lo);
-        const float d = __uint_as_float(s.hi) - m.lo;
+        m.lo = key_of_bits<SIGNED>(s.lo);
+        const float d = key_of_bits<SIGNED>(s.hi) - m.lo;
         m.scale = d > 0.f ? __fdiv_rn((float)kBuckets, d) : 0.f;
         map[level] = m;
         for (int i = tid; i < cnt; i += BD) {
-            const float key = entry_key(__ldg(list + i));
+            const float key = Shared::key(__ldg(list + i));
             if (mine(key, level)) atomicAdd(&s.cur[m(key)], 1);
         }
         __syncthreads();
@@ -444,7 +460,7 @@ struct WindowLoader : WindowState {
             const KeyMap m = map[level];
             for (int i = threadIdx.x; i < cnt; i += BD) {
                 const unsigned long long v = __ldg(list + i);
-                const float key = entry_key(v);
+                const float key = Shared::key(v);
                 if (!mine(key, level)) continue;
                 const int k = m(key);
                 if (k < b || k >= e) continue;
@@ -475,7 +491,7 @@ struct WindowLoader : WindowState {
                 const int m = min(WIN, cnt - seg);
                 for (int i = threadIdx.x; i < m; i += BD) {
                     const unsigned long long v = __ldg(list + seg + i);
-                    const float key = entry_key(v);
+                    const float key = Shared::key(v);
                     if (map[0](key) == b0 && map[1](key) == b1) s.ent[atomicAdd(&s.n, 1)] = v;
                 }
                 seg += m;
@@ -514,8 +530,8 @@ struct WindowLoader : WindowState {
 
 // Starts on a list; `ordered` false hands it out as it is.  Every thread of the
 // block calls this and window_next.
-template <int BD, int WIN>
-__device__ __forceinline__ void window_begin(WindowShared<WIN> &s, const unsigned long long *list, int cnt,
+template <int BD, int WIN, bool SIGNED>
+__device__ __forceinline__ void window_begin(WindowShared<WIN, SIGNED> &s, const unsigned long long *list, int cnt,
                                              bool ordered) {
     __syncthreads();
     if (threadIdx.x == 0) {
@@ -535,9 +551,9 @@ __device__ __forceinline__ void window_begin(WindowShared<WIN> &s, const unsigne
 // Loads the next window into s.ent and returns its size; 0 at the end.  Every
 // thread must be done with the last window.  Not inlined: the walk between two
 // windows keeps its registers.
-template <int BD, int WIN>
-static __device__ __noinline__ int window_next(WindowShared<WIN> &s) {
-    WindowLoader<BD, WIN> w(s);
+template <int BD, int WIN, bool SIGNED>
+static __device__ __noinline__ int window_next(WindowShared<WIN, SIGNED> &s) {
+    WindowLoader<BD, WIN, SIGNED> w(s);
     if (w.cnt <= 0) return 0;
     if (w.b0 < 0) {
         w.template deal<0>();

@@ -179,9 +179,9 @@ __global__ void __launch_bounds__(256) k_pfill(PtArgs a) {
         }
         return n;
     };
-    // depth bits (positive float) in the high word: integer order = front to back, ties by id
+    // depth in the high word, so that integer order is front to back, ties by id
     auto entry = [](const PtRec &R, int64_t i) {
-        return ((unsigned long long)__float_as_uint(R.b.x) << 32) | (unsigned)i;
+        return ((unsigned long long)signed_key_bits(R.b.x) << 32) | (unsigned)i;
     };
     if constexpr (!HIST) {
         for (int u = 0; u < PER; ++u) {
@@ -328,7 +328,7 @@ __device__ __forceinline__ void pt_composite(const PtArgs &a, const int *ids, co
 template <int BS, bool RENDER>
 __global__ void __launch_bounds__(kPfineThreads) k_pfine(PtArgs a) {
     constexpr int BD = kPfineThreads, WIN = kPfineWindow, PX = BS * BS;
-    __shared__ WindowShared<WIN> s_win;
+    __shared__ WindowShared<WIN, true> s_win;
     __shared__ int s_ids[WIN];             // the window's points, in order
     __shared__ unsigned s_bits[WIN / 32][PX];
     __shared__ float2 s_cx[BS], s_cy[BS];  // pixel centres of the bin's columns and rows
@@ -369,7 +369,7 @@ __global__ void __launch_bounds__(kPfineThreads) k_pfine(PtArgs a) {
                 const unsigned long long e = s_win.ent[i];
                 int lo = 0, hi = m;
                 if (lvl >= 0) {
-                    const int k = s_win.rank(entry_key(e));
+                    const int k = s_win.rank(s_win.key(e));
                     lo = s_win.pre[lvl][k] - s_win.st.base;
                     hi = s_win.pre[lvl][k + 1] - s_win.st.base;
                 }
@@ -450,7 +450,7 @@ __global__ void __launch_bounds__(kPfineThreads) k_pfine(PtArgs a) {
                                 if (held < K) l[held++] = oid;
                                 continue;
                             }
-                            const float z = entry_key(s_win.ent[jb + src]);
+                            const float z = s_win.key(s_win.ent[jb + src]);
                             auto before = [&](int other) {
                                 return key_less(z, oid, __ldg(reinterpret_cast<const float *>(a.rec + other) + 4), other);
                             };
