@@ -179,8 +179,10 @@ __device__ __forceinline__ void sort_stage_local(unsigned long long (&v)[E], int
     }
 }
 
+// From k_first = N2: only the last merge, of a sequence that is bitonic already.
 template <int BD, int E>
-__device__ __forceinline__ void sort_entries_regs(unsigned long long *s_sort, const unsigned long long *src, int m) {
+__device__ __forceinline__ void sort_entries_regs(unsigned long long *s_sort, const unsigned long long *src, int m,
+                                                  int k_first = 2) {
     constexpr int N2 = BD * E;
     const int tid = threadIdx.x;
     unsigned long long v[E];
@@ -190,7 +192,7 @@ __device__ __forceinline__ void sort_entries_regs(unsigned long long *s_sort, co
         v[e] = i < m ? src[i] : ~0ull;
     }
 #pragma unroll 1
-    for (int k2 = 2; k2 <= N2; k2 <<= 1) {
+    for (int k2 = k_first; k2 <= N2; k2 <<= 1) {
 #pragma unroll 1
         for (int j2 = k2 >> 1; j2 > 0; j2 >>= 1) {
             if (j2 < E) {
@@ -210,13 +212,14 @@ __device__ __forceinline__ void sort_entries_regs(unsigned long long *s_sort, co
                 }
                 continue;
             }
+            // (entries e of the threads side by side: no bank conflicts)
 #pragma unroll
-            for (int e = 0; e < E; ++e) s_sort[tid * E + e] = v[e];
+            for (int e = 0; e < E; ++e) s_sort[e * BD + tid] = v[e];
             __syncthreads();
 #pragma unroll
             for (int e = 0; e < E; ++e) {
                 const int i = tid * E + e;
-                const unsigned long long o = s_sort[i ^ j2];
+                const unsigned long long o = s_sort[e * BD + (tid ^ (j2 / E))];
                 const bool keep_min = ((i & j2) == 0) == ((i & k2) == 0);
                 v[e] = keep_min ? (o < v[e] ? o : v[e]) : (o > v[e] ? o : v[e]);
             }
@@ -317,6 +320,15 @@ __device__ __forceinline__ void sort_entries(unsigned long long *s_sort, const u
 // the bucket of a pixel's K-th depth with a window's buckets decides, without
 // knowing any window's smallest key, that everything from there on is behind.
 // ---------------------------------------------------------------------------
+//
+// Every window reads the whole list for its entries, so a list beyond kLongList
+// entries is sorted in place before the fine pass (sort_long.cu) and handed out
+// as it lies: 1.6M points on 16 px, K = 1, bins of 8: dealt 307 ms, sorted 6.9;
+// 200,000 on 64 px, bins of 16: 1,696 us, 356; 1.3M faces on 16 px, bins of 8: 331
+// ms, 30.7.  With the line at 8,192, 16,384 and 32,768 entries: 1.6M points on 128 px,
+// bins of 8, 560, 902, 1,132 us; 1.3M faces on 128 px, K = 8, 1,934, 2,632, 2,509.  Where
+// few of a list's windows are needed the order is not paid back in full: 328k
+// faces on 64 px, bins of 16, K = 1: dealt 1,760, sorted 1,857.
 constexpr int kBuckets = 256;
 
 struct KeyMap {
@@ -347,8 +359,9 @@ struct WindowState {
     int cnt;
     KeyMap map[2];
     int b0, b1;      // next bucket of level 0; of level 1 while `deep`
-    int seg;         // >= 0: next piece of the list (unordered, or a level-1 bucket that does not fit)
+    int seg;         // >= 0: next piece of the list (as it lies, or a level-1 bucket that does not fit)
     int deep, plain;
+    int ascending;   // plain, and the list is sorted
     int sorted;      // level whose buckets order the current window, -1: none
     int base;        // entries of that level in front of the current window
 };
@@ -369,9 +382,14 @@ struct WindowShared {
     // bucket that orders the current window (constant when nothing does)
     __device__ __forceinline__ int rank(float key) const { return st.sorted < 0 ? 0 : st.map[st.sorted](key); }
 
+    // whether the key and all that follow it in the current window lie behind depth z
+    __device__ __forceinline__ bool behind(float key, float z) const {
+        return st.ascending ? z < key : rank(z) < rank(key);
+    }
+
     // whether every entry not yet handed out lies behind depth z
     __device__ __forceinline__ bool rest_behind(float z) const {
-        if (st.plain) return false;
+        if (st.plain) return st.ascending && (st.seg >= st.cnt || z < WindowShared::key(__ldg(st.list + st.seg)));
         const int k = st.map[0](z);
         return k < st.b0 || (st.deep && k == st.b0 && st.map[1](z) < st.b1);
     }
@@ -385,6 +403,21 @@ struct WindowLoader : WindowState {
 
     __device__ __forceinline__ bool mine(float key, int level) const { return level == 0 || map[0](key) == b0; }
 
+    // f on every entry of the list, several loads in flight per thread (one at a
+    // time, 64 threads wait for 128 round trips to L2 on a list of 8,192)
+    template <class F>
+    __device__ __forceinline__ void for_list(const F &f) const {
+        constexpr int U = WIN / BD < 4 ? 4 : WIN / BD;
+        for (int i = threadIdx.x; i < cnt; i += U * BD) {
+            unsigned long long e[U];
+#pragma unroll
+            for (int u = 0; u < U; ++u) e[u] = i + u * BD < cnt ? __ldg(list + i + u * BD) : 0ull;
+#pragma unroll
+            for (int u = 0; u < U; ++u)
+                if (i + u * BD < cnt) f(e[u]);
+        }
+    }
+
     // ranges and counts of the buckets of a level
     template <int level>
     __device__ __forceinline__ void deal() {
@@ -394,12 +427,11 @@ struct WindowLoader : WindowState {
         for (int b = tid; b < kBuckets; b += BD) s.cur[b] = 0;
         __syncthreads();
         unsigned lo = 0xffffffffu, hi = 0u;  // the bits order like the values
-        for (int i = tid; i < cnt; i += BD) {
-            const unsigned long long e = __ldg(list + i);
-            if (!mine(Shared::key(e), level)) continue;
+        for_list([&](unsigned long long e) {
+            if (!mine(Shared::key(e), level)) return;
             lo = min(lo, (unsigned)(e >> 32));
             hi = max(hi, (unsigned)(e >> 32));
-        }
+        });
         lo = __reduce_min_sync(0xffffffffu, lo);
         hi = __reduce_max_sync(0xffffffffu, hi);
         if ((tid & 31) == 0) { atomicMin(&s.lo, lo); atomicMax(&s.hi, hi); }
@@ -409,10 +441,10 @@ struct WindowLoader : WindowState {
         const float d = key_of_bits<SIGNED>(s.hi) - m.lo;
         m.scale = d > 0.f ? __fdiv_rn((float)kBuckets, d) : 0.f;
         map[level] = m;
-        for (int i = tid; i < cnt; i += BD) {
-            const float key = Shared::key(__ldg(list + i));
+        for_list([&](unsigned long long e) {
+            const float key = Shared::key(e);
             if (mine(key, level)) atomicAdd(&s.cur[m(key)], 1);
-        }
+        });
         __syncthreads();
         // exclusive prefix of the counts: kBuckets / BD consecutive buckets per thread
         constexpr int E = kBuckets / BD;
@@ -458,14 +490,13 @@ struct WindowLoader : WindowState {
         const int n = s.pre[level][e] - s.pre[level][b];
         if (n > 0) {
             const KeyMap m = map[level];
-            for (int i = threadIdx.x; i < cnt; i += BD) {
-                const unsigned long long v = __ldg(list + i);
+            for_list([&](unsigned long long v) {
                 const float key = Shared::key(v);
-                if (!mine(key, level)) continue;
+                if (!mine(key, level)) return;
                 const int k = m(key);
-                if (k < b || k >= e) continue;
+                if (k < b || k >= e) return;
                 s.ent[s.pre[level][k] - s.pre[level][b] + atomicAdd(&s.cur[k], 1)] = v;
-            }
+            });
             __syncthreads();
         }
         sorted = level;
@@ -528,11 +559,12 @@ struct WindowLoader : WindowState {
     }
 };
 
-// Starts on a list; `ordered` false hands it out as it is.  Every thread of the
-// block calls this and window_next.
+// Starts on a list; `ordered` false hands it out as it is, `ascending` says that
+// it is sorted.  Every thread of the block calls this and window_next.
 template <int BD, int WIN, bool SIGNED>
 __device__ __forceinline__ void window_begin(WindowShared<WIN, SIGNED> &s, const unsigned long long *list, int cnt,
-                                             bool ordered) {
+                                             bool ordered, bool ascending) {
+    ordered = ordered && !ascending;
     __syncthreads();
     if (threadIdx.x == 0) {
         s.st.list = list;
@@ -542,6 +574,7 @@ __device__ __forceinline__ void window_begin(WindowShared<WIN, SIGNED> &s, const
         s.st.seg = ordered ? -1 : 0;
         s.st.deep = 0;
         s.st.plain = !ordered;
+        s.st.ascending = ascending;
         s.st.sorted = -1;
         s.st.base = 0;
     }

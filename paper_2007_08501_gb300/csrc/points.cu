@@ -6,6 +6,7 @@
 //              (NDC position hi/lo, depth), warp-aggregated bin counts
 //   k_scan     (shared with the mesh rasterizer) clamp counts, prefix scan
 //   k_pfill    one thread per point: append depth-keyed entries to its bins
+//   k_sort_long (sort_long.cu) lists of more than 8,192 entries
 //   k_pfine    persistent blocks over (image, bin) items: the bin's entries
 //              front to back in windows, each pixel's points appended in
 //              (depth, id) order; stops a bin once every pixel holds K
@@ -51,6 +52,7 @@ struct PtArgs {
     const int *eff, *offsets;
     unsigned long long *lists;
     unsigned *queue, *status;
+    int sorted_long;   // lists beyond kLongList entries are sorted
     int64_t *idx;
     float *zbuf, *dists;
     // rendering on packed slots (distance bits << 32 | id, ended by kPtEnd)
@@ -281,7 +283,7 @@ __device__ __forceinline__ void pt_write(const PtArgs &a, int64_t pix, const Top
 // A splat's depth is the same at every pixel, so once a bin's entries are in
 // (depth, id) order every pixel gets its fragments by appending.  Per window of
 // the bin's list (depth buckets, bin_common.cuh):
-//   1. the entries of a bucket (a handful) are put in order by counting, for
+//   1. the entries of a bucket (a handful; a list sorted before is in order) are put in order by counting, for
 //      each, the bucket's smaller ones;
 //   2. small splats: one thread per point sets the point's bit in the row of
 //      each pixel it covers; large splats: a warp walks the points for its 32
@@ -358,7 +360,8 @@ __global__ void __launch_bounds__(kPfineThreads) k_pfine(PtArgs a) {
         for (int i = tid; i < PX; i += BD) s_cnt[i] = (i / BS < rows && i % BS < cols) ? 0 : K;
         auto centre = [&](int r, int c) { return PixC{s_cx[c].x, s_cx[c].y, s_cy[r].x, s_cy[r].y}; };
         const int cnt = a.eff[item];
-        window_begin<BD>(s_win, a.lists + a.offsets[item], cnt, cnt > 32);
+        const bool ascending = a.sorted_long && cnt > kLongList;
+        window_begin<BD>(s_win, a.lists + a.offsets[item], cnt, cnt > 32, ascending);
         while (const int m = window_next<BD>(s_win)) {
             // pieces of a bucket that fits no window come in any order, and so do
             // their entries: those are inserted
@@ -367,6 +370,10 @@ __global__ void __launch_bounds__(kPfineThreads) k_pfine(PtArgs a) {
             bool big = false;
             for (int i = tid; i < m && !pieces; i += BD) {
                 const unsigned long long e = s_win.ent[i];
+                if (ascending) {
+                    s_ids[i] = (int)(unsigned)(e & 0xffffffffull);
+                    continue;
+                }
                 int lo = 0, hi = m;
                 if (lvl >= 0) {
                     const int k = s_win.rank(s_win.key(e));
@@ -1175,6 +1182,9 @@ static int pts_forward(mr::PtArgs &out, const pts_params *p, const float *points
     if (P > 0) {
         if (mr::launch_pfill(a, st) != cudaSuccess) return MESHRAST_ERR_CUDA;
     }
+    a.sorted_long = p->max_points_per_bin > mr::kLongList;
+    if (a.sorted_long && mr::launch_sort_long({a.lists, a.eff, a.offsets, sa.maxcount, a.items}, st) != cudaSuccess)
+        return MESHRAST_ERR_CUDA;
     return mr::launch_pfine(a, p->bin_size, st) == cudaSuccess ? MESHRAST_OK : MESHRAST_ERR_CUDA;
 }
 

@@ -17,6 +17,7 @@ namespace mr {
 
 constexpr float kCullArea = 1e-12f;
 constexpr int kMaxK = 64;
+constexpr int kLongList = 8192;  // entries beyond which a bin's list is sorted before the fine pass
 
 // ---------------------------------------------------------------------------
 // Staged face record: 96 bytes, six float4, written once per face by the

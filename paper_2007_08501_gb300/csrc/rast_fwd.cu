@@ -8,6 +8,8 @@
 //               record, warp-aggregated bin counts
 //   k_scan      one block: clamp counts to capacity, exclusive scan -> offsets
 //   k_fill      one thread per face: warp-aggregated atomic append into lists
+//   k_sort_long (sort_long.cu) lists of more than 8,192 entries, where bins may
+//               hold as many
 //   k_fine      persistent blocks pull (image, bin) items from a global queue,
 //               walk each bin's faces front to back, keep a register-resident
 //               top-K per pixel, write the fragments
@@ -610,14 +612,14 @@ __global__ void __launch_bounds__(BS *BS, fine_blocks(KM) * 256 / (BS * BS)) k_f
         // against 633 us at 1.3M faces, 1024 px, K = 8, 225 against 176 for 5
         // meshes at 225 px; reading them from L1 one by one, 297 against 246
         // where few faces reach a warp: 1.3M faces, K = 1, no blur.)
-        window_begin<BD>(s_win, a.lists + off, cnt, zcull && cnt > 64);
+        window_begin<BD>(s_win, a.lists + off, cnt, zcull && cnt > 64, a.sorted_long && cnt > kLongList);
         while (const int m = window_next<BD>(s_win)) {
             for (int i = tid; i < m; i += BD)
                 s_box[i] = __ldg(reinterpret_cast<const float4 *>(a.rec + (unsigned)s_win.ent[i]) + kRecC);
             __syncthreads();
             for (int jb = 0; jb < m; jb += 32) {
                 const float wthr = warp_kth();
-                if (zcull && s_win.rank(wthr) < s_win.rank(entry_key(s_win.ent[jb]))) break;
+                if (zcull && s_win.behind(entry_key(s_win.ent[jb]), wthr)) break;
                 const int jl = jb + lane;
                 bool hit = false;
                 if (jl < m) {

@@ -81,6 +81,7 @@ struct FineArgs {
     unsigned *queue;
     unsigned *spilled;          // large-K streaming pass: pixels whose unsettled candidates outgrew the ring
     int items, nb, S, K;
+    int sorted_long;  // lists beyond kLongList entries are sorted
     int sort_cap;  // streaming pass: bin entries sorted at a time (power of two)
     float inv_sigma;  // streaming pass with packed slots: 1 / sigma
     EvalFlags fl;
@@ -117,6 +118,14 @@ struct SilBwdArgs {
     int64_t F, V;
     int N, S, K;
     float sigma;
+};
+
+// Lists beyond kLongList entries sorted in place.
+struct SortLongArgs {
+    unsigned long long *lists;
+    const int *eff, *offsets;
+    const int *maxcount;  // largest count of any bin
+    int64_t items;
 };
 
 struct NaiveArgs {
@@ -166,6 +175,7 @@ cudaError_t launch_scan(const ScanArgs &a, cudaStream_t st);
 cudaError_t launch_fill(const FillArgs &a, cudaStream_t st);
 cudaError_t launch_fine(const FineArgs &a, int bin, cudaStream_t st);
 bool fine_blends(int K, bool rgb);  // whether launch_fine applies FineArgs::blend
+cudaError_t launch_sort_long(const SortLongArgs &a, cudaStream_t st);
 cudaError_t launch_naive(const NaiveArgs &a, int N, cudaStream_t st);
 // large K: front-to-back streaming fine pass + attribute pass (fine_stream.cu)
 cudaError_t launch_fine_stream(const FineArgs &a, int bin, cudaStream_t st);
