@@ -24,8 +24,8 @@
 //                for the spatial index (knn_index.cu), which serves the rest.
 //   k_pair_sums / k_mean   per-pair Chamfer terms and the batch mean, fixed
 //                reduction order
-//   k_chamfer_bwd / k_knn_bwd   gradients, scattered to the neighbours by
-//                vector reductions
+//   k_chamfer_bwd / k_knn_bwd   gradients, scattered to the neighbours with
+//                warp aggregation by target row
 #include <cuda_runtime.h>
 
 #include <climits>
@@ -556,6 +556,24 @@ __device__ __forceinline__ int cloud_of(long long r, const int64_t *first, const
     return r < first[lo] + len[lo] ? lo : -1;
 }
 
+// -v added to row `target` (-1: none) of g, equal rows of the warp as one.  Every
+// lane of the warp calls it.  Sent one by one, the terms of one row queue up, 20
+// ns each: clouds of 50,000 points against a cloud beside them, whose few
+// nearest points are every query's neighbours (8 clouds of 50,000, K = 8: 538 us,
+// grouped 67), or against a few points (32 x 50,000 against 8, K = 1: 518, 77).
+// Where a warp's neighbours all differ the grouping costs little (8 x 50,000
+// against 50,000 around it, K = 8: 62.6, 64.6).
+template <int D>
+__device__ __forceinline__ void red_sub_grouped(float *g, long long target, float (&v)[D]) {
+    const unsigned lane = threadIdx.x & 31u;
+    const unsigned peers = __match_any_sync(0xffffffffu, target >= 0 ? target : -1 - (long long)lane);
+    group_sum<D>(peers, v);
+    if (target < 0 || (__ffs(peers) - 1) != (int)lane) return;
+#pragma unroll
+    for (int c = 0; c < D; ++c) v[c] = -v[c];
+    red_add_row<D>(g, target, v, (reinterpret_cast<uintptr_t>(g) & 7u) == 0);
+}
+
 struct ChamferBwdArgs {
     const float *p, *q;
     const int64_t *first1, *len1, *first2, *len2;
@@ -566,30 +584,40 @@ struct ChamferBwdArgs {
     int N;
 };
 
-// A thread per point of either batch: its own term and its neighbour's, sent
-// straight to the reduction units (see k_knn_bwd).
+// A thread per point of either batch: its own term, and its neighbour's summed
+// over the warp's equal neighbours.
 template <int D>
 __global__ void __launch_bounds__(256) k_chamfer_bwd(ChamferBwdArgs a) {
     const long long r = (long long)blockIdx.x * blockDim.x + threadIdx.x;
     const bool dir = r >= a.P1;   // false: rows of p (p -> q), true: rows of q (q -> p)
     const long long rr = dir ? r - a.P1 : r;
-    if (r >= a.P1 + a.P2) return;
+    const bool in = r < a.P1 + a.P2;
     const float *x = dir ? a.q : a.p, *y = dir ? a.p : a.q;
-    float *gx = dir ? a.grad_q : a.grad_p, *gy = dir ? a.grad_p : a.grad_q;
-    const int i = dir ? cloud_of(rr, a.first2, a.len2, a.N) : cloud_of(rr, a.first1, a.len1, a.N);
-    const long long nb = (dir ? a.idx_qp : a.idx_pq)[rr];
-    if (i < 0 || nb < 0) return;
-    float w = a.grad_per_pair ? a.grad_per_pair[i] : 0.f;
-    if (a.grad_loss) w += a.grad_loss[0] / (float)a.N;
-    const float coef = 2.f * w / (float)(dir ? a.len2[i] : a.len1[i]);
-    float v[D], m[D];
+    float *gx = dir ? a.grad_q : a.grad_p;
+    const int i = !in ? -1 : dir ? cloud_of(rr, a.first2, a.len2, a.N) : cloud_of(rr, a.first1, a.len1, a.N);
+    const long long nb = i < 0 ? -1 : (dir ? a.idx_qp : a.idx_pq)[rr];
+    float v[D];
 #pragma unroll
-    for (int c = 0; c < D; ++c) {
-        v[c] = coef * (x[rr * D + c] - y[nb * D + c]);
-        m[c] = -v[c];
+    for (int c = 0; c < D; ++c) v[c] = 0.f;
+    if (nb >= 0) {
+        float w = a.grad_per_pair ? a.grad_per_pair[i] : 0.f;
+        if (a.grad_loss) w += a.grad_loss[0] / (float)a.N;
+        const float coef = 2.f * w / (float)(dir ? a.len2[i] : a.len1[i]);
+#pragma unroll
+        for (int c = 0; c < D; ++c) v[c] = coef * (x[rr * D + c] - y[nb * D + c]);
+        red_add_row<D>(gx, rr, v, (reinterpret_cast<uintptr_t>(gx) & 7u) == 0);
     }
-    red_add_row<D>(gx, rr, v, (reinterpret_cast<uintptr_t>(gx) & 7u) == 0);
-    red_add_row<D>(gy, nb, m, (reinterpret_cast<uintptr_t>(gy) & 7u) == 0);
+    // lanes of one warp may straddle the two directions: one at a time
+    const unsigned both = __ballot_sync(0xffffffffu, dir);
+    if (both == 0u || both == 0xffffffffu) {
+        red_sub_grouped<D>(dir ? a.grad_p : a.grad_q, nb, v);
+        return;
+    }
+    float u[D];
+#pragma unroll
+    for (int c = 0; c < D; ++c) u[c] = v[c];
+    red_sub_grouped<D>(a.grad_q, dir ? -1 : nb, v);
+    red_sub_grouped<D>(a.grad_p, dir ? nb : -1, u);
 }
 
 struct KnnBwdArgs {
@@ -601,34 +629,36 @@ struct KnnBwdArgs {
     int K;
 };
 
-// A thread per query, its K neighbours' terms sent straight to the reduction
-// units.  Bound by the reductions; grouping a warp's equal targets first only
-// pays when neighbouring rows share neighbours, which sampled clouds do not.
+// A thread per query; its K neighbours' terms summed over the warp's equal
+// neighbours.  Bound by the reductions.
 template <int D>
 __global__ void __launch_bounds__(256) k_knn_bwd(KnnBwdArgs a) {
     const long long r = (long long)blockIdx.x * blockDim.x + threadIdx.x;
-    if (r >= a.P1) return;
-    const bool pairs = (reinterpret_cast<uintptr_t>(a.grad_p2) & 7u) == 0;
+    const bool in = r < a.P1;
     float x[D], own[D];
 #pragma unroll
     for (int c = 0; c < D; ++c) {
-        x[c] = a.p1[r * D + c];
+        x[c] = in ? a.p1[r * D + c] : 0.f;
         own[c] = 0.f;
     }
 #pragma unroll 4
     for (int k = 0; k < a.K; ++k) {
-        const long long nb = a.idx[r * a.K + k];
-        if (nb < 0 || nb >= a.P2) continue;
-        const float g2 = 2.f * a.grad_dists[r * a.K + k];
+        long long nb = in ? a.idx[r * a.K + k] : -1;
+        if (nb >= a.P2) nb = -1;
         float v[D];
 #pragma unroll
-        for (int c = 0; c < D; ++c) {
-            const float t = g2 * (x[c] - a.p2[nb * D + c]);
-            own[c] += t;
-            v[c] = -t;
+        for (int c = 0; c < D; ++c) v[c] = 0.f;
+        if (nb >= 0) {
+            const float g2 = 2.f * a.grad_dists[r * a.K + k];
+#pragma unroll
+            for (int c = 0; c < D; ++c) {
+                v[c] = g2 * (x[c] - a.p2[nb * D + c]);
+                own[c] += v[c];
+            }
         }
-        red_add_row<D>(a.grad_p2, nb, v, pairs);
+        red_sub_grouped<D>(a.grad_p2, nb, v);
     }
+    if (!in) return;
 #pragma unroll
     for (int c = 0; c < D; ++c) a.grad_p1[r * D + c] = own[c];
 }
