@@ -309,9 +309,11 @@ static int forward(const rast_params *p, const float *verts, int64_t V, const in
         if (blended) *blended = true;
     }
     // (no order without depth culling)
-    ka.sorted_long = p->max_faces_per_bin > mr::kLongList && (fl.clip || !(fl.blur > 0.f));
-    if (ka.sorted_long && mr::launch_sort_long({ka.lists, ka.eff, ka.offsets, sa.maxcount, L.NB}, st) != cudaSuccess)
-        return MESHRAST_ERR_CUDA;
+    if (p->max_faces_per_bin > mr::kLongList && (fl.clip || !(fl.blur > 0.f))) {
+        ka.total = sa.total;
+        if (mr::launch_sort_long({ka.lists, ka.eff, ka.offsets, sa.maxcount, sa.total, L.NB}, st) != cudaSuccess)
+            return MESHRAST_ERR_CUDA;
+    }
     return mr::launch_fine(ka, p->bin_size, st) == cudaSuccess ? MESHRAST_OK : MESHRAST_ERR_CUDA;
 }
 

@@ -321,14 +321,15 @@ __device__ __forceinline__ void sort_entries(unsigned long long *s_sort, const u
 // knowing any window's smallest key, that everything from there on is behind.
 // ---------------------------------------------------------------------------
 //
-// Every window reads the whole list for its entries, so a list beyond kLongList
-// entries is sorted in place before the fine pass (sort_long.cu) and handed out
-// as it lies: 1.6M points on 16 px, K = 1, bins of 8: dealt 307 ms, sorted 6.9;
-// 200,000 on 64 px, bins of 16: 1,696 us, 356; 1.3M faces on 16 px, bins of 8: 331
-// ms, 30.7.  With the line at 8,192, 16,384 and 32,768 entries: 1.6M points on 128 px,
-// bins of 8, 560, 902, 1,132 us; 1.3M faces on 128 px, K = 8, 1,934, 2,632, 2,509.  Where
-// few of a list's windows are needed the order is not paid back in full: 328k
-// faces on 64 px, bins of 16, K = 1: dealt 1,760, sorted 1,857.
+// Every window reads the whole list for its entries.  Where few lists are long
+// (beyond 16,384 entries and a 64th of all bins' entries), those are sorted in place
+// before the fine pass (sort_long.cu) and handed out as they lie: 1.6M points on 16
+// px, K = 1, bins of 8: dealt 307 ms, sorted 7.2; 200,000 on 64 px, bins of 16: 1,696
+// us, 573; 1.3M faces on 16 px, K = 8, soft, bins of 8: 378 ms, 40.0; on 64 px, hard,
+// bins of 16: 29.9, 14.7.  Where many are, they fill the GPU as they are and most stop
+// after a few windows: 1.3M faces on 1,024 px (1,600 lists of 8,000 to 20,000), K = 8:
+// 972 us dealt, 1,764 with all of them sorted.  In between it is a draw: 328k faces on
+// 64 px, bins of 16, K = 1: dealt 1,760, sorted 1,869; on 128 px, K = 8, soft: 931, 1,076.
 constexpr int kBuckets = 256;
 
 struct KeyMap {

@@ -6,7 +6,8 @@
 //              (NDC position hi/lo, depth), warp-aggregated bin counts
 //   k_scan     (shared with the mesh rasterizer) clamp counts, prefix scan
 //   k_pfill    one thread per point: append depth-keyed entries to its bins
-//   k_sort_long (sort_long.cu) lists of more than 8,192 entries
+//   k_sort_runs, k_merge_runs (sort_long.cu) where bins may hold more than
+//              kLongList entries: long lists
 //   k_pfine    persistent blocks over (image, bin) items: the bin's entries
 //              front to back in windows, each pixel's points appended in
 //              (depth, id) order; stops a bin once every pixel holds K
@@ -52,7 +53,7 @@ struct PtArgs {
     const int *eff, *offsets;
     unsigned long long *lists;
     unsigned *queue, *status;
-    int sorted_long;   // lists beyond kLongList entries are sorted
+    const long long *total;  // entries of all bins, where long lists are sorted (else NULL)
     int64_t *idx;
     float *zbuf, *dists;
     // rendering on packed slots (distance bits << 32 | id, ended by kPtEnd)
@@ -339,6 +340,7 @@ __global__ void __launch_bounds__(kPfineThreads) k_pfine(PtArgs a) {
     extern __shared__ int s_list[];        // [pixel][K] ids, rows an odd number of words apart
     const int tid = threadIdx.x, lane = tid & 31;
     const int nb2 = a.nb * a.nb, K = a.K, stride = K | 1;
+    const int sorted_from = a.total ? long_list(*a.total) : 0x7fffffff;
     const unsigned magic_K = (unsigned)((0x100000000ull + (unsigned)K - 1) / (unsigned)K);
     const float w = a.radius * (1.f + kPtSlack);
     // a splat's half width in pixels, with slack for the rounding of its centre's column
@@ -360,7 +362,7 @@ __global__ void __launch_bounds__(kPfineThreads) k_pfine(PtArgs a) {
         for (int i = tid; i < PX; i += BD) s_cnt[i] = (i / BS < rows && i % BS < cols) ? 0 : K;
         auto centre = [&](int r, int c) { return PixC{s_cx[c].x, s_cx[c].y, s_cy[r].x, s_cy[r].y}; };
         const int cnt = a.eff[item];
-        const bool ascending = a.sorted_long && cnt > kLongList;
+        const bool ascending = cnt > sorted_from;
         window_begin<BD>(s_win, a.lists + a.offsets[item], cnt, cnt > 32, ascending);
         while (const int m = window_next<BD>(s_win)) {
             // pieces of a bucket that fits no window come in any order, and so do
@@ -1182,9 +1184,11 @@ static int pts_forward(mr::PtArgs &out, const pts_params *p, const float *points
     if (P > 0) {
         if (mr::launch_pfill(a, st) != cudaSuccess) return MESHRAST_ERR_CUDA;
     }
-    a.sorted_long = p->max_points_per_bin > mr::kLongList;
-    if (a.sorted_long && mr::launch_sort_long({a.lists, a.eff, a.offsets, sa.maxcount, a.items}, st) != cudaSuccess)
-        return MESHRAST_ERR_CUDA;
+    if (p->max_points_per_bin > mr::kLongList) {
+        a.total = sa.total;
+        if (mr::launch_sort_long({a.lists, a.eff, a.offsets, sa.maxcount, sa.total, a.items}, st) != cudaSuccess)
+            return MESHRAST_ERR_CUDA;
+    }
     return mr::launch_pfine(a, p->bin_size, st) == cudaSuccess ? MESHRAST_OK : MESHRAST_ERR_CUDA;
 }
 

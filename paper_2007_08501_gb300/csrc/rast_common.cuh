@@ -17,7 +17,14 @@ namespace mr {
 
 constexpr float kCullArea = 1e-12f;
 constexpr int kMaxK = 64;
-constexpr int kLongList = 8192;  // entries beyond which a bin's list is sorted before the fine pass
+
+// Entries beyond which a bin's list is sorted before the fine pass, with `total`
+// in all bins (bin_common.cuh says why).
+constexpr int kLongList = 16384;
+__host__ __device__ __forceinline__ int long_list(long long total) {
+    const long long share = total / 64;
+    return share < kLongList ? kLongList : share > 0x7fffffffLL ? 0x7fffffff : (int)share;
+}
 
 // ---------------------------------------------------------------------------
 // Staged face record: 96 bytes, six float4, written once per face by the

@@ -8,8 +8,8 @@
 //               record, warp-aggregated bin counts
 //   k_scan      one block: clamp counts to capacity, exclusive scan -> offsets
 //   k_fill      one thread per face: warp-aggregated atomic append into lists
-//   k_sort_long (sort_long.cu) lists of more than 8,192 entries, where bins may
-//               hold as many
+//   k_sort_runs, k_merge_runs (sort_long.cu) where bins may hold more than
+//               kLongList entries: long lists
 //   k_fine      persistent blocks pull (image, bin) items from a global queue,
 //               walk each bin's faces front to back, keep a register-resident
 //               top-K per pixel, write the fragments
@@ -545,6 +545,7 @@ __global__ void __launch_bounds__(BS *BS, fine_blocks(KM) * 256 / (BS * BS)) k_f
     EvalFlags fl = a.fl;
     const bool zcull = fl.clip || !(fl.blur > 0.f);
     const int nb2 = a.nb * a.nb;
+    const int sorted_from = a.total ? long_list(*a.total) : 0x7fffffff;
     float4 (*const rec)[5] = s_rec[tid >> 5];
     while (true) {
         if (tid == 0) s_item = (int)atomicAdd(a.queue, 1u);
@@ -612,7 +613,7 @@ __global__ void __launch_bounds__(BS *BS, fine_blocks(KM) * 256 / (BS * BS)) k_f
         // against 633 us at 1.3M faces, 1024 px, K = 8, 225 against 176 for 5
         // meshes at 225 px; reading them from L1 one by one, 297 against 246
         // where few faces reach a warp: 1.3M faces, K = 1, no blur.)
-        window_begin<BD>(s_win, a.lists + off, cnt, zcull && cnt > 64, a.sorted_long && cnt > kLongList);
+        window_begin<BD>(s_win, a.lists + off, cnt, zcull && cnt > 64, cnt > sorted_from);
         while (const int m = window_next<BD>(s_win)) {
             for (int i = tid; i < m; i += BD)
                 s_box[i] = __ldg(reinterpret_cast<const float4 *>(a.rec + (unsigned)s_win.ent[i]) + kRecC);

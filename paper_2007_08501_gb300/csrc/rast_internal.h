@@ -81,7 +81,7 @@ struct FineArgs {
     unsigned *queue;
     unsigned *spilled;          // large-K streaming pass: pixels whose unsettled candidates outgrew the ring
     int items, nb, S, K;
-    int sorted_long;  // lists beyond kLongList entries are sorted
+    const long long *total;  // entries of all bins, where long lists are sorted (else NULL)
     int sort_cap;  // streaming pass: bin entries sorted at a time (power of two)
     float inv_sigma;  // streaming pass with packed slots: 1 / sigma
     EvalFlags fl;
@@ -120,11 +120,12 @@ struct SilBwdArgs {
     float sigma;
 };
 
-// Lists beyond kLongList entries sorted in place.
+// Lists beyond long_list entries sorted in place.
 struct SortLongArgs {
     unsigned long long *lists;
     const int *eff, *offsets;
-    const int *maxcount;  // largest count of any bin
+    const int *maxcount;     // largest count of any bin
+    const long long *total;  // entries of all bins
     int64_t items;
 };
 

@@ -2,7 +2,7 @@
 //
 // A fine pass fetches its windows from the list it has, so a list of n entries
 // that no early stop shortens costs it n^2 / window loads.  Lists beyond
-// kLongList entries are therefore sorted in place first: runs of 8,192, each by
+// long_list entries are therefore sorted in place first: runs of 8,192, each by
 // a block of its own, in registers and shared memory; then one block per list
 // merges them in global memory (L2) down to runs, the rest of each merge in
 // shared memory again.  The network sorts ascending throughout (each merge
@@ -66,12 +66,13 @@ template <class F>
 __device__ __forceinline__ void for_long(const SortLongArgs &a, const F &f) {
     __shared__ int s_bins[kSortThreads];
     __shared__ int s_n;
-    if (*a.maxcount <= kLongList) return;
+    const int from = long_list(*a.total);
+    if (*a.maxcount <= from) return;
     for (int64_t base = blockIdx.x; base < a.items; base += (int64_t)gridDim.x * kSortThreads) {
         if (threadIdx.x == 0) s_n = 0;
         __syncthreads();
         const int64_t b = base + (int64_t)threadIdx.x * gridDim.x;
-        if (b < a.items && a.eff[b] > kLongList) s_bins[atomicAdd(&s_n, 1)] = (int)b;
+        if (b < a.items && a.eff[b] > from) s_bins[atomicAdd(&s_n, 1)] = (int)b;
         __syncthreads();
         for (int q = 0; q < s_n; ++q) f(a.lists + a.offsets[s_bins[q]], (unsigned)a.eff[s_bins[q]]);
         __syncthreads();

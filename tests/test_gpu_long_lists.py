@@ -1,6 +1,6 @@
-"""Bins of more entries than a list is dealt into windows for: their lists are
-sorted first.  Every Fragment value is bit-exact against the plain form, which
-meets faces and points in packed order."""
+"""Bins of so many entries that the fine pass leaves them to a second round on
+sorted lists, beside bins that it finishes.  Every Fragment value is bit-exact
+against the plain form, which meets faces and points in packed order."""
 import numpy as np
 import pytest
 import torch
@@ -20,9 +20,9 @@ def _depths(kind, n, rng):
 
 
 @pytest.mark.parametrize("kind,n,K,blur,clip", [
-    ("mixed", 8192, 1, 0.0, False), ("mixed", 8193, 8, 1e-3, True), ("levels", 16_385, 5, 1e-3, True),
-    ("flat", 20_000, 3, 0.0, False), ("mixed", 70_001, 8, 1e-3, True), ("mixed", 24_577, 24, 1e-3, True),
-    ("levels", 9_000, 50, 0.0, False), ("mixed", 20_000, 24, 1e-3, False), ("mixed", 20_000, 16, 1e-3, False)])
+    ("mixed", 32_768, 1, 0.0, False), ("mixed", 32_769, 8, 1e-3, True), ("levels", 40_961, 5, 1e-3, True),
+    ("flat", 50_000, 3, 0.0, False), ("mixed", 70_001, 8, 1e-3, True), ("mixed", 33_000, 24, 1e-3, True),
+    ("levels", 40_000, 50, 0.0, False), ("mixed", 40_000, 24, 1e-3, False), ("mixed", 40_000, 16, 1e-3, False)])
 def test_long_face_lists_match_the_plain_form(kind, n, K, blur, clip):
     rng = np.random.default_rng(n + K)
     z = _depths(kind, n, rng)[:, None] * np.ones(3)
@@ -41,7 +41,7 @@ def test_long_face_lists_match_the_plain_form(kind, n, K, blur, clip):
 
 
 @pytest.mark.parametrize("kind,n,K,radius", [
-    ("mixed", 8192, 4, 0.05), ("mixed", 8193, 10, 0.02), ("levels", 16_385, 50, 0.1), ("flat", 20_000, 3, 0.9),
+    ("mixed", 32_768, 4, 0.05), ("mixed", 32_769, 10, 0.02), ("levels", 40_961, 50, 0.1), ("flat", 50_000, 3, 0.9),
     ("mixed", 70_001, 50, 0.03), ("levels", 300_000, 1, 0.02), ("mixed", 131_073, 64, 0.02)])
 def test_long_point_lists_match_the_plain_form(kind, n, K, radius):
     rng = np.random.default_rng(3 * n + K)
