@@ -799,6 +799,13 @@ struct PtsBwdArgs {
     float inv_r2;
 };
 
+// Splats of this radius in pixels and up: a warp's slots of one point are summed
+// before the reduction.  Reductions into one accumulator queue up, 20 ns each, and a
+// large splat has thousands: 8 clouds of 100 points, radius 128 px, K = 8, D = 3,
+// forward and backward 1,577 us, grouped 315; 8 of 2,000, radius 26 px, K = 50, D = 3,
+// 785, 673.  Small ones find few peers: the same at 6.4 px 392, 401 (D = 1: 362, 383).
+constexpr float kGroupRadius = 16.f;
+
 constexpr int pts_acc_vecs(int D) { return D <= 2 ? 1 : D <= 6 ? 2 : 3; }
 
 __device__ __forceinline__ void red_add4(float4 *p, float x, float y, float z, float w) {
@@ -806,27 +813,27 @@ __device__ __forceinline__ void red_add4(float4 *p, float x, float y, float z, f
                  : "memory");
 }
 
-template <int DM>
+template <int DM, bool GROUP>
 __global__ void __launch_bounds__(256) k_pts_bwd(PtsBwdArgs a) {
     __shared__ float s_T[kCompChunks][256];
     const int tid = threadIdx.x;
     const int tx = ((tid >> 5) & 1) * 8 + (tid & 7), ty = (tid >> 6) * 4 + ((tid >> 3) & 3);
     const int row = blockIdx.y * 16 + ty, col = blockIdx.x * 16 + tx;
-    if (row >= a.S || col >= a.S) return;
     const int64_t pix = ((int64_t)blockIdx.z * a.S + row) * a.S + col;
     const unsigned long long *s = a.slots + pix * a.K;
-    if (__ldg(s) == kPtEnd) return;
+    const bool any = row < a.S && col < a.S && __ldg(s) != kPtEnd;
+    if (GROUP ? !__any_sync(0xffffffffu, any) : !any) return;
     const bool norm = a.mode == PTS_COMPOSITE_NORM;
     float g[DM], out[DM], E[DM], f_next[DM];
 #pragma unroll
     for (int ch = 0; ch < DM; ++ch) {
-        g[ch] = ch < a.D ? a.grad_image[pix * a.D + ch] : 0.f;
+        g[ch] = any && ch < a.D ? a.grad_image[pix * a.D + ch] : 0.f;
         out[ch] = E[ch] = f_next[ch] = 0.f;
     }
     // forward: the transmittance at the start of each chunk, Norm's mean
     float T = 1.f, asum = 0.f;
     int held = 0, chunks = 0;
-    for (bool more = true; more && held < a.K; ++chunks) {
+    for (bool more = any; more && held < a.K; ++chunks) {
         s_T[chunks][tid] = T;
         unsigned long long v[kCompChunk];
 #pragma unroll
@@ -854,10 +861,11 @@ __global__ void __launch_bounds__(256) k_pts_bwd(PtsBwdArgs a) {
     const PixC p = pixel_centre(row, col, a.S);
     float q_next = 0.f;
     bool has_next = false;
-    for (int c = chunks - 1; c >= 0; --c) {
+    // (GROUP: the warp's lanes take the same chunk and rank, with or without a slot there)
+    for (int c = (GROUP ? (int)__reduce_max_sync(0xffffffffu, (unsigned)chunks) : chunks) - 1; c >= 0; --c) {
         unsigned long long v[kCompChunk];
         float4 pos[kCompChunk];
-        float Tv[kCompChunk], Tc = s_T[c][tid];
+        float Tv[kCompChunk], Tc = !GROUP || c < chunks ? s_T[c][tid] : 1.f;
 #pragma unroll
         for (int j = 0; j < kCompChunk; ++j) {
             const bool in = c * kCompChunk + j < held;
@@ -868,38 +876,51 @@ __global__ void __launch_bounds__(256) k_pts_bwd(PtsBwdArgs a) {
         }
 #pragma unroll
         for (int j = kCompChunk - 1; j >= 0; --j) {
-            if (c * kCompChunk + j >= held) continue;
+            const bool in = c * kCompChunk + j < held;
+            if (!GROUP && !in) continue;
             const int64_t i = (unsigned)v[j];
-            const float q = __uint_as_float((unsigned)(v[j] >> 32)) * a.inv_r2, al = 1.f - q;
-            float ga = 0.f, gf[DM > 2 ? DM : 2];
-            gf[1] = 0.f;
+            // the slot's sums: x, y, features (even: room for the second of a pair)
+            constexpr int NS = 2 + (DM > 2 ? DM : 2);
+            float sum[NS];
 #pragma unroll
-            for (int ch = 0; ch < DM; ++ch) {
-                gf[ch] = 0.f;
-                if (ch >= a.D) continue;
-                const float fc = __ldg(a.features + i * a.D + ch);
-                if (norm) {
-                    gf[ch] = al * inv_a * g[ch];
-                    ga += g[ch] * (fc - out[ch]) * inv_a;
-                } else {
-                    E[ch] = has_next ? (fc - f_next[ch]) + q_next * E[ch] : fc;
-                    f_next[ch] = fc;
-                    gf[ch] = al * Tv[j] * g[ch];
-                    ga += g[ch] * Tv[j] * E[ch];
+            for (int u = 0; u < NS; ++u) sum[u] = 0.f;
+            if (in) {
+                const float q = __uint_as_float((unsigned)(v[j] >> 32)) * a.inv_r2, al = 1.f - q;
+                float ga = 0.f;
+#pragma unroll
+                for (int ch = 0; ch < DM; ++ch) {
+                    if (ch >= a.D) continue;
+                    const float fc = __ldg(a.features + i * a.D + ch);
+                    if (norm) {
+                        sum[2 + ch] = al * inv_a * g[ch];
+                        ga += g[ch] * (fc - out[ch]) * inv_a;
+                    } else {
+                        E[ch] = has_next ? (fc - f_next[ch]) + q_next * E[ch] : fc;
+                        f_next[ch] = fc;
+                        sum[2 + ch] = al * Tv[j] * g[ch];
+                        ga += g[ch] * Tv[j] * E[ch];
+                    }
                 }
+                q_next = q;
+                has_next = true;
+                const float gd = -ga * a.inv_r2;
+                const float qx = __fadd_rn(__fsub_rn(p.xh, pos[j].x), __fsub_rn(p.xl, pos[j].z));
+                const float qy = __fadd_rn(__fsub_rn(p.yh, pos[j].y), __fsub_rn(p.yl, pos[j].w));
+                sum[0] = -2.f * gd * qx;
+                sum[1] = -2.f * gd * qy;
             }
-            q_next = q;
-            has_next = true;
-            const float gd = -ga * a.inv_r2;
-            const float qx = __fadd_rn(__fsub_rn(p.xh, pos[j].x), __fsub_rn(p.xl, pos[j].z));
-            const float qy = __fadd_rn(__fsub_rn(p.yh, pos[j].y), __fsub_rn(p.yl, pos[j].w));
+            if constexpr (GROUP) {
+                const unsigned peers = __match_any_sync(0xffffffffu, in ? (int)i : -1 - (tid & 31));
+                group_sum<NS>(peers, sum);
+                if (!in || (tid & 31) != __ffs(peers) - 1) continue;
+            }
             float4 *acc = a.acc + i * pts_acc_vecs(a.D);
-            red_add4(acc, -2.f * gd * qx, -2.f * gd * qy, gf[0], gf[1]);
+            red_add4(acc, sum[0], sum[1], sum[2], sum[3]);
             if constexpr (DM >= 4) {
-                if (a.D > 2) red_add4(acc + 1, gf[2], gf[3], DM > 4 ? gf[DM > 4 ? 4 : 0] : 0.f, DM > 4 ? gf[DM > 4 ? 5 : 0] : 0.f);
+                if (a.D > 2) red_add4(acc + 1, sum[4], sum[5], DM > 4 ? sum[DM > 4 ? 6 : 0] : 0.f, DM > 4 ? sum[DM > 4 ? 7 : 0] : 0.f);
             }
             if constexpr (DM > 6) {
-                if (a.D > 6) red_add4(acc + 2, gf[6], gf[7], 0.f, 0.f);
+                if (a.D > 6) red_add4(acc + 2, sum[8], sum[9], 0.f, 0.f);
             }
         }
     }
@@ -938,6 +959,13 @@ __global__ void __launch_bounds__(256) k_pts_gather(PtsBwdArgs a) {
 // ---------------------------------------------------------------------------
 // host side
 // ---------------------------------------------------------------------------
+template <bool GROUP>
+static void launch_pts_bwd(const PtsBwdArgs &a, const dim3 &grid, cudaStream_t st) {
+    if (a.D == 1) k_pts_bwd<1, GROUP><<<grid, 256, 0, st>>>(a);
+    else if (a.D <= 4) k_pts_bwd<4, GROUP><<<grid, 256, 0, st>>>(a);
+    else k_pts_bwd<8, GROUP><<<grid, 256, 0, st>>>(a);
+}
+
 static int km_for_points(int K) {
     if (K <= 1) return 1;
     if (K <= 2) return 2;
@@ -1369,9 +1397,8 @@ int pts_render_bwd(const pts_params *p, int32_t mode, int64_t P, const float *ca
     if (cudaMemsetAsync(scratch, 0, bytes, st) != cudaSuccess) return MESHRAST_ERR_CUDA;
     const unsigned tiles = (unsigned)((p->image_size + 15) / 16);
     const dim3 grid(tiles, tiles, (unsigned)p->N);
-    if (D == 1) mr::k_pts_bwd<1><<<grid, 256, 0, st>>>(a);
-    else if (D <= 4) mr::k_pts_bwd<4><<<grid, 256, 0, st>>>(a);
-    else mr::k_pts_bwd<8><<<grid, 256, 0, st>>>(a);
+    if (0.5f * p->radius * (float)p->image_size >= mr::kGroupRadius) mr::launch_pts_bwd<true>(a, grid, st);
+    else mr::launch_pts_bwd<false>(a, grid, st);
     if (cudaGetLastError() != cudaSuccess) return MESHRAST_ERR_CUDA;
     mr::k_pts_gather<<<(unsigned)((P + 255) / 256), 256, 0, st>>>(a);
     return cudaGetLastError() == cudaSuccess ? MESHRAST_OK : MESHRAST_ERR_CUDA;
