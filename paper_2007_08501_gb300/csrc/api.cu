@@ -308,8 +308,8 @@ static int forward(const rast_params *p, const float *verts, int64_t V, const in
         ka.blend.frag = no_frag ? 0 : 1;
         if (blended) *blended = true;
     }
-    // (no order without depth culling)
-    if (p->max_faces_per_bin > mr::kLongList && (fl.clip || !(fl.blur > 0.f))) {
+    // (an order pays with depth culling, or where the pixels' lists are inserted into from their ends)
+    if (p->max_faces_per_bin > mr::kLongList && (fl.clip || !(fl.blur > 0.f) || K > 16)) {
         ka.total = sa.total;
         if (mr::launch_sort_long({ka.lists, ka.eff, ka.offsets, sa.maxcount, sa.total, L.NB}, st) != cudaSuccess)
             return MESHRAST_ERR_CUDA;

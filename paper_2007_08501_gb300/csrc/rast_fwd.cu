@@ -519,19 +519,32 @@ __device__ __forceinline__ void write_pixel_packed(const FineBlend &bl, int64_t 
 // ---------------------------------------------------------------------------
 // fine pass: persistent blocks, one bin (bin x bin pixels = block) per item
 // ---------------------------------------------------------------------------
-// entries per window of the bin's list: a window of the usual bin is the whole
-// of it, and at 8 KB the blocks an SM holds stay limited by registers
-constexpr int fine_window(int BS) { return BS >= 16 ? 1024 : 512; }
-// blocks of 256 threads per SM: 64, 80 and 128 registers hold the lists and the face test
-constexpr int fine_blocks(int KM) { return KM <= 4 ? 4 : KM == 8 ? 3 : 2; }
+// Two forms of a window.  0: what an early stop shortens; as many entries as fit the
+// usual bin whole.  1: K > 16 without depth culling, where every face is met: an order
+// only keeps the insertions short (unordered, 4 meshes of 81,920 faces, 256 px, K = 50:
+// 7,008 us; ordered 4,673), and room for another block counts for more than long
+// windows.  Shared memory of a block, besides the lists, and blocks per SM: form 0 48 KB
+// (bins of 16) or 13 KB, limited by registers; form 1 27 or 11 KB, 3 blocks of bins of
+// 16 at K = 24 (8 meshes of 5,120 faces, 256 px: 483 -> 421 us; bins of 8, K = 50: 663 ->
+// 595).
+constexpr int fine_window(int BS, int FORM) { return FORM ? (BS >= 16 ? 384 : 256) : BS >= 16 ? 1024 : 512; }
+// Where the walk has a window's boxes from: the eight warps of a bin of 16 share them
+// in shared memory (1.3M faces, K = 1: 382 us; with the records 402); the two warps of a
+// bin of 8 bring them with the records, which leaves room for 16 blocks (8 meshes of
+// 5,120 faces, 256 px, K = 4: 144 -> 132); form 1 reads them from L1.
+enum { kBoxWindow, kBoxRecord, kBoxL1 };
+constexpr int fine_boxes(int BS, int FORM) { return BS < 16 ? kBoxRecord : FORM ? kBoxL1 : kBoxWindow; }
+// blocks per SM: 64, 80 and 128 registers hold the lists and the face test (K > 16: the
+// lists in shared memory leave room for fewer)
+constexpr int fine_blocks(int KM, int BS) { return (KM <= 4 ? 4 : KM == 8 ? 3 : 2) * 256 / (BS * BS); }
 
 // OUT: 0 Fragment data, 1 with the silhouette blend, 2 packed silhouette slots with it
-template <int KM, int BS, int OUT>
-__global__ void __launch_bounds__(BS *BS, fine_blocks(KM) * 256 / (BS * BS)) k_fine(FineArgs a) {
+template <int KM, int BS, int OUT, int FORM>
+__global__ void __launch_bounds__(BS *BS, fine_blocks(KM, BS)) k_fine(FineArgs a) {
     constexpr int BD = BS * BS;
-    constexpr int WIN = fine_window(BS);
-    __shared__ float4 s_box[WIN];               // the window's bboxes: lanes read them side by side
-    __shared__ float4 s_rec[BD / 32][32][5];    // per warp: a, b, d, e, h of the faces it walks next
+    constexpr int WIN = fine_window(BS, FORM), BOX = fine_boxes(BS, FORM), NREC = BOX == kBoxRecord ? 6 : 5;
+    __shared__ float4 s_box[BOX == kBoxWindow ? WIN : 1];  // the window's bboxes: lanes read them side by side
+    __shared__ float4 s_rec[BD / 32][32][NREC];            // per warp: a, b, d, e, h (c) of the faces it walks next
     __shared__ WindowShared<WIN> s_win;
     __shared__ int s_item;
     // K > 16: the per-thread lists
@@ -546,7 +559,7 @@ __global__ void __launch_bounds__(BS *BS, fine_blocks(KM) * 256 / (BS * BS)) k_f
     const bool zcull = fl.clip || !(fl.blur > 0.f);
     const int nb2 = a.nb * a.nb;
     const int sorted_from = a.total ? long_list(*a.total) : 0x7fffffff;
-    float4 (*const rec)[5] = s_rec[tid >> 5];
+    float4 (*const rec)[NREC] = s_rec[tid >> 5];
     while (true) {
         if (tid == 0) s_item = (int)atomicAdd(a.queue, 1u);
         __syncthreads();
@@ -597,7 +610,8 @@ __global__ void __launch_bounds__(BS *BS, fine_blocks(KM) * 256 / (BS * BS)) k_f
             return __int_as_float(__reduce_max_sync(0xffffffffu, valid ? __float_as_int(kth()) : 0));
         };
         // The bin's faces in front-to-back windows (two warps' worth is not
-        // worth ordering; without depth culling the order buys nothing).
+        // worth ordering; without depth culling the order only helps lists in
+        // shared memory, which are inserted into from their ends).
         // Within a window the warps go their own way.  Faces are culled 32 at
         // a time for the whole warp: lane j tests face jb + j against the
         // rectangle spanned by the warp's pixel centres and against the warp's
@@ -613,19 +627,22 @@ __global__ void __launch_bounds__(BS *BS, fine_blocks(KM) * 256 / (BS * BS)) k_f
         // against 633 us at 1.3M faces, 1024 px, K = 8, 225 against 176 for 5
         // meshes at 225 px; reading them from L1 one by one, 297 against 246
         // where few faces reach a warp: 1.3M faces, K = 1, no blur.)
-        window_begin<BD>(s_win, a.lists + off, cnt, zcull && cnt > 64, cnt > sorted_from);
+        window_begin<BD>(s_win, a.lists + off, cnt, (zcull || KM == 0) && cnt > 64, cnt > sorted_from);
         while (const int m = window_next<BD>(s_win)) {
-            for (int i = tid; i < m; i += BD)
-                s_box[i] = __ldg(reinterpret_cast<const float4 *>(a.rec + (unsigned)s_win.ent[i]) + kRecC);
-            __syncthreads();
+            if constexpr (BOX == kBoxWindow) {
+                for (int i = tid; i < m; i += BD)
+                    s_box[i] = __ldg(reinterpret_cast<const float4 *>(a.rec + (unsigned)s_win.ent[i]) + kRecC);
+                __syncthreads();
+            }
             for (int jb = 0; jb < m; jb += 32) {
                 const float wthr = warp_kth();
                 if (zcull && s_win.behind(entry_key(s_win.ent[jb]), wthr)) break;
                 const int jl = jb + lane;
                 bool hit = false;
                 if (jl < m) {
-                    const float4 bb = s_box[jl];
                     const unsigned long long e = s_win.ent[jl];
+                    const float4 bb =
+                        BOX == kBoxWindow ? s_box[jl] : __ldg(reinterpret_cast<const float4 *>(a.rec + (unsigned)e) + kRecC);
                     hit = bb.x <= wx1 && bb.y >= wx0 && bb.z <= wy1 && bb.w >= wy0 && !(zcull && entry_key(e) > wthr);
                     if (hit) {
                         const float4 *src = reinterpret_cast<const float4 *>(a.rec + (unsigned)e);
@@ -634,6 +651,7 @@ __global__ void __launch_bounds__(BS *BS, fine_blocks(KM) * 256 / (BS * BS)) k_f
                         rec[lane][2] = __ldg(src + kRecD);
                         rec[lane][3] = __ldg(src + kRecE);
                         rec[lane][4] = __ldg(src + kRecH);
+                        if constexpr (BOX == kBoxRecord) rec[lane][5] = bb;
                     }
                 }
                 unsigned mask = __ballot_sync(0xffffffffu, hit);
@@ -643,7 +661,9 @@ __global__ void __launch_bounds__(BS *BS, fine_blocks(KM) * 256 / (BS * BS)) k_f
                     mask &= mask - 1;
                     if (!valid) continue;
                     FaceRec R;
-                    R.c = s_box[jj];
+                    if constexpr (BOX == kBoxWindow) R.c = s_box[jj];
+                    else if constexpr (BOX == kBoxRecord) R.c = rec[j][5];
+                    else R.c = __ldg(reinterpret_cast<const float4 *>(a.rec + (unsigned)s_win.ent[jj]) + kRecC);
                     if (!in_bbox(R, p)) continue;
                     const unsigned long long e = s_win.ent[jj];
                     if (zcull && entry_key(e) > kth()) continue;
@@ -868,11 +888,11 @@ static int km_for(int K) {
     return 0;  // shared-memory lists
 }
 
-template <int KM, int BS, int OUT>
+template <int KM, int BS, int OUT, int FORM = 0>
 static cudaError_t launch_fine_t(const FineArgs &a, cudaStream_t st) {
     constexpr int BD = BS * BS;
     const size_t dyn = (KM > 0) ? (size_t)0 : (size_t)BD * a.K * 8;
-    auto kern = k_fine<KM, BS, OUT>;
+    auto kern = k_fine<KM, BS, OUT, FORM>;
     cudaError_t e = cudaSuccess;
     if (dyn > 0) {  // static + dynamic above 48 KB needs the opt-in
         e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)dyn);
@@ -899,8 +919,9 @@ cudaError_t launch_fine(const FineArgs &a, int bin, cudaStream_t st) {
     MR_FINE(1, 16) MR_FINE(2, 16) MR_FINE(4, 16) MR_FINE(8, 16) MR_FINE(16, 16)
 #undef MR_FINE
     if (km == 0) {
-        if (bin == 8) return launch_fine_t<0, 8, 0>(a, st);
-        if (bin == 16) return launch_fine_t<0, 16, 0>(a, st);
+        const bool zcull = a.fl.clip || !(a.fl.blur > 0.f);
+        if (bin == 8) return zcull ? launch_fine_t<0, 8, 0>(a, st) : launch_fine_t<0, 8, 0, 1>(a, st);
+        if (bin == 16) return zcull ? launch_fine_t<0, 16, 0>(a, st) : launch_fine_t<0, 16, 0, 1>(a, st);
     }
     return cudaErrorInvalidValue;
 }

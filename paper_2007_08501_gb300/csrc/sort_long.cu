@@ -115,7 +115,7 @@ cudaError_t launch_sort_long(const SortLongArgs &a, cudaStream_t st) {
     if (e != cudaSuccess) return e;
     e = cudaFuncSetAttribute(k_merge_runs, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)dyn);
     if (e != cudaSuccess) return e;
-    const int lists = mr_host::queue_blocks(a.items, 1);
+    const int lists = (int)(a.items < 64 ? a.items : 64);  // (fewer than 64 are long)
     k_sort_runs<<<dim3((unsigned)lists, 8), kSortThreads, dyn, st>>>(a);
     k_merge_runs<<<lists, kSortThreads, dyn, st>>>(a);
     return cudaGetLastError();
