@@ -456,17 +456,6 @@ int rast_blend_fwd(const rast_params *p, const blend_params *bp, const float *ve
     fbl.on = 1;
     fbl.rgb = rgb ? 1 : 0;
     fbl.sigma = bp->sigma;
-    fbl.gamma = bp->gamma;
-    fbl.znear = bp->znear;
-    fbl.zfar = bp->zfar;
-    fbl.eps = bp->eps;
-    fbl.bg0 = bp->bg[0];
-    fbl.bg1 = bp->bg[1];
-    fbl.bg2 = bp->bg[2];
-    fbl.faces = faces;
-    fbl.colors = vert_colors;
-    fbl.F = F;
-    fbl.V = V;
     fbl.image = image;
     bool blended = false;
     rc = forward(p, verts, V, faces, F, first_face, num_faces, cams, pix_to_face, zbuf, bary, dists, workspace,
@@ -593,11 +582,6 @@ int sil_fwd(const rast_params *p, const blend_params *bp, const float *verts, in
     std::memset(&fbl, 0, sizeof(fbl));
     fbl.on = 1;
     fbl.sigma = bp->sigma;
-    fbl.gamma = bp->gamma;
-    fbl.znear = bp->znear;
-    fbl.zfar = bp->zfar;
-    fbl.eps = bp->eps;
-    fbl.F = F;
     fbl.image = image;
     fbl.slots = reinterpret_cast<unsigned long long *>(slots);
     fbl.keep = keep;

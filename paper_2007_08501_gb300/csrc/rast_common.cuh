@@ -427,14 +427,6 @@ struct TopK {
             f[k] = unused ? -1 : 0x7fffffff;
         }
     }
-    // nearest entry (slot KM - K)
-    __device__ __forceinline__ void first(int K, float &zz, int &ff) const {
-        zz = z[0];
-        ff = f[0];
-#pragma unroll
-        for (int k = 1; k < KM; ++k)
-            if (k == KM - K) { zz = z[k]; ff = f[k]; }
-    }
     __device__ __forceinline__ bool admits(float zz, int ff) const { return key_less(zz, ff, z[KM - 1], f[KM - 1]); }
     __device__ __forceinline__ void insert(float zz, int ff) {
         z[KM - 1] = zz;

@@ -381,12 +381,6 @@ __device__ __forceinline__ void write_pixel(const FineOut &o, int64_t pix, int K
                                             const FineBlend &bl) {
     const int64_t s0 = pix * (int64_t)K;
     FwdBlend fb;
-    if constexpr (BL) {
-        float z0;
-        int f0;
-        tk.first(K, z0, f0);
-        fb.begin(bl, f0 != 0x7fffffff, z0);
-    }
 #pragma unroll
     for (int k = 0; k < KM; ++k) {
         if (k < KM - K) continue;
@@ -420,7 +414,7 @@ __device__ __forceinline__ void write_pixel(const FineOut &o, int64_t pix, int K
                 o.bary[3 * s + 2] = bp[2];
                 o.dists[s] = d;
             }
-            if constexpr (BL) fb.slot(bl, f, tk.z[k], d, bp);
+            if constexpr (BL) fb.slot(bl, d);
         }
     }
     if constexpr (BL) fb.end(bl, pix);
@@ -439,7 +433,6 @@ __device__ __forceinline__ void write_pixel_vec(const FineOut &o, int64_t pix, i
         return;
     }
     FwdBlend fb;
-    if constexpr (BL) fb.begin(bl, tk.f[0] != 0x7fffffff, tk.z[0]);
     const bool store = !BL || bl.frag;
     const int64_t s0 = pix * KM;
     const unsigned long long pol = l2_keep_policy();
@@ -475,7 +468,7 @@ __device__ __forceinline__ void write_pixel_vec(const FineOut &o, int64_t pix, i
             R.e = __ldg(src + kRecE);
             face_fragment(R, p, fl, bb[i], dd[i]);
             zz[i] = tk.z[k];
-            if constexpr (BL) fb.slot(bl, tk.f[k], zz[i], dd[i], bb[i]);
+            if constexpr (BL) fb.slot(bl, dd[i]);
         }
         if (!store) continue;
         st_keep(zp + j, make_float4(zz[0], zz[1], zz[2], zz[3]), pol);

@@ -55,16 +55,13 @@ struct FineOut {
     float *zbuf, *bary, *dists;
 };
 
-// Blend (Algorithm 1; the fields of Algorithm 2 are kept for FwdBlend) applied
-// by the fine pass to each pixel's fragments as it writes them (register path,
-// K <= 16): same arithmetic as blend_fwd.
+// Silhouette blend (Algorithm 1) applied by the fine pass to each pixel's
+// fragments as it writes them (register path, K <= 16): same arithmetic as
+// blend_fwd.  `rgb` asks for Algorithm 2, which the fine pass leaves alone.
 struct FineBlend {
     int on, rgb;
     int frag;   // 0: blend only, no Fragment data written (silhouette, fine-pass blend)
-    float sigma, gamma, znear, zfar, eps, bg0, bg1, bg2;
-    const int64_t *faces;
-    const float *colors;
-    int64_t F, V;
+    float sigma;
     float *image;
     // packed silhouette slots (instead of Fragment data; sil.cuh) and the
     // product of 1 - prob per pixel; NULL elsewhere
