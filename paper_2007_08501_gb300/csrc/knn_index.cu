@@ -25,7 +25,8 @@
 // scan of knn.cu 1,810 and 3,729.
 //
 //   k_nn_bounds   bounds of every cloud; one more block per batch checks its
-//                 ranges and plans the tiles of such a scan
+//                 ranges and plans the tiles of such a scan, one per cloud
+//                 bounds its grid by a sample
 //   k_nn_count    cell of every point and its rank there (warp-aggregated)
 //   k_nn_tiles    sums of kNnTile cells (clouds of more cells than that)
 //   k_nn_starts   exclusive scan of a cloud's cells
@@ -102,6 +103,33 @@ __device__ __forceinline__ void load_point(const float *x, long long row, float 
 // ---------------------------------------------------------------------------
 // building
 // ---------------------------------------------------------------------------
+// Ends of a cloud's grid, from 32 of its points: per axis, all but the outermost
+// two, and as much again on either side.  That takes in the whole of most clouds;
+// what lies farther out goes to the border cells.  A grid over everything lets one
+// far point put all others into one cell, in no order, and their boxes part
+// nothing: 8 clouds of 30,000 + 30,000 points with one outlier each, K = 1: 3,680 ->
+// 215 us (K = 8: 3,202 -> 422; the scan takes 1,857 and 3,738).  One warp's work.
+template <int D>
+__device__ __forceinline__ void sample_span(const NnSide &s, int cloud) {
+    const int t = threadIdx.x;
+    const long long n = s.len[cloud];
+    if (t >= 32 || n <= 0) return;   // (an empty cloud has no cells to fill)
+    float v[D];
+    load_point<D>(s.x, s.first[cloud] + t * n / 32, v);
+    float *o = s.span + 8 * (size_t)cloud;
+#pragma unroll
+    for (int c = 0; c < D; ++c) {
+        int rank = 0;
+#pragma unroll
+        for (int j = 0; j < 32; ++j) {
+            const float u = __shfl_sync(kAll, v[c], j);
+            rank += u < v[c] || (u == v[c] && j < t);
+        }
+        if (rank == 1) o[c] = v[c];
+        if (rank == 30) o[4 + c] = v[c];
+    }
+}
+
 // box[cloud]: enc(high) in 0..3, enc(-low) in 4..7, both by atomicMax from 0.
 // A block takes 4,096 rows, so that few atomics meet at a cloud's words.  (It
 // runs beside the check of the ranges; unfit ones have it read rows of their own
@@ -109,7 +137,11 @@ __device__ __forceinline__ void load_point(const float *x, long long row, float 
 template <int D>
 __global__ void __launch_bounds__(256) k_nn_bounds(NnSide a, NnSide b) {
     const NnSide &s = blockIdx.y ? b : a;
-    if (blockIdx.x == gridDim.x - 1) {
+    if ((int)blockIdx.x < s.N) {
+        sample_span<D>(s, (int)blockIdx.x);
+        return;
+    }
+    if ((int)blockIdx.x == s.N) {
         for (int i = threadIdx.x; i < s.N; i += 256) {
             const long long f = s.first[i], n = s.len[i], next = i + 1 < s.N ? s.first[i + 1] : s.P;
             if (f < 0 || n < 0 || n > s.P || f > next - n) s.control->unfit = 1;
@@ -120,7 +152,7 @@ __global__ void __launch_bounds__(256) k_nn_bounds(NnSide a, NnSide b) {
     __shared__ unsigned s_m[2 * D];
     int cloud, n;
     long long row0;
-    if (!tile_of(s, blockIdx.x, 12, cloud, row0, n)) return;   // uniform for the block
+    if (!tile_of(s, (long long)blockIdx.x - s.N - 1, 12, cloud, row0, n)) return;   // uniform for the block
     if (threadIdx.x < 2 * D) s_m[threadIdx.x] = 0u;
     __syncthreads();
     float hi[D], lo[D];
@@ -181,23 +213,49 @@ __device__ __forceinline__ unsigned curve_of(unsigned (&g)[D], int bits) {
     return code;
 }
 
-// Cell of v in a cloud's grid, numbered along the curve: cubic cells, 2^bits
-// along the longest side.  Any point maps to some cell (outside ones to the
-// border).
+// A cloud's grid: cubic cells, 2^bits along the longest side of its bounds within
+// the span.
 template <int D>
-__device__ __forceinline__ int cell_of(const NnSide &s, int cloud, const float (&v)[D]) {
+struct Grid {
+    float lo[D], scale;
+};
+
+template <int D>
+__device__ __forceinline__ Grid<D> grid_of(const NnSide &s, int cloud) {
     const unsigned *bx = s.box + 8 * (size_t)cloud;
-    float lo[D], ext = 0.f;
+    const float *span = s.span + 8 * (size_t)cloud;
+    Grid<D> g;
+    float ext = 0.f;
 #pragma unroll
     for (int c = 0; c < D; ++c) {
-        lo[c] = -dec(__ldg(bx + 4 + c));
-        ext = fmaxf(ext, dec(__ldg(bx + c)) - lo[c]);
+        const float a = __ldg(span + c), b = __ldg(span + 4 + c), w = b > a ? b - a : INFINITY;
+        g.lo[c] = fmaxf(-dec(__ldg(bx + 4 + c)), a - w);
+        ext = fmaxf(ext, fminf(dec(__ldg(bx + c)), b + w) - g.lo[c]);
     }
+    g.scale = (ext > 0.f && ext < 1e37f) ? (float)(1 << s.bits) / ext : 0.f;
+    return g;
+}
+
+// the same once k_nn_count has left it behind
+template <int D>
+__device__ __forceinline__ Grid<D> kept_grid(const NnSide &s, int cloud) {
+    const float4 a = __ldg(s.grid + 2 * (size_t)cloud);
+    const float v[4] = {a.x, a.y, a.z, a.w};
+    Grid<D> g;
+#pragma unroll
+    for (int c = 0; c < D; ++c) g.lo[c] = v[c];
+    g.scale = __ldg(&s.grid[2 * (size_t)cloud + 1].x);
+    return g;
+}
+
+// Cell of v, numbered along the curve.  Any point maps to some cell (outside
+// ones to the border).
+template <int D>
+__device__ __forceinline__ int cell_of(const NnSide &s, const Grid<D> &grid, const float (&v)[D]) {
     const float top = (float)((1 << s.bits) - 1);
-    const float scale = (ext > 0.f && ext < 1e37f) ? (top + 1.f) / ext : 0.f;
     unsigned g[D];
 #pragma unroll
-    for (int c = 0; c < D; ++c) g[c] = (unsigned)fminf(fmaxf((v[c] - lo[c]) * scale, 0.f), top);
+    for (int c = 0; c < D; ++c) g[c] = (unsigned)fminf(fmaxf((v[c] - grid.lo[c]) * grid.scale, 0.f), top);
     return (int)curve_of<D>(g, s.bits);
 }
 
@@ -208,11 +266,19 @@ __global__ void __launch_bounds__(256) k_nn_count(NnSide a, NnSide b) {
     long long row0;
     if (!tile_of(s, blockIdx.x, 8, cloud, row0, n)) return;
     const long long r = row0 + threadIdx.x;
+    const Grid<D> grid = grid_of<D>(s, cloud);
     int cell = -1;
     if (r < n) {
         float v[D];
         load_point<D>(s.x, s.first[cloud] + r, v);
-        cell = cell_of<D>(s, cloud, v);
+        cell = cell_of<D>(s, grid, v);
+    }
+    if (r == 0) {   // (a cloud without points has no search)
+        float lo[4] = {0.f, 0.f, 0.f, 0.f};
+#pragma unroll
+        for (int c = 0; c < D; ++c) lo[c] = grid.lo[c];
+        s.grid[2 * (size_t)cloud] = make_float4(lo[0], lo[1], lo[2], lo[3]);
+        s.grid[2 * (size_t)cloud + 1].x = grid.scale;
     }
     // lanes of one cell (clustered points, duplicates) share an atomic
     const unsigned peers = __match_any_sync(kAll, cell);
@@ -570,7 +636,7 @@ __global__ void __launch_bounds__(kLaneThreads, KM <= 8 ? 8 : 4) k_nn_lanes(NnQu
         float m[D];
 #pragma unroll
         for (int c = 0; c < D; ++c) m[c] = __shfl_sync(kAll, q[c], 16);
-        const int s = __ldg(a.c.start + (size_t)cloud * a.c.cells + cell_of<D>(a.c, cloud, m));
+        const int s = __ldg(a.c.start + (size_t)cloud * a.c.cells + cell_of<D>(a.c, kept_grid<D>(a.c, cloud), m));
         seed = min(s / kLeaf, nleaf - 1);
         visit(seed);
     }
@@ -642,7 +708,7 @@ __global__ void __launch_bounds__(kLaneThreads, KM <= 8 ? 8 : 4) k_nn_lanes(NnQu
 // take a leaf's candidates, and an admitted one is inserted by the whole warp
 // (a ballot ranks it, the later entries move one lane up).
 template <int D>
-__global__ void __launch_bounds__(kLaneThreads) k_nn_warps(NnQuery a) {
+__global__ void __launch_bounds__(kLaneThreads, 16) k_nn_warps(NnQuery a) {
     int cloud, n;
     long long row0;
     bool scan;
@@ -712,7 +778,7 @@ __global__ void __launch_bounds__(kLaneThreads) k_nn_warps(NnQuery a) {
     if (!scan) {
         int seed = -1;
         if (cn > 0) {
-            seed = min(__ldg(a.c.start + (size_t)cloud * a.c.cells + cell_of<D>(a.c, cloud, q)) / kLeaf, nleaf - 1);
+            seed = min(__ldg(a.c.start + (size_t)cloud * a.c.cells + cell_of<D>(a.c, kept_grid<D>(a.c, cloud), q)) / kLeaf, nleaf - 1);
             visit(seed);
         }
         unsigned bits;
@@ -797,6 +863,10 @@ void layout_side(NnSide &s, int64_t N, int64_t P, int D, char *ws, size_t &zero,
     zero = up256(zero + (size_t)N * 8 * sizeof(unsigned));
     s.start = reinterpret_cast<int *>(ws + zero);
     zero = up256(zero + (size_t)N * s.cells * sizeof(int));
+    s.span = reinterpret_cast<float *>(ws + off);
+    off = up256(off + (size_t)N * 8 * sizeof(float));
+    s.grid = reinterpret_cast<float4 *>(ws + off);
+    off = up256(off + (size_t)N * 2 * sizeof(float4));
     s.tile_sum = reinterpret_cast<int *>(ws + off);
     off = up256(off + (size_t)N * s.tiles * sizeof(int));
     s.cell_rank = reinterpret_cast<int2 *>(ws + off);
@@ -833,7 +903,7 @@ cudaError_t build_t(NnSide (&s)[2], int64_t N, bool boxes1, size_t zero, char *w
     const int64_t P = std::max(s[0].P, s[1].P);
     const unsigned g12 = (unsigned)((P >> 12) + N), g10 = (unsigned)((P >> 10) + N), g8 = (unsigned)((P >> 8) + N);
     const unsigned gt = (unsigned)(N * std::max(s[0].tiles, s[1].tiles));
-    k_nn_bounds<D><<<dim3(g12 + 1, 2), 256, 0, st>>>(s[0], s[1]);
+    k_nn_bounds<D><<<dim3(g12 + 1 + (unsigned)N, 2), 256, 0, st>>>(s[0], s[1]);
     k_nn_count<D><<<dim3(g8, 2), 256, 0, st>>>(s[0], s[1]);
     if (s[0].tiles > 1 || s[1].tiles > 1) k_nn_tiles<<<dim3(gt, 2), 1024, 0, st>>>(s[0], s[1]);
     k_nn_starts<<<dim3(gt, 2), 1024, 0, st>>>(s[0], s[1]);

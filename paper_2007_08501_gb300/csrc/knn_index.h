@@ -27,6 +27,8 @@ struct NnSide {
     int per;                    // queries of such a tile
     int N, bits, cells, tiles;  // cells = 2^(bits D) per cloud, tiles of kNnTile cells
     unsigned *box;              // N x 8: running bounds, order-preserving bits
+    float *span;                // N x 8: what k_nn_bounds sampled
+    float4 *grid;               // N x 2: low corner; cells per unit
     int *start;                 // N x cells: counts, then the first sorted position of each cell
     int *tile_sum;              // N x tiles
     int2 *cell_rank;            // P: cell of the point, its rank there
