@@ -57,6 +57,12 @@ MESHRAST_API size_t knn_workspace_bytes(int64_t N);
 MESHRAST_API size_t knn_index_workspace_bytes(int64_t N, int64_t P1, int64_t P2, int32_t D,
                                               int32_t K);
 
+/* How knn_points (chamfer_fwd, p to q: K = 1) answers for these sizes, given the
+ * workspace above: by scanning every candidate, or through the index with a
+ * query per lane or per warp.  MESHRAST_ERR_INVALID_ARG for invalid sizes. */
+enum { KNN_SCAN = 0, KNN_INDEX_LANES = 1, KNN_INDEX_WARPS = 2 };
+MESHRAST_API int knn_search_form(int64_t N, int64_t P1, int64_t P2, int32_t D, int32_t K);
+
 /* K nearest neighbours (Section 3.1, "K Nearest Neighbors").
  * idx (P1, K) int64: the global row in p2 of the k-th nearest candidate of
  * each query row, -1 where the candidate cloud has fewer than k + 1 points;

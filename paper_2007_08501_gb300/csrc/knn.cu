@@ -773,6 +773,12 @@ MESHRAST_API size_t knn_index_workspace_bytes(int64_t N, int64_t P1, int64_t P2,
     return ws_bytes(N) + (nn_index_wins(N, P1, P2, K) ? nn_index_bytes(N, P1, P2, D) : 0);
 }
 
+MESHRAST_API int knn_search_form(int64_t N, int64_t P1, int64_t P2, int32_t D, int32_t K) {
+    if (N < 0 || P1 < 0 || P2 < 0 || D < 1 || D > 4 || K < 1 || K > 32) return MESHRAST_ERR_INVALID_ARG;
+    if (!nn_index_wins(N, P1, P2, K)) return KNN_SCAN;
+    return nn_search_per_warp(P1, P2, K) ? KNN_INDEX_WARPS : KNN_INDEX_LANES;
+}
+
 MESHRAST_API int knn_points(const float *p1, int64_t P1, const int64_t *first1, const int64_t *len1,
                             const float *p2, int64_t P2, const int64_t *first2, const int64_t *len2, int64_t N,
                             int32_t D, int32_t K, int64_t *idx, float *dists, void *workspace,

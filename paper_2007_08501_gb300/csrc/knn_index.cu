@@ -955,7 +955,7 @@ bool nn_index_wins(int64_t N, int64_t P1, int64_t P2, int K) {
 // K = 8 a lane's insertions are long (K = 20: 32 of 50,000 4,737, 6,596),
 // unless 32 queries share the very same few candidates (32 of 50,000 + 1,000:
 // 3,617, 1,831).
-bool per_warp(int64_t P1, int64_t P2, int K) {
+bool nn_search_per_warp(int64_t P1, int64_t P2, int K) {
     if (P1 <= P2 / 8) return true;
     if (K > 8) return P1 < 8 * P2 || P1 < 200000;
     return P1 < (K <= 4 ? 100000 : 60000);
@@ -973,9 +973,9 @@ cudaError_t nn_index_build(NnSide (&s)[2], const float *p1, int64_t P1, const in
     size_t zero;
     layout(s, N, P1, P2, D, ws, zero);
     s[0].plan = plans;
-    s[0].per = 1 << (per_warp(P1, P2, K) ? kWarpShift : kLaneShift);
+    s[0].per = 1 << (nn_search_per_warp(P1, P2, K) ? kWarpShift : kLaneShift);
     s[1].plan = both_ways ? plans + N + 1 : nullptr;
-    s[1].per = 1 << (per_warp(P2, P1, K) ? kWarpShift : kLaneShift);
+    s[1].per = 1 << (nn_search_per_warp(P2, P1, K) ? kWarpShift : kLaneShift);
     s[0].x = p1;
     s[0].first = first1;
     s[0].len = len1;
@@ -993,7 +993,7 @@ cudaError_t nn_index_build(NnSide (&s)[2], const float *p1, int64_t P1, const in
 cudaError_t nn_index_search(const NnSide &q, const NnSide &c, int D, int K, int64_t *idx, float *dists,
                             cudaStream_t st) {
     const NnQuery a{q, c, idx, dists, K};
-    const bool warps = per_warp(q.P, c.P, K);
+    const bool warps = nn_search_per_warp(q.P, c.P, K);
     switch (D) {
         case 1: return search_t<1>(a, warps, st);
         case 2: return search_t<2>(a, warps, st);

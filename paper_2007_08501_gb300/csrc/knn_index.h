@@ -46,6 +46,8 @@ struct NnQuery {
 
 // Whether searching through the index beats scanning every candidate.
 bool nn_index_wins(int64_t N, int64_t P1, int64_t P2, int K);
+// Whether its search gives every query a warp instead of a lane.
+bool nn_search_per_warp(int64_t P1, int64_t P2, int K);
 size_t nn_index_bytes(int64_t N, int64_t P1, int64_t P2, int D);
 // Sides laid out in `ws` (nn_index_bytes), built on `st`: sides[0] the first batch, sides[1] the second.  The
 // first is searched for K neighbours; with `both_ways` the second is, too.  `plans`: 2 (N + 1) words.

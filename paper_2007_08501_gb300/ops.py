@@ -38,10 +38,12 @@ EXPORTED = ("rast_workspace_bytes", "rast_mesh_fwd", "rast_mesh_bwd", "blend_fwd
             "pts_workspace_bytes", "pts_rasterize_fwd", "pts_rasterize_bwd", "pts_composite_fwd",
             "pts_composite_bwd", "pts_bin_occupancy", "pts_staged_bytes", "pts_render_fwd", "pts_render_bwd",
              "shade_fwd", "shade_bwd",
-            "knn_workspace_bytes", "knn_index_workspace_bytes", "knn_points", "knn_points_bwd", "chamfer_fwd", "chamfer_bwd")
+            "knn_workspace_bytes", "knn_index_workspace_bytes", "knn_search_form",
+            "knn_points", "knn_points_bwd", "chamfer_fwd", "chamfer_bwd")
 
 SHADE_FLAT, SHADE_GOURAUD, SHADE_PHONG = 0, 1, 2
 SHADE_SOFTMAX, SHADE_HARD = 0, 1
+KNN_SCAN, KNN_INDEX_LANES, KNN_INDEX_WARPS = 0, 1, 2
 
 PTS_ALPHA = 0
 PTS_NORM = 1
@@ -173,6 +175,8 @@ def load(build_if_missing: bool = False):
     L.knn_workspace_bytes.restype = sz
     L.knn_index_workspace_bytes.argtypes = [i64, i64, i64, i32, i32]
     L.knn_index_workspace_bytes.restype = sz
+    L.knn_search_form.argtypes = [i64, i64, i64, i32, i32]
+    L.knn_search_form.restype = ctypes.c_int
     L.knn_points.argtypes = [vp, i64, vp, vp, vp, i64, vp, vp, i64, i32, i32, vp, vp, vp, sz, vp]
     L.knn_points.restype = ctypes.c_int
     L.knn_points_bwd.argtypes = [vp, i64, vp, i64, i32, i32, vp, vp, vp, vp, vp]
@@ -696,6 +700,14 @@ def shade_bwd(bp, sp, N, S, K, pix_to_face, zbuf, bary, dists, faces, verts, nor
 # ---------------------------------------------------------------------------
 def knn_workspace_bytes(N):
     return int(load().knn_workspace_bytes(int(N)))
+
+
+def knn_search_form(N, P1, P2, D, K):
+    """KNN_SCAN, KNN_INDEX_LANES or KNN_INDEX_WARPS: how knn_points (Chamfer: K = 1) answers for these sizes."""
+    rc = load().knn_search_form(int(N), int(P1), int(P2), int(D), int(K))
+    if rc < 0:
+        _check(rc, "knn_search_form")
+    return rc
 
 
 def alloc_knn_workspace(N, device="cuda", P1=0, P2=0, D=3, K=1):
