@@ -734,7 +734,7 @@ bool ws_ok(void *ws, size_t bytes, int64_t N) {
 
 // The index is used when the sizes favour it and the workspace has room for it.
 bool use_index(int64_t N, int64_t P1, int64_t P2, int D, int K, size_t bytes) {
-    return nn_index_wins(N, P1, P2, K) && bytes >= ws_bytes(N) + nn_index_bytes(N, P1, P2, D);
+    return nn_index_wins(N, P1, P2, D, K) && bytes >= ws_bytes(N) + nn_index_bytes(N, P1, P2, D);
 }
 
 // fill one problem; returns its number of blocks (an upper bound of its tiles)
@@ -770,12 +770,12 @@ MESHRAST_API size_t knn_workspace_bytes(int64_t N) { return N < 0 ? 0 : ws_bytes
 
 MESHRAST_API size_t knn_index_workspace_bytes(int64_t N, int64_t P1, int64_t P2, int32_t D, int32_t K) {
     if (N < 0 || P1 < 0 || P2 < 0 || D < 1 || D > 4 || K < 1 || K > 32) return 0;
-    return ws_bytes(N) + (nn_index_wins(N, P1, P2, K) ? nn_index_bytes(N, P1, P2, D) : 0);
+    return ws_bytes(N) + (nn_index_wins(N, P1, P2, D, K) ? nn_index_bytes(N, P1, P2, D) : 0);
 }
 
 MESHRAST_API int knn_search_form(int64_t N, int64_t P1, int64_t P2, int32_t D, int32_t K) {
     if (N < 0 || P1 < 0 || P2 < 0 || D < 1 || D > 4 || K < 1 || K > 32) return MESHRAST_ERR_INVALID_ARG;
-    if (!nn_index_wins(N, P1, P2, K)) return KNN_SCAN;
+    if (!nn_index_wins(N, P1, P2, D, K)) return KNN_SCAN;
     return nn_search_per_warp(P1, P2, K) ? KNN_INDEX_WARPS : KNN_INDEX_LANES;
 }
 

@@ -932,18 +932,23 @@ cudaError_t search_t(const NnQuery &a, bool warps, cudaStream_t st) {
 }  // namespace
 
 // Building takes about 40 us plus the points' share, so short scans stay.
-// Measured (D = 3, sphere surfaces; index, scan in us):
-//   K >= 5: the scan serves admissions one by one; 32 clouds of 200 + 200
-//     points, K = 8: 52, 172; 1 of 1,000 + 1,000: 44, 497; 32 of 50,000 +
-//     50,000: 1,441, 23,640
+// Measured (D = 3 unless said; index, scan in us of one call):
+//   K >= 5: the scan serves admissions one by one; 1 cloud of 100 + 100 points,
+//     normally distributed, K = 5: 25, 87, and at D = 1, 2, 3, 4 and K = 5, 8, 16, 32 alike
+//     (20 to 33, 37 to 240); 32 clouds of 1,000 + 20, K = 16: 60, 72; 1 of 1,000 + 1,000, K =
+//     8: 27, 497; 32 of 50,000 + 50,000: 947, 23,640
 //   K <= 4: by the pairs and the length of a candidate cloud; K = 1, 32 of
-//     2,000 + 2,000: 79, 69; 32 of 4,000 + 4,000: 114, 173; 1 of 10,000 +
-//     10,000: 48, 70; 1 of 1,000 + 50,000: 48, 155
-bool nn_index_wins(int64_t N, int64_t P1, int64_t P2, int K) {
+//     2,500 + 2,500: 87, 90, but D = 1 74, 67 and D = 2 82, 75, whose distances cost the
+//     scan less; 32 of 4,000 + 4,000: 101, 168; 1 of 5,000 + 8,192: 31, 43; 1 of 1,000 +
+//     32,000: 33, 101
+// The order of two or three distinct points repeated thousands of times parts
+// nothing, and the scan, which meets equal distances in the order of their rows,
+// stays up to 6 times as fast there (D = 1, coordinates of -1 and 1 only).
+bool nn_index_wins(int64_t N, int64_t P1, int64_t P2, int D, int K) {
     if (N <= 0 || P1 <= 0 || P2 <= 0 || N > (1 << 20) || P1 > (1LL << 30) || P2 > (1LL << 30)) return false;
     const double pairs = (double)P1 * (double)P2 / (double)N;
     if (K >= 5) return pairs >= 1e4;
-    return pairs >= 2e8 || (pairs >= 3e7 && P2 / N >= 8192);
+    return pairs >= (D <= 2 ? 3e8 : 2e8) || (pairs >= 3e7 && P2 / N >= 8192);
 }
 
 // Whether a search gives every query a warp instead of a lane.  A warp per

@@ -45,7 +45,7 @@ struct NnQuery {
 };
 
 // Whether searching through the index beats scanning every candidate.
-bool nn_index_wins(int64_t N, int64_t P1, int64_t P2, int K);
+bool nn_index_wins(int64_t N, int64_t P1, int64_t P2, int D, int K);
 // Whether its search gives every query a warp instead of a lane.
 bool nn_search_per_warp(int64_t P1, int64_t P2, int K);
 size_t nn_index_bytes(int64_t N, int64_t P1, int64_t P2, int D);
