@@ -86,7 +86,7 @@ MESHRAST_API int knn_points_bwd(const float *p1, int64_t P1, const float *p2, in
  * d_pq (P1,) and idx_qp (P2,) with d_qp (P2,) (as knn_points with K = 1),
  * the per-pair losses loss_per_pair (N,) and their mean loss (1,).  An empty
  * cloud contributes 0 to both terms of its pair; loss is 0 when N = 0.
- * Sums are taken in fp32 in a fixed order (deterministic). */
+ * Sums of the fp32 distances are taken in FP64 in a fixed order (deterministic). */
 MESHRAST_API int chamfer_fwd(const float *p, int64_t P1, const int64_t *first1, const int64_t *len1,
                              const float *q, int64_t P2, const int64_t *first2, const int64_t *len2,
                              int64_t N, int32_t D, int64_t *idx_pq, float *d_pq, int64_t *idx_qp,

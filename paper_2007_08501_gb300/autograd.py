@@ -6,10 +6,13 @@ recomputes barycentrics, depth and distance from ``pix_to_face`` instead of
 keeping them for the backward pass.  ``blend`` applies Algorithm 1
 (silhouette) or Algorithms 1 + 2 (softmax rgb + silhouette alpha) and
 differentiates through ``blend_bwd``.  ``render_meshes`` does both in one
-Function: its forward is ``rast_blend_fwd`` (the fine pass blends as it
-writes the fragments) and its backward ``blend_rast_bwd`` (the blend adjoint
-goes straight into the rasterizer adjoint without materialising fragment
-gradients).  ``knn_points`` and ``chamfer_distance`` (Section 3.1, Eq. 1)
+Function.  For the silhouette, where ``sil_packed`` takes the parameters, that
+is ``sil_fwd`` and ``sil_bwd``: packed slots and the staged face records go to
+the backward instead of Fragment data.  Otherwise (softmax blend, plain form)
+it is ``rast_blend_fwd`` and ``blend_rast_bwd``: the blend adjoint goes
+straight into the rasterizer adjoint without materialising fragment
+gradients.  ``render_points`` keeps packed slots likewise (``pts_render_fwd``,
+``pts_render_bwd``; the plain form the Fragment calls).  ``knn_points`` and ``chamfer_distance`` (Section 3.1, Eq. 1)
 wrap the exact nearest-neighbour search on packed point-cloud batches.
 """
 from __future__ import annotations
@@ -313,7 +316,7 @@ def render_points(points, features, first_point, num_points, cams, settings: Poi
     if settings.bin_size > 0 and features.dim() == 2 and features.shape[0] == points.shape[0]:
         fn = _RenderPointsPacked
     return fn.apply(points.contiguous(), features.contiguous(), first_point.contiguous(),
-                               num_points.contiguous(), cams.contiguous(), settings, ws)
+                    num_points.contiguous(), cams.contiguous(), settings, ws)
 
 
 # ---------------------------------------------------------------------------

@@ -256,9 +256,9 @@ __device__ __forceinline__ void bitonic_shared(unsigned long long *s_sort, int n
 // Sorts m <= sort-buffer bin entries (64-bit keys) from src into s_sort,
 // ascending; every thread of the block (BD threads) must call it.  A segment
 // that fits one entry per thread sorts in registers: partners closer than 32
-// trade through shuffles, farther ones through shared memory.  Larger ones
-// run a bitonic sort in shared memory.  Padding entries (all ones) sort last.
-template <int BD, bool REGS = false>
+// trade through shuffles, farther ones through shared memory.  Up to eight per
+// thread sort likewise, larger ones in shared memory.  Padding entries (all ones) sort last.
+template <int BD>
 __device__ __forceinline__ void sort_entries(unsigned long long *s_sort, const unsigned long long *src, int m) {
     const int tid = threadIdx.x;
     int n2 = 32;
@@ -288,13 +288,10 @@ __device__ __forceinline__ void sort_entries(unsigned long long *s_sort, const u
         __syncthreads();
         return;
     }
-    // REGS: two to eight entries per thread in registers and shuffles (more
-    // registers, far fewer barriers)
-    if constexpr (REGS) {
-        if (n2 == 2 * BD) { sort_entries_regs<BD, 2>(s_sort, src, m); return; }
-        if (n2 == 4 * BD) { sort_entries_regs<BD, 4>(s_sort, src, m); return; }
-        if (n2 == 8 * BD) { sort_entries_regs<BD, 8>(s_sort, src, m); return; }
-    }
+    // two to eight entries per thread in registers and shuffles (far fewer barriers)
+    if (n2 == 2 * BD) { sort_entries_regs<BD, 2>(s_sort, src, m); return; }
+    if (n2 == 4 * BD) { sort_entries_regs<BD, 4>(s_sort, src, m); return; }
+    if (n2 == 8 * BD) { sort_entries_regs<BD, 8>(s_sort, src, m); return; }
     for (int i = tid; i < n2; i += BD) s_sort[i] = i < m ? src[i] : ~0ull;
     __syncthreads();
     bitonic_shared<BD>(s_sort, n2);

@@ -63,7 +63,7 @@ __global__ void __launch_bounds__(256) k_sort_bins(FineArgs a) {
         const int cnt = a.eff[bin];  // <= sort_cap (checked on the host); uniform over the block
         if (cnt <= 1) continue;
         unsigned long long *list = a.lists + a.offsets[bin];
-        sort_entries<256, true>(s_sort, list, cnt);
+        sort_entries<256>(s_sort, list, cnt);
         for (int i = threadIdx.x; i < cnt; i += 256) list[i] = s_sort[i];
         __syncthreads();
     }
