@@ -24,7 +24,9 @@ bool ws_layout(const rast_params *p, int64_t V, int64_t F, mr::WsLayout *L) {
     L->total = 8;
     L->maxcount = 16;
     L->redo = 20;
-    off = 256;
+    L->longs = 24;
+    L->long_bins = 512;
+    off = 512 + (mr::kMaxLong + 1) * sizeof(mr::LongBin);
     L->records = off;
     off = align256(off + (size_t)F * sizeof(mr::FaceRec));
     L->face_mesh = off;
@@ -244,6 +246,10 @@ static int forward(const rast_params *p, const float *verts, int64_t V, const in
     sa.status = reinterpret_cast<unsigned *>(ws + L.status);
     sa.total = reinterpret_cast<long long *>(ws + L.total);
     sa.maxcount = reinterpret_cast<int *>(ws + L.maxcount);
+    // (an order pays with depth culling, or where the pixels' lists are inserted into from their ends)
+    const bool by_depth = p->max_faces_per_bin > mr::kLongList && !streaming && (fl.clip || !(fl.blur > 0.f) || K > 16);
+    sa.longs = by_depth ? reinterpret_cast<unsigned *>(ws + L.longs) : nullptr;
+    sa.long_bins = reinterpret_cast<mr::LongBin *>(ws + L.long_bins);
     sa.first_face = first_face;
     sa.num_faces = num_faces;
     sa.N = p->N;
@@ -308,10 +314,10 @@ static int forward(const rast_params *p, const float *verts, int64_t V, const in
         ka.blend.frag = no_frag ? 0 : 1;
         if (blended) *blended = true;
     }
-    // (an order pays with depth culling, or where the pixels' lists are inserted into from their ends)
-    if (p->max_faces_per_bin > mr::kLongList && (fl.clip || !(fl.blur > 0.f) || K > 16)) {
+    if (sa.longs) {
         ka.total = sa.total;
-        if (mr::launch_sort_long({ka.lists, ka.eff, ka.offsets, sa.maxcount, sa.total, L.NB}, st) != cudaSuccess)
+        ka.maxcount = sa.maxcount;
+        if (mr::launch_sort_long({ka.lists, ka.eff, ka.offsets, sa.longs, sa.long_bins}, st) != cudaSuccess)
             return MESHRAST_ERR_CUDA;
     }
     return mr::launch_fine(ka, p->bin_size, st) == cudaSuccess ? MESHRAST_OK : MESHRAST_ERR_CUDA;

@@ -318,15 +318,17 @@ __device__ __forceinline__ void sort_entries(unsigned long long *s_sort, const u
 // knowing any window's smallest key, that everything from there on is behind.
 // ---------------------------------------------------------------------------
 //
-// Every window reads the whole list for its entries.  Where few lists are long
-// (beyond 16,384 entries and a 64th of all bins' entries), those are sorted in place
-// before the fine pass (sort_long.cu) and handed out as they lie: 1.6M points on 16
-// px, K = 1, bins of 8: dealt 307 ms, sorted 7.2; 200,000 on 64 px, bins of 16: 1,696
-// us, 573; 1.3M faces on 16 px, K = 8, soft, bins of 8: 378 ms, 40.0; on 64 px, hard,
-// bins of 16: 29.9, 14.7.  Where many are, they fill the GPU as they are and most stop
-// after a few windows: 1.3M faces on 1,024 px (1,600 lists of 8,000 to 20,000), K = 8:
-// 972 us dealt, 1,764 with all of them sorted.  In between it is a draw: 328k faces on
-// 64 px, bins of 16, K = 1: dealt 1,760, sorted 1,869; on 128 px, K = 8, soft: 931, 1,076.
+// Every window reads the whole list for its entries.  Where few lists are long, they
+// are sorted in place before the fine pass (sort_long.cu) and handed out as they lie:
+// 1.6M points on 16 px, K = 1, bins of 8: dealt 307 ms, sorted 7.2; 200,000 on 64 px, bins
+// of 16: 1,696 us, 406; 1.3M faces on 16 px, K = 8, soft, bins of 8: 378 ms, 40.0; on 64 px,
+// hard, bins of 16: 29.9, 14.7.  Where many are, they fill the GPU as they are and most
+// stop after a few windows: 1.3M faces on 1,024 px (1,600 lists of 8,000 to 20,000), K = 8:
+// 972 us dealt, 1,764 with all of them sorted.  The line: some list has more than 16,384
+// entries and a 64th of all bins' entries; then all of half that length are sorted, so
+// that the pass does not wait for those just below.  (With T / 48: 4 meshes of 328k faces
+// on 48 px, K = 8, bins of 8: 4,726 us against 3,688; with 24,576: 2 of them on 64 px, K = 1,
+// bins of 16: 2,140 against 1,928, dealt 1,818.)
 constexpr int kBuckets = 256;
 
 struct KeyMap {

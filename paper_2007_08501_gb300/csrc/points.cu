@@ -7,8 +7,8 @@
 //              counts in shared memory where there are many
 //   k_scan     (shared with the mesh rasterizer) clamp counts, prefix scan
 //   k_pfill    append depth-keyed entries to the points' bins, as many to a thread
-//   k_sort_runs, k_merge_runs (sort_long.cu) where bins may hold more than
-//              kLongList entries: long lists
+//   k_sort_long (sort_long.cu) where bins may hold more than kLongList
+//              entries: long lists, where few are long
 //   k_pfine    persistent blocks over (image, bin) items: the bin's entries
 //              front to back in windows, each pixel's points appended in
 //              (depth, id) order; stops a bin once every pixel holds K
@@ -55,6 +55,7 @@ struct PtArgs {
     unsigned long long *lists;
     unsigned *queue, *status;
     const long long *total;  // entries of all bins, where long lists are sorted (else NULL)
+    const int *maxcount;     // and of the fullest
     int64_t *idx;
     float *zbuf, *dists;
     // rendering on packed slots (distance bits << 32 | id, ended by kPtEnd)
@@ -341,7 +342,7 @@ __global__ void __launch_bounds__(kPfineThreads) k_pfine(PtArgs a) {
     extern __shared__ int s_list[];        // [pixel][K] ids, rows an odd number of words apart
     const int tid = threadIdx.x, lane = tid & 31;
     const int nb2 = a.nb * a.nb, K = a.K, stride = K | 1;
-    const int sorted_from = a.total ? long_list(*a.total) : 0x7fffffff;
+    const int sorted_from = a.total ? long_list(*a.total, *a.maxcount) : 0x7fffffff;
     const unsigned magic_K = (unsigned)((0x100000000ull + (unsigned)K - 1) / (unsigned)K);
     const float w = a.radius * (1.f + kPtSlack);
     // a splat's half width in pixels, with slack for the rounding of its centre's column
@@ -1010,7 +1011,7 @@ static size_t al256(size_t x) { return (x + 255) & ~(size_t)255; }
 
 static void pt_layout(const pts_params *p, int64_t P, PtLayout *L) {
     std::memset(L, 0, sizeof(*L));
-    size_t off = 256;  // header: status @0, queue @4, total @8, max count @16 (as the mesh workspace)
+    size_t off = 1536;  // header: status @0, queue @4, total @8, max count @16, long lists @24, @512 (as the mesh workspace)
     L->records = off;
     off = al256(off + (size_t)P * sizeof(PtRec));
     L->cloud = off;
@@ -1209,6 +1210,8 @@ static int pts_forward(mr::PtArgs &out, const pts_params *p, const float *points
     sa.status = a.status;
     sa.total = reinterpret_cast<long long *>(ws + 8);
     sa.maxcount = reinterpret_cast<int *>(ws + 16);
+    sa.longs = p->max_points_per_bin > mr::kLongList ? reinterpret_cast<unsigned *>(ws + 24) : nullptr;
+    sa.long_bins = reinterpret_cast<mr::LongBin *>(ws + 512);
     sa.first_face = first_point;
     sa.num_faces = num_points;
     sa.N = p->N;
@@ -1217,9 +1220,10 @@ static int pts_forward(mr::PtArgs &out, const pts_params *p, const float *points
     if (P > 0) {
         if (mr::launch_pfill(a, st) != cudaSuccess) return MESHRAST_ERR_CUDA;
     }
-    if (p->max_points_per_bin > mr::kLongList) {
+    if (sa.longs) {
         a.total = sa.total;
-        if (mr::launch_sort_long({a.lists, a.eff, a.offsets, sa.maxcount, sa.total, a.items}, st) != cudaSuccess)
+        a.maxcount = sa.maxcount;
+        if (mr::launch_sort_long({a.lists, a.eff, a.offsets, sa.longs, sa.long_bins}, st) != cudaSuccess)
             return MESHRAST_ERR_CUDA;
     }
     return mr::launch_pfine(a, p->bin_size, st) == cudaSuccess ? MESHRAST_OK : MESHRAST_ERR_CUDA;

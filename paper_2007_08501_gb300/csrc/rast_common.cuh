@@ -18,13 +18,14 @@ namespace mr {
 constexpr float kCullArea = 1e-12f;
 constexpr int kMaxK = 64;
 
-// Entries beyond which a bin's list is sorted before the fine pass, with `total`
-// in all bins (bin_common.cuh says why).
+// Entries beyond which a bin's list is sorted before the fine pass, with `total` in
+// all bins and `most` in the fullest (bin_common.cuh says why).
 constexpr int kLongList = 16384;
-__host__ __device__ __forceinline__ int long_list(long long total) {
-    const long long share = total / 64;
-    return share < kLongList ? kLongList : share > 0x7fffffffLL ? 0x7fffffff : (int)share;
+__device__ __forceinline__ int long_list(long long total, int most) {
+    const long long share = total / 64 > kLongList ? total / 64 : kLongList;
+    return most <= share ? 0x7fffffff : (int)(share / 2);
 }
+constexpr int kMaxLong = 127;  // so many lists can be longer than half of a 64th of all entries
 
 // ---------------------------------------------------------------------------
 // Staged face record: 96 bytes, six float4, written once per face by the
@@ -510,6 +511,8 @@ struct WsLayout {
     size_t queue;       // uint32 work-queue head of the fine pass
     size_t total;       // int64 sum of raw bin counts
     size_t maxcount;    // int32 largest raw bin count
+    size_t longs;       // uint32 bins with long lists
+    size_t long_bins;   // kMaxLong x LongBin
     size_t redo;        // uint32 pixels of the large-K streaming pass whose unsettled candidates outgrew the ring
     size_t records;     // F x FaceRec
     size_t face_mesh;   // F x int32

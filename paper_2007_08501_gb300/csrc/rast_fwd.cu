@@ -6,10 +6,11 @@
 // Fragment data of those faces.  Launch sequence of one binned forward:
 //   k_stage     one thread per face: double-float projection, 96-byte face
 //               record, warp-aggregated bin counts
-//   k_scan      one block: clamp counts to capacity, exclusive scan -> offsets
+//   k_scan      one block: clamp counts to capacity, exclusive scan -> offsets;
+//               finds the long lists
 //   k_fill      one thread per face: warp-aggregated atomic append into lists
-//   k_sort_runs, k_merge_runs (sort_long.cu) where bins may hold more than
-//               kLongList entries: long lists
+//   k_sort_long (sort_long.cu) where bins may hold more than kLongList entries:
+//               long lists, where few are long
 //   k_fine      persistent blocks pull (image, bin) items from a global queue,
 //               walk each bin's faces front to back, keep a register-resident
 //               top-K per pixel, write the fragments
@@ -176,7 +177,7 @@ __global__ void __launch_bounds__(256) k_stage(StageArgs a) {
 }
 
 // ---------------------------------------------------------------------------
-// scan: one block; clamps counts, exclusive scan, resets cursors and queue
+// scan: one block; clamps counts, exclusive scan, resets cursors and queue, finds the long lists
 // ---------------------------------------------------------------------------
 // Bound by the latency of its rounds, so a thread takes four bins in each (16
 // bytes at a time): 32,768 bins 56 -> 27 us.
@@ -286,6 +287,15 @@ __global__ void __launch_bounds__(1024) k_scan(ScanArgs a) {
         a.offsets[a.NB] = (int)min(carry_s, (long long)a.capacity);
         *a.maxcount = maxc_s;
         *a.total = (long long)tot_s;
+        if (a.longs) *a.longs = 0u;
+    }
+    if (a.longs) {
+        const int from = long_list((long long)tot_s, maxc_s);
+        if (from < maxc_s) {
+            __syncthreads();
+            for (int64_t b = tid; b < a.NB; b += 1024)
+                if (a.eff[b] > from) a.long_bins[atomicAdd(a.longs, 1u)] = {(int)b, 0u};
+        }
     }
     if (!a.order) return;
     // Queue order of the fine pass: bins by descending work class (the bit
@@ -552,7 +562,7 @@ __global__ void __launch_bounds__(BS *BS, fine_blocks(KM, BS)) k_fine(FineArgs a
     EvalFlags fl = a.fl;
     const bool zcull = fl.clip || !(fl.blur > 0.f);
     const int nb2 = a.nb * a.nb;
-    const int sorted_from = a.total ? long_list(*a.total) : 0x7fffffff;
+    const int sorted_from = a.total ? long_list(*a.total, *a.maxcount) : 0x7fffffff;
     float4 (*const rec)[NREC] = s_rec[tid >> 5];
     while (true) {
         if (tid == 0) s_item = (int)atomicAdd(a.queue, 1u);

@@ -26,6 +26,11 @@ struct StageArgs {
     unsigned *status;
 };
 
+struct LongBin {
+    int bin;
+    unsigned runs;  // sorted so far (k_sort_long)
+};
+
 struct ScanArgs {
     const int *counts;
     int *eff, *offsets, *cursor;
@@ -35,6 +40,8 @@ struct ScanArgs {
     unsigned *queue, *status;
     long long *total;
     int *maxcount;
+    unsigned *longs;     // non-NULL: number of the long lists
+    LongBin *long_bins;  // and those lists (kMaxLong)
     const int64_t *first_face, *num_faces;
     int N;
     int64_t F;
@@ -79,6 +86,7 @@ struct FineArgs {
     unsigned *spilled;          // large-K streaming pass: pixels whose unsettled candidates outgrew the ring
     int items, nb, S, K;
     const long long *total;  // entries of all bins, where long lists are sorted (else NULL)
+    const int *maxcount;     // and of the fullest
     int sort_cap;  // streaming pass: bin entries sorted at a time (power of two)
     float inv_sigma;  // streaming pass with packed slots: 1 / sigma
     EvalFlags fl;
@@ -117,13 +125,12 @@ struct SilBwdArgs {
     float sigma;
 };
 
-// Lists beyond long_list entries sorted in place.
+// Long lists sorted in place.
 struct SortLongArgs {
     unsigned long long *lists;
     const int *eff, *offsets;
-    const int *maxcount;     // largest count of any bin
-    const long long *total;  // entries of all bins
-    int64_t items;
+    const unsigned *n;  // long lists, and
+    LongBin *long_bins; // which (k_scan)
 };
 
 struct NaiveArgs {

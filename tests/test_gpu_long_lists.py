@@ -22,7 +22,7 @@ def _depths(kind, n, rng):
 @pytest.mark.parametrize("kind,n,K,blur,clip", [
     ("mixed", 32_768, 1, 0.0, False), ("mixed", 32_769, 8, 1e-3, True), ("levels", 40_961, 5, 1e-3, True),
     ("flat", 50_000, 3, 0.0, False), ("mixed", 70_001, 8, 1e-3, True), ("mixed", 33_000, 24, 1e-3, True),
-    ("levels", 40_000, 50, 0.0, False), ("mixed", 40_000, 24, 1e-3, False), ("mixed", 40_000, 16, 1e-3, False)])
+    ("levels", 40_000, 50, 0.0, False), ("mixed", 40_000, 24, 1e-3, False), ("mixed", 40_000, 16, 1e-3, False), ("mixed", 17_000, 4, 1e-3, True)])
 def test_long_face_lists_match_the_plain_form(kind, n, K, blur, clip):
     rng = np.random.default_rng(n + K)
     z = _depths(kind, n, rng)[:, None] * np.ones(3)
