@@ -74,10 +74,12 @@ WORKLOADS = {
 #   K <= 16: k_fine (+ k_blend_fwd for the softmax blend);
 #   K > 16 with clipped barycentrics (or no blur): k_sort_bins, k_fine_stream,
 #   k_frag_attr (which blends the silhouette; + k_blend_fwd for softmax);
+#   bins of more than 16,384 entries: k_sort_long before k_fine, where depths
+#   order the candidates;
 # blend_rast_bwd = k_stage, k_blend_rast_bwd
 
 
-def mesh_kernels_per_step(w):
+def mesh_kernels_per_step(w, max_faces_per_bin=0):
     rgb = w.blend_mode == "rgb"
     if w.K <= 16:
         fwd = 4 + (1 if rgb else 0)
@@ -85,12 +87,27 @@ def mesh_kernels_per_step(w):
         fwd = 6 + (1 if rgb else 0)
     else:
         fwd = 5          # k_fine with shared-memory lists, then k_blend_fwd
+    if max_faces_per_bin > 16384 and (w.K > 16 or w.clip_barycentric_coords or not w.blur_radius > 0):
+        fwd += 1
     return fwd + 2
+
+
 # DRAM bytes (read + write) per C-ABI call of a stage -- every kernel of the
 # call, from one ncu capture (gpu__time_duration, dram__bytes_read/write,
-# --clock-control none) of the current kernel source -- keyed by (workload,
-# stage, bin size); a combination without an entry reports null.
-TRAFFIC_BYTES = {}
+# --clock-control none, caches flushed before each kernel) of the current kernel
+# source -- keyed by (workload, stage, bin size); a combination without an entry
+# reports null.
+_TRAFFIC = "profiles/dram_traffic_of_the_bench_calls.md"
+TRAFFIC_BYTES = {
+    ("1", "fwd", 16): {"kernel": "k_stage, k_scan, k_fill, k_fine, k_blend_fwd", "bytes": 142_300_000,
+                       "profile": _TRAFFIC},
+    ("1", "bwd", 16): {"kernel": "k_stage, k_blend_rast_bwd", "bytes": 106_000_000, "profile": _TRAFFIC},
+    ("4", "fwd", 16): {"kernel": "k_stage, k_scan, k_fill, k_sort_bins, k_fine_stream, k_frag_attr",
+                       "bytes": 11_629_000_000, "profile": _TRAFFIC + " (2 of the 20 views, times 10)"},
+    ("4", "bwd", 16): {"kernel": "k_stage, k_blend_rast_bwd_any", "bytes": 4_202_000_000,
+                       "profile": _TRAFFIC + " (2 of the 20 views, times 10)"},
+    ("points", "composite_bwd", 8): {"kernel": "k_pcomp_bwd", "bytes": 595_100_000, "profile": _TRAFFIC},
+}
 
 
 def _args():
@@ -576,7 +593,7 @@ def run_ours(args):
     alg = algorithmic_bytes(w)
     peak, peak_kind = _peaks()
     achieved = alg[dom] / (stages[dom] / 1e3) / 1e9
-    tr = TRAFFIC_BYTES.get((args.workload, dom, tuned["bin_size"]))
+    tr = None if args.max_images else TRAFFIC_BYTES.get((args.workload, dom, tuned["bin_size"]))
     roofline = {"bound": "hbm", "achieved": round(achieved, 1), "peak": peak, "unit": "GB/s",
                 "frac": round(achieved / peak, 4), "traffic": tr["bytes"] if tr else None,
                 "traffic_kernel": tr["kernel"] if tr else None,
@@ -757,7 +774,8 @@ def run_ours(args):
             "stages_ms": {k: round(v, 4) for k, v in stages.items()},
             "stages_hbm_frac": stage_frac,
             "cpu_baseline": cpu, "cpu_baseline_parallel": cpu_par, "e2e": e2e,
-            "gpu_launches": (8 if shading is not None else mesh_kernels_per_step(w)) * args.steps,
+            "gpu_launches": (8 if shading is not None else mesh_kernels_per_step(w, tuned["max_faces_per_bin"]))
+            * args.steps,
             "ms_per_step_median": round(statistics.median(step_ms), 4),
             "fine_pass": {"face_pixel_tests": fine_tests,
                           "tests_per_s": round(fine_tests / (stages.get("fwd", stages.get("rast_fwd")) / 1e3), 1),
