@@ -320,8 +320,8 @@ __device__ __forceinline__ void sort_entries(unsigned long long *s_sort, const u
 //
 // Every window reads the whole list for its entries.  Where few lists are long, they
 // are sorted in place before the fine pass (sort_long.cu) and handed out as they lie:
-// 1.6M points on 16 px, K = 1, bins of 8: dealt 307 ms, sorted 7.2; 200,000 on 64 px, bins
-// of 16: 1,696 us, 406; 1.3M faces on 16 px, K = 8, soft, bins of 8: 378 ms, 40.0; on 64 px,
+// 1.6M points on 16 px, K = 1, bins of 8: dealt 307 ms, sorted 7.0; 200,000 on 64 px, bins
+// of 16: 1,696 us, 386; 1.3M faces on 16 px, K = 8, soft, bins of 8: 378 ms, 40.0; on 64 px,
 // hard, bins of 16: 29.9, 14.7.  Where many are, they fill the GPU as they are and most
 // stop after a few windows: 1.3M faces on 1,024 px (1,600 lists of 8,000 to 20,000), K = 8:
 // 972 us dealt, 1,764 with all of them sorted.  The line: some list has more than 16,384
